@@ -337,7 +337,8 @@ int teno_profile_read(teno_ctx* ctx, double* ms, int64_t* launches);
  * efficiency note).  The mesh's cells are split into n_parts contiguous
  * ranges of the Hilbert order made of whole 32-cell tiles ("owned" cells).
  * A partition reconstructs its owned cells and the first layer of cells
- * across its boundary (the face neighbours of owned cells), so that it
+ * across its boundary (the face neighbours of owned cells; where the FP64
+ * paths take the W form, the whole tiles that hold them), so that it
  * evaluates every face flux its owned cells need by itself, and keeps the
  * states of every cell those stencils reach (its "halo").  Per RK stage one
  * halo exchange brings the stage state of the halo from the owners; the

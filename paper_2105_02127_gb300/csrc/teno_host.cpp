@@ -69,7 +69,7 @@ struct teno_ctx {
   std::vector<int32_t> st_large, st_small;  // user ids, [nc][ns], [nc][36]
   // device data
   DeviceMesh dm;
-  DevBuf b_halo_off, b_halo_ids, b_halo_loc, b_g32, b_wq, b_psi, b_cspeed, b_coef;
+  DevBuf b_halo_off, b_halo_ids, b_halo_loc, b_g32, b_wq, b_wstat, b_wtile, b_wpos, b_psi, b_cspeed, b_coef;
   DevBuf b_ahat, b_nbr, b_smask, b_fcells, b_fedges, b_fgeom, b_fgeom2, b_cfaces, b_inv_area, b_cfl_len, b_cfl_ilen2,
       b_perm;
   DevBuf b_fo;  // the outflow layer: local ids of the cells with an outflow face
@@ -471,6 +471,74 @@ int make_ref(int order, int nq, RefData& R) {
   return TENO_OK;
 }
 
+// The W form's split of the coefficients a (beta-orthonormal basis, so
+// beta = |a|^2): with Psi'^T = Q R (Householder, Q orthogonal m x m) the
+// values y = Psi' a give Q1^T a = R^-T y, and q2 holds the remaining m - P
+// rows Q2^T.  With more points than coefficients (P > m) Psi' = Q R gives
+// a = R^-1 Q1^T y.
+struct WBasis {
+  double q2[kMaxM * kMaxM];
+  WTable table;
+};
+
+void w_basis(const RefData& R, WBasis& B) {
+  const int m = R.m, P = 3 * R.nq, r = std::min(m, P), n = std::max(m, P);
+  // A (n x r) = Psi'^T or Psi'; reflections accumulate in Q^T (n x n)
+  std::vector<double> A((size_t)n * r), Qt((size_t)n * n, 0.0);
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < r; ++j)
+      A[i * r + j] = P <= m ? R.psi_t[j * kMaxM + i] : R.psi_t[i * kMaxM + j];
+  for (int i = 0; i < n; ++i) Qt[i * n + i] = 1.0;
+  for (int j = 0; j < r && j < n - 1; ++j) {
+    double s = 0.0;
+    for (int i = j; i < n; ++i) s += A[i * r + j] * A[i * r + j];
+    const double al = A[j * r + j] > 0.0 ? -std::sqrt(s) : std::sqrt(s);
+    std::vector<double> u(n, 0.0);
+    for (int i = j; i < n; ++i) u[i] = A[i * r + j];
+    u[j] -= al;
+    double uu = 0.0;
+    for (int i = j; i < n; ++i) uu += u[i] * u[i];
+    if (uu == 0.0) continue;
+    auto reflect = [&](double* M, int cols) {
+      for (int c = 0; c < cols; ++c) {
+        double d = 0.0;
+        for (int i = j; i < n; ++i) d += u[i] * M[i * cols + c];
+        d *= 2.0 / uu;
+        for (int i = j; i < n; ++i) M[i * cols + c] -= d * u[i];
+      }
+    };
+    reflect(A.data(), r);
+    reflect(Qt.data(), n);
+  }
+  // inverse of the upper triangle
+  std::vector<double> Ri((size_t)r * r, 0.0);
+  for (int c = 0; c < r; ++c)
+    for (int i = c; i >= 0; --i) {
+      double s = i == c ? 1.0 : 0.0;
+      for (int k = i + 1; k <= c; ++k) s -= A[i * r + k] * Ri[k * r + c];
+      Ri[i * r + c] = s / A[i * r + i];
+    }
+  memset(&B, 0, sizeof(B));
+  double all = 0.0;
+  for (int p = 0; p < P; ++p) {
+    double cs = 0.0;
+    for (int i = 0; i < r; ++i) {
+      double t = 0.0;
+      if (P <= m)
+        t = p <= i ? Ri[p * r + i] : 0.0;
+      else
+        for (int k = i; k < r; ++k) t += Ri[i * r + k] * Qt[k * n + p];
+      B.table.t[i * P + p] = (float)t;
+      cs += std::fabs(t);
+    }
+    B.table.cs[p] = (float)(cs * (1.0 + 1e-6));
+    all += cs;
+  }
+  B.table.cs_all = (float)(all * (1.0 + 1e-6));
+  for (int l = 0; l < wform_rows(m, P); ++l)
+    for (int i = 0; i < m; ++i) B.q2[l * kMaxM + i] = Qt[(P + l) * n + i];
+}
+
 // ========================================================================
 // stencils (user ids)
 
@@ -833,6 +901,10 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   if (make_ref(p.order, ctx->nq, R)) return fail(ctx, TENO_EINVAL, "reference data");
   const int m = R.m, ns = ctx->ns, SL = ctx->SL, E = ctx->E;
   const int64_t nc = ctx->nc, ntile_g = ctx->npad / kTile;
+  const int store = p.precision;
+  // Euler TENO on the FP64 paths with the bulk-copy kernel (the W form)
+  const bool wform = (store == TENO_FP64 || store == TENO_FP64_NATIVE) && p.n_var == 4 &&
+                     p.recon_variant == 2 && p.scheme == 0 && p.charvar == 0;
   // the global tiles whose cells are built: all of them, or those holding a
   // partition's compute set (every lane of such a tile, for its slot colouring)
   PartCells pc;
@@ -844,6 +916,15 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
     for (int32_t c : pc.layer1) tiles_g.push_back(c / kTile);
     std::sort(tiles_g.begin(), tiles_g.end());
     tiles_g.erase(std::unique(tiles_g.begin(), tiles_g.end()), tiles_g.end());
+    if (wform) {
+      // the W form's fixed-point unit is a tile's: the part reconstructs the
+      // whole tiles of its boundary layer, so that every cell's tile is the
+      // whole mesh's and so are its bits
+      pc.layer1.clear();
+      for (int64_t t : tiles_g)
+        for (int64_t c = t * kTile; c < std::min(nc, (t + 1) * kTile); ++c)
+          if (c < pc.c0 || c >= pc.c1) pc.layer1.push_back((int32_t)c);
+    }
   } else {
     tiles_g.resize(ntile_g);
     for (int64_t t = 0; t < ntile_g; ++t) tiles_g[t] = t;
@@ -853,20 +934,19 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   ctx->st_small.assign(nc * kSmallK * kSmallN, -1);
   // matrix storage: double (native FP64), (hi, lo) float pairs (FP64 via
   // double-float) or float (mixed)
-  const int store = p.precision;
   const size_t esz = store == TENO_FP32_MIXED ? sizeof(float) : 8;
   std::vector<unsigned char> ahat((size_t)ntile * E * kTile * esz, 0);
-  // Euler on the FP64 paths with the bulk-copy kernel (the W form): FP32
-  // selection matrices with column sums of |G| (large slots M + 1 floats,
-  // directional slots 5 + 1) and W = Psi' G, the large polynomial's
-  // Gauss-point values per unit difference, as (hi, lo) pairs on the pair
-  // path and as doubles (the same 8 bytes) on the native path
-  const bool wform = (store == TENO_FP64 || store == TENO_FP64_NATIVE) && p.n_var == 4 &&
-                     p.recon_variant == 2 && p.scheme == 0 && p.charvar == 0;
+  // the W form: W = Psi' G, the large polynomial's Gauss-point values per unit difference,
+  // in fixed point; the FP32 rows of the smoothness indicators that W does not
+  // give; and the bounds' norms (DeviceMesh::g32, wq, wstat)
   const int nq3 = 3 * ctx->nq;
-  const int E32 = ns * (m + 1) + kSmallK * kSmallN * (kSmallM + 1), EW = ns * nq3;
+  const int mc = wform_rows(m, nq3);
+  const int E32 = ns * mc + kSmallK * kSmallN * kSmallM, EW = ns * nq3;
+  WBasis wb;
+  if (wform) w_basis(R, wb);
   std::vector<float> g32(wform ? (size_t)ntile * E32 * kTile : 0, 0.f);
-  std::vector<float2> wq(wform ? (size_t)ntile * EW * kTile : 0, make_float2(0.f, 0.f));
+  std::vector<int2> wq(wform ? (size_t)ntile * EW * kTile : 0, make_int2(0, 0));
+  std::vector<int32_t> wstat(wform ? (size_t)ntile * kWStat * kTile : 0, 60);
   std::vector<int32_t> nbr((size_t)ntile * SL * kTile, 0);
   std::vector<uint8_t> smask((size_t)ntile * kTile, 0);
   int rc = TENO_OK;
@@ -874,7 +954,7 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
 #pragma omp parallel
   {
     Searcher S(ctx);
-    std::vector<double> G(kMaxM * kMaxNs);
+    std::vector<double> G(kMaxM * kMaxNs), W(kMaxNs * kMaxPts);
 #pragma omp for schedule(dynamic, 8)
     for (int64_t k = 0; k < ntile; ++k) {
       for (int64_t lane = 0; lane < kTile; ++lane) {
@@ -897,36 +977,71 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
             reinterpret_cast<float*>(ahat.data())[pos] = (float)x;
           }
         };
-        // FP32 rows plus an upper bound of their absolute column sum
-        auto put32 = [&](int e0, const double* col, int stride, int rows) {
+        // FP32 rows; adds the square of their absolute column sum to n2
+        float* gt = wform ? &g32[(size_t)tile * E32 * kTile] : nullptr;
+        int2* wt = wform ? &wq[(size_t)tile * EW * kTile] : nullptr;
+        auto put32 = [&](bool lg, int slot, const double* col, int stride, int rows, double& n2) {
           double cs = 0.0;
           for (int l = 0; l < rows; ++l) {
-            const float x = (float)col[l * stride];
-            g32[((size_t)tile * E32 + e0 + l) * kTile + lane] = x;
-            cs += std::fabs((double)x);
+            gt[lg ? wform_g_index(ns, mc, slot, l, (int)lane)
+                  : wform_s_index(ns, mc, slot, l, (int)lane)] = (float)col[l * stride];
+            cs += std::fabs(col[l * stride]);
           }
-          g32[((size_t)tile * E32 + e0 + rows) * kTile + lane] = (float)(cs * (1.0 + 1e-6));
+          n2 += cs * cs;
+        };
+        int32_t stat[kWStat] = {0, 0, 0, 0, 0};
+        auto put_norm = [&](int k, double n2) {
+          const float x = (float)(std::sqrt(n2) * (1.0 + 1e-6));
+          memcpy(&stat[k], &x, sizeof(float));
         };
         if (!r) r = stencil_matrix(ctx, R, t, lg, ns, m, G.data());
         if (!r) {
           for (int s = 0; s < ns; ++s) {
             nbr[((size_t)tile * SL + s) * kTile + lane] = ctx->iperm[lg[s]];
             for (int l = 0; l < m; ++l) put(s * m + l, G[l * ns + s]);
-            if (wform) {
-              put32(s * (m + 1), &G[s], ns, m);
+          }
+          if (wform) {
+            double n2 = 0.0, l1 = 0.0;
+            for (int s = 0; s < ns; ++s) {
+              double row[kMaxM];
+              for (int l = 0; l < mc; ++l) {
+                double x = 0.0;
+                for (int i = 0; i < m; ++i) x += wb.q2[l * kMaxM + i] * G[i * ns + s];
+                row[l] = x;
+              }
+              put32(true, s, row, 1, mc, n2);
+            }
+            put_norm(kSmallK, n2);
+            // W and the exponent of its unit: the largest row sum just below 2^31
+            // (pairs: integer and FP32 fraction) or 2^60 (FP64: two integers)
+            double rs[kMaxPts] = {0.0};
+            for (int s = 0; s < ns; ++s)
               for (int q = 0; q < nq3; ++q) {
                 double w = 0.0;
                 for (int l = 0; l < m; ++l) w += R.psi_t[q * kMaxM + l] * G[l * ns + s];
-                float2& dst = wq[((size_t)tile * EW + s * nq3 + q) * kTile + lane];
-                if (store == TENO_FP64_NATIVE) {
-                  static_assert(sizeof(float2) == sizeof(double), "8-byte W entries");
-                  memcpy(&dst, &w, sizeof(double));
+                W[s * nq3 + q] = w;
+                rs[q] += std::fabs(w);
+              }
+            for (int q = 0; q < nq3; ++q) l1 = std::max(l1, rs[q]);
+            int ex = 0;
+            if (l1 > 0.0) std::frexp(l1 * (1.0 + 1e-6), &ex);
+            const int kc = (store == TENO_FP64 ? 31 : 60) - ex;
+            stat[kWStat - 1] = kc & 0xffff;
+            for (int s = 0; s < ns; ++s)
+              for (int q = 0; q < nq3; ++q) {
+                const double z = std::ldexp(W[s * nq3 + q], kc);
+                int2& dst = wt[wform_w_index(ns, nq3, s, q, (int)lane)];
+                if (store == TENO_FP64) {
+                  const double h = std::nearbyint(z);
+                  const float l = (float)(z - h);
+                  dst.x = (int)h;
+                  memcpy(&dst.y, &l, sizeof(float));
                 } else {
-                  const float hi = (float)w;
-                  dst = make_float2(hi, (float)(w - (double)hi));
+                  const int64_t x = std::llrint(z);
+                  const int64_t h = (x + (1ll << 29)) >> 30;
+                  dst = make_int2((int)h, (int)(x - (int64_t)((uint64_t)h << 30)));
                 }
               }
-            }
           }
           uint8_t mask = 0;
           for (int j = 0; j < kSmallK && !r; ++j) {
@@ -943,15 +1058,22 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
             r = stencil_matrix(ctx, R, t, ids, kSmallN, kSmallM, G.data());
             if (r) break;
             mask |= (uint8_t)(1u << j);
+            double n2 = 0.0;
             for (int s = 0; s < kSmallN; ++s) {
               nbr[((size_t)tile * SL + slot0 + s) * kTile + lane] = ctx->iperm[ids[s]];
               for (int l = 0; l < kSmallM; ++l)
                 put(m * ns + (j * kSmallN + s) * kSmallM + l, G[l * kSmallN + s]);
               if (wform)
-                put32(ns * (m + 1) + (j * kSmallN + s) * (kSmallM + 1), &G[s], kSmallN, kSmallM);
+                put32(false, j * kSmallN + s, &G[s], kSmallN, kSmallM, n2);
             }
+            put_norm(j, n2);
           }
           smask[(size_t)tile * kTile + lane] = mask;
+          if (wform) {
+            stat[kWStat - 1] |= (int32_t)mask << 16;
+            for (int k = 0; k < kWStat; ++k)
+              wstat[((size_t)tile * kWStat + k) * kTile + lane] = stat[k];
+          }
         }
         if (r) {
 #pragma omp critical
@@ -965,11 +1087,12 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   }
   if (rc)
     return fail(ctx, rc, "stencil or least-squares failure at user cell " + std::to_string(bad));
-  // pad lanes of the last tile point at cell 0
+  // pad lanes of the last tile point at its first cell
   for (int64_t k = 0; k < ntile; ++k)
     for (int64_t lane = 0; lane < kTile; ++lane)
       if (tiles_g[k] * kTile + lane >= nc)
-        for (int s = 0; s < SL; ++s) nbr[((size_t)k * SL + s) * kTile + lane] = 0;
+        for (int s = 0; s < SL; ++s)
+          nbr[((size_t)k * SL + s) * kTile + lane] = (int32_t)(tiles_g[k] * kTile);
   // Slot order of the large stencils (for the adjoint's halo accumulation):
   // within each tile the members of the cells' large stencils are assigned
   // to the ns slots by a proper edge colouring of the bipartite graph (lane,
@@ -1001,16 +1124,22 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
         for (int ln = 0; ln < nval; ++ln) {
           for (int s = 0; s < ns; ++s) perm[s] = slot_of[(size_t)ln * ns + s];
           // entries s * per_slot + l of lane ln in a [tile][entry][lane] array
-          auto permute = [&](auto* base, size_t stride_e, size_t per_slot) {
+          // (at: position of (slot, l) of the lane in the tile's block)
+          auto permute_at = [&](auto* base, size_t stride_e, int per_slot, auto&& at) {
             using T = std::remove_pointer_t<decltype(base)>;
             T* tb = reinterpret_cast<T*>(tmp.data());
-            T* row = base + (size_t)t * stride_e * kTile + ln;
+            T* blk = base + (size_t)t * stride_e * kTile;
             for (int s = 0; s < ns; ++s)
-              for (size_t l = 0; l < per_slot; ++l)
-                tb[(size_t)perm[s] * per_slot + l] = row[((size_t)s * per_slot + l) * kTile];
-            for (size_t e = 0; e < (size_t)ns * per_slot; ++e) row[e * kTile] = tb[e];
+              for (int l = 0; l < per_slot; ++l) tb[(size_t)perm[s] * per_slot + l] = blk[at(s, l)];
+            for (int s = 0; s < ns; ++s)
+              for (int l = 0; l < per_slot; ++l) blk[at(s, l)] = tb[(size_t)s * per_slot + l];
           };
-          tmp.resize((size_t)ns * (size_t)std::max({m * 8, (m + 1) * 4, nq3 * 8, 4}));
+          auto permute = [&](auto* base, size_t stride_e, int per_slot) {
+            permute_at(base, stride_e, per_slot, [&](int s, int l) {
+              return ((size_t)s * per_slot + l) * kTile + ln;
+            });
+          };
+          tmp.resize((size_t)ns * (size_t)std::max({m * 8, nq3 * 8, 4}));
           permute(nbr.data(), SL, 1);
           if (store == TENO_FP64_NATIVE)
             permute(reinterpret_cast<double*>(ahat.data()), E, m);
@@ -1019,8 +1148,10 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
           else
             permute(reinterpret_cast<float*>(ahat.data()), E, m);
           if (wform) {
-            permute(g32.data(), E32s, m + 1);
-            permute(wq.data(), EWs, nq3);
+            permute_at(g32.data(), E32s, mc,
+                       [&](int s, int l) { return wform_g_index(ns, mc, s, l, ln); });
+            permute_at(wq.data(), EWs, nq3,
+                       [&](int s, int l) { return wform_w_index(ns, nq3, s, l, ln); });
           }
         }
       }
@@ -1077,9 +1208,13 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
       const int64_t ntl = nrp / kTile;
       std::vector<unsigned char> ahat_l((size_t)ntl * E * kTile * esz, 0);
       std::vector<float> g32_l(wform ? (size_t)ntl * E32 * kTile : 0, 0.f);
-      std::vector<float2> wq_l(wform ? (size_t)ntl * EW * kTile : 0, make_float2(0.f, 0.f));
-      std::vector<int32_t> nbr_l((size_t)ntl * SL * kTile, 0);
-      std::vector<uint8_t> smask_l((size_t)ntl * kTile, 0);
+      std::vector<int2> wq_l(wform ? (size_t)ntl * EW * kTile : 0, make_int2(0, 0));
+      std::vector<int32_t> wstat_l(wform ? (size_t)ntl * kWStat * kTile : 0, 60);
+      // (lanes without a cell point at their tile's first cell)
+      std::vector<int32_t> nbr_l((size_t)ntl * SL * kTile);
+      for (int64_t t = 0; t < ntl; ++t)
+        std::fill_n(&nbr_l[(size_t)t * SL * kTile], (size_t)SL * kTile, (int32_t)(t * kTile));
+      std::vector<uint8_t> smask_l((size_t)ntl * kTile, kMaskInert);
       for (size_t i = 0; i < comp.size(); ++i) {
         const int32_t c = comp[i];
         const int64_t k = slot_of_tile[c / kTile], lane = c % kTile;
@@ -1088,10 +1223,21 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
           memcpy(&ahat_l[(((size_t)kl * E + e) * kTile + ll) * esz],
                  &ahat[(((size_t)k * E + e) * kTile + lane) * esz], esz);
         if (wform) {
-          for (int e = 0; e < E32; ++e)
-            g32_l[((size_t)kl * E32 + e) * kTile + ll] = g32[((size_t)k * E32 + e) * kTile + lane];
-          for (int e = 0; e < EW; ++e)
-            wq_l[((size_t)kl * EW + e) * kTile + ll] = wq[((size_t)k * EW + e) * kTile + lane];
+          float* gd = &g32_l[(size_t)kl * E32 * kTile];
+          const float* gs = &g32[(size_t)k * E32 * kTile];
+          for (int s = 0; s < ns; ++s) {
+            for (int l = 0; l < mc; ++l)
+              gd[wform_g_index(ns, mc, s, l, (int)ll)] = gs[wform_g_index(ns, mc, s, l, (int)lane)];
+            for (int q = 0; q < nq3; ++q)
+              wq_l[(size_t)kl * EW * kTile + wform_w_index(ns, nq3, s, q, (int)ll)] =
+                  wq[(size_t)k * EW * kTile + wform_w_index(ns, nq3, s, q, (int)lane)];
+          }
+          for (int s = 0; s < kSmallK * kSmallN; ++s)
+            for (int l = 0; l < kSmallM; ++l)
+              gd[wform_s_index(ns, mc, s, l, (int)ll)] = gs[wform_s_index(ns, mc, s, l, (int)lane)];
+          for (int e = 0; e < kWStat; ++e)
+            wstat_l[((size_t)kl * kWStat + e) * kTile + ll] =
+                wstat[((size_t)k * kWStat + e) * kTile + lane];
         }
         for (int s = 0; s < SL; ++s)
           nbr_l[((size_t)kl * SL + s) * kTile + ll] =
@@ -1112,6 +1258,7 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
       ahat.swap(ahat_l);
       g32.swap(g32_l);
       wq.swap(wq_l);
+      wstat.swap(wstat_l);
       nbr.swap(nbr_l);
       smask.swap(smask_l);
       ntile = ntl;
@@ -1169,6 +1316,8 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   bool halo_ok = true;
   std::vector<int32_t> hoff(ntile + 1, 0), hids;
   std::vector<uint16_t> hloc((size_t)ntile * SL * kTile, 0);
+  std::vector<int32_t> wtile(wform ? (size_t)ntile * kWTile : 0, 0);
+  std::vector<uint16_t> wpos(wform ? (size_t)ntile * SL * kTile : 0, 0);
   {
     std::vector<int32_t> ids;
     for (int64_t t = 0; t < ntile && halo_ok; ++t) {
@@ -1191,7 +1340,17 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
           if (ln < nval)
             for (int j = 0; j < ln; ++j) rank += tn[(size_t)s * kTile + j] == tn[i];
           hloc[(size_t)t * SL * kTile + i] = (uint16_t)(pos | (rank << 8));
+          if (wform) wpos[(size_t)t * SL * kTile + i] = (uint16_t)(pos * 8);
         }
+      if (wform) {
+        int32_t* tb = &wtile[(size_t)t * kWTile];
+        tb[0] = (int32_t)ids.size();
+        uint32_t held = 0;
+        for (int ln = 0; ln < nval; ++ln)
+          if (!(smask[(size_t)t * kTile + ln] & kMaskInert)) held |= 1u << ln;
+        memcpy(&tb[1], &held, sizeof(held));
+        std::copy(ids.begin(), ids.end(), tb + 4);
+      }
       hids.insert(hids.end(), ids.begin(), ids.end());
       hoff[t + 1] = (int32_t)hids.size();
     }
@@ -1216,7 +1375,10 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   if (!e && halo_ok) e = upload(ctx, ctx->b_halo_loc, hloc.data(), hloc.size() * 2);
   if (!e) e = upload(ctx, ctx->b_smask, smask.data(), smask.size());
   if (!e && wform) e = upload(ctx, ctx->b_g32, g32.data(), g32.size() * sizeof(float));
-  if (!e && wform) e = upload(ctx, ctx->b_wq, wq.data(), wq.size() * sizeof(float2));
+  if (!e && wform) e = upload(ctx, ctx->b_wq, wq.data(), wq.size() * sizeof(int2));
+  if (!e && wform && halo_ok) e = upload(ctx, ctx->b_wtile, wtile.data(), wtile.size() * 4);
+  if (!e && wform && halo_ok) e = upload(ctx, ctx->b_wpos, wpos.data(), wpos.size() * 2);
+  if (!e && wform) e = upload(ctx, ctx->b_wstat, wstat.data(), wstat.size() * sizeof(int32_t));
   if (e) return e;
   // device mesh descriptor
   DeviceMesh& dm = ctx->dm;
@@ -1288,7 +1450,11 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   dm.err_flag = (int*)ctx->b_flag.p;
   dm.ahat = ctx->b_ahat.p;
   dm.g32 = wform ? (const float*)ctx->b_g32.p : nullptr;
-  dm.wq = wform ? (const float2*)ctx->b_wq.p : nullptr;
+  dm.wq = wform ? (const int2*)ctx->b_wq.p : nullptr;
+  dm.wstat = wform ? (const int32_t*)ctx->b_wstat.p : nullptr;
+  dm.wtile = wform && halo_ok ? (const int32_t*)ctx->b_wtile.p : nullptr;
+  dm.wpos = wform && halo_ok ? (const uint16_t*)ctx->b_wpos.p : nullptr;
+  if (wform) dm.wt = wb.table;
   dm.nbr = (const int32_t*)ctx->b_nbr.p;
   dm.smask = (const uint8_t*)ctx->b_smask.p;
   std::copy(R.psi_t, R.psi_t + kMaxPts * kMaxM, dm.eval.psi);
@@ -1806,7 +1972,7 @@ int teno_destroy(teno_ctx* ctx) {
   }
   cudaSetDevice(ctx->device);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  DevBuf* bufs[] = {&ctx->b_halo_off, &ctx->b_halo_ids, &ctx->b_halo_loc, &ctx->b_g32, &ctx->b_wq, &ctx->b_psi, &ctx->b_cspeed, &ctx->b_coef, &ctx->b_ahat, &ctx->b_nbr, &ctx->b_smask, &ctx->b_fcells, &ctx->b_fedges,
+  DevBuf* bufs[] = {&ctx->b_halo_off, &ctx->b_halo_ids, &ctx->b_halo_loc, &ctx->b_g32, &ctx->b_wq, &ctx->b_wstat, &ctx->b_wtile, &ctx->b_wpos, &ctx->b_psi, &ctx->b_cspeed, &ctx->b_coef, &ctx->b_ahat, &ctx->b_nbr, &ctx->b_smask, &ctx->b_fcells, &ctx->b_fedges,
                     &ctx->b_fgeom, &ctx->b_fgeom2, &ctx->b_cfaces, &ctx->b_inv_area, &ctx->b_cfl_len, &ctx->b_cfl_ilen2,
                     &ctx->b_perm, &ctx->b_U, &ctx->b_U1, &ctx->b_U2, &ctx->b_R, &ctx->b_tmp,
                     &ctx->b_Uq, &ctx->b_K, &ctx->b_sel, &ctx->b_sel_ovr, &ctx->b_maxlam,

@@ -11,6 +11,12 @@
 
 namespace teno {
 
+#ifdef __CUDACC__
+#define TENO_HD __host__ __device__
+#else
+#define TENO_HD
+#endif
+
 constexpr int kTile = 32;       // cells per tile of the cell-interleaved layouts
 constexpr int kSmallN = 12;     // neighbours of a directional stencil (2 N_k, r = 2)
 constexpr int kSmallM = 5;      // unknowns of a quadratic polynomial
@@ -36,6 +42,36 @@ struct DFTable {
   float2 psi[kMaxPts * kMaxM];
 };
 
+// W form of the Euler reconstruction (P = 3 nq Gauss points): smoothness rows
+// stored beside W, those of the orthogonal complement of Psi's row space
+TENO_HD constexpr int wform_rows(int m, int pts) { return m > pts ? m - pts : 0; }
+// words per cell and tile row of DeviceMesh::wstat
+constexpr int kWStat = 5;
+// large slots per ring stage (6 to 8.5 KB with their rows)
+TENO_HD constexpr int wform_lps(int ns) { return ns > 20 ? 2 : 4; }
+// Positions in a tile's rows (floats) and W (8-byte entries): stage by stage,
+// the entries of a stage in fours (pairs) of 16 bytes a lane, the rest singly.
+TENO_HD constexpr int wform_g_index(int ns, int rows, int s, int l, int lane) {
+  const int per = wform_lps(ns) * rows, r = (s % wform_lps(ns)) * rows + l;
+  return (s / wform_lps(ns)) * per * 32 +
+         (r < per / 4 * 4 ? ((r / 4) * 32 + lane) * 4 + r % 4 : r * 32 + lane);
+}
+TENO_HD constexpr int wform_s_index(int ns, int rows, int slot, int l, int lane) {  // slot: 0 .. 35
+  const int r = (slot % 12) * 5 + l;
+  return (ns * rows + (slot / 12) * 60) * 32 + ((r / 4) * 32 + lane) * 4 + r % 4;
+}
+TENO_HD constexpr int wform_w_index(int ns, int pts, int s, int p, int lane) {
+  const int per = wform_lps(ns) * pts, r = (s % wform_lps(ns)) * pts + p;
+  return (s / wform_lps(ns)) * per * 32 +
+         (r < per / 2 * 2 ? ((r / 2) * 32 + lane) * 2 + r % 2 : r * 32 + lane);
+}
+// the coefficients' part in the row space of Psi' from the values y = W d:
+// row i of t (min(m, P) rows of P; lower triangular when P <= m), and bounds
+// from above of its absolute column sums and of their sum
+struct WTable {
+  float t[81], cs[12], cs_all;
+};
+
 // Per-tile stencil halo: the distinct cells of a tile's stencils (internal
 // ids, at most kHaloMax per tile) and the stencil slots as halo-local indices.
 constexpr int kHaloMax = 256;
@@ -43,7 +79,11 @@ constexpr int kHaloMax = 256;
 // rank among the tile's lanes that hold the same cell in that slot (the
 // order of the adjoint's halo accumulation)
 constexpr int kHaloPosMask = 0xFF;
+constexpr int kMaskInert = 0x80;
 static_assert(kHaloMax <= kHaloPosMask + 1, "halo positions must fit in 8 bits");
+// words per tile of DeviceMesh::wtile: halo cells, lanes that hold a cell (bit
+// mask), two unused, the halo ids
+constexpr int kWTile = 4 + kHaloMax;
 struct HaloArgs {
   const int32_t* off = nullptr;       // [n_tiles + 1]
   const int32_t* ids = nullptr;       // [off[n_tiles]]
@@ -76,13 +116,27 @@ struct DeviceMesh {
   // reconstruction data, tile-interleaved [tile][entry][32]
   const void* ahat = nullptr;     // double (FP64_NATIVE), float2 (FP64) or float (mixed)
   const int32_t* nbr = nullptr;   // [tile][ns+36][32] internal cell ids
-  const uint8_t* smask = nullptr; // [n_pad] bit k: directional stencil k present
-  // Euler on the FP64 paths, recon_variant 2 (else null): FP32 matrices for
-  // the selection, per slot the rows then sum_l |G_ls| ([tile][ns*(m+1) +
-  // 36*6][32]), and W = Psi' G ([tile][ns*3*nq][32]) as (hi, lo) pairs on the
-  // pair path, as doubles (in the same 8 bytes) on the native path
+  // [n_pad] bit k: directional stencil k present; kMaskInert: a lane of a
+  // partition's layout that holds no cell
+  const uint8_t* smask = nullptr;
+  // Euler on the FP64 paths, recon_variant 2 (else null): FP32 rows for the
+  // selection, per large slot the wform_rows() of the complement Q2' G, per
+  // directional slot its 5 rows ([tile][ns*rows + 36*5][32]); W = Psi' G in
+  // fixed point in units of 2^-kc per cell ([tile][ns*3*nq][32]): on the pair
+  // path the integer x and the FP32 fraction y (its bits), sum_s |w_ps| < 2^31;
+  // on the native path x 2^30 + y, sum_s |w_ps| < 2^60; and per cell ([tile][kWStat][32]) the 2-norms
+  // of the column sums sum_l |.| of the complement rows and of the three
+  // directional stencils (FP32, rounded up), then kc (low half) and the
+  // stencil mask (from bit 16)
+  // (rows and W laid out by wform_*_index); per tile the halo ids
+  // ([tile][kWTile]) and the stencil slots as byte offsets in a row of 8-byte
+  // halo states ([tile][slot][32])
   const float* g32 = nullptr;
-  const float2* wq = nullptr;
+  const int2* wq = nullptr;
+  const int32_t* wstat = nullptr;
+  const int32_t* wtile = nullptr;
+  const uint16_t* wpos = nullptr;
+  WTable wt{};
   const float2* psi_df = nullptr;   // device copy of eval_df.psi (pair W form)
   const double* psi_d = nullptr;    // device copy of eval.psi (native W form)
   // faces

@@ -199,6 +199,10 @@ __device__ __forceinline__ void df_mac(DF& acc, float2 a, DF b) {
   acc.l += s.l + e;
 }
 __device__ __forceinline__ DF df_norm(DF a) { return two_sum(a.h, a.l); }
+__device__ __forceinline__ DF d_to_df(double x) {
+  const float h = (float)x;
+  return {h, (float)(x - (double)h)};
+}
 __device__ __forceinline__ double df_to_double(DF a) { return (double)a.h + (double)a.l; }
 
 
@@ -1535,11 +1539,6 @@ __device__ __forceinline__ void consumer_sync() {
 #ifndef TENO_STAGE_OUT
 #define TENO_STAGE_OUT 1
 #endif
-// the W-form kernel measured faster with its direct 8-byte pair stores (the
-// stage costs it a ring slot and a barrier per tile)
-#ifndef TENO_STAGE_OUT_W
-#define TENO_STAGE_OUT_W 0
-#endif
 template <int kPer, typename TO>
 __device__ __forceinline__ void store_out_stage(const TO* stg, TO* __restrict__ dst, int nvalid,
                                                 int tid) {
@@ -1883,585 +1882,1066 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), (kDF && kExt) ? 2 : 
   cp_async_wait<0>();
 }
 
-// ------------------------------------------- FP64 path, W form (variant 2)
-// Algebraically the same reconstruction as recon_tma_kernel<kDF = true>, with
-// the work split by what each quantity needs:
-//  - the Gauss-point values of the large polynomial, U_0 + Psi' (G d), are
-//    accumulated in pairs as U_0 + W d with W = Psi' G precomputed per cell
-//    (3 N_q pair products per stencil slot instead of m);
-//  - the smoothness indicators feed only the cutoff decision, so the stencil
-//    coefficients for beta are FP32 products G d with a rigorous error bound
-//    (per slot the column sum sum_l |G_ls| is stored next to the rows);
-//    where the bound does not separate chi from C_T the coefficients and
-//    beta are recomputed in pairs from the (hi, lo) matrices and the
-//    decision is taken in FP64;
-//  - directional-stencil values (cells where the large stencil is cut) are
-//    evaluated in pairs from the (hi, lo) matrices.
-#ifndef TENO_W_BLOCKS
-#define TENO_W_BLOCKS 3  // 3: three blocks per SM; 0: four where the ring fits
-#endif
-constexpr int kWBlocks = TENO_W_BLOCKS;
+// ------------------------------------------- FP64 paths, W form (variant 2)
+// The reconstruction with the work split by what each quantity needs:
+//  - the Gauss-point values of the large polynomial are U_0 + W d with
+//    W = Psi' G precomputed per cell.  The sums W d run in fixed point: the
+//    tile's halo states become integers Y of one power-of-two unit per tile
+//    and variable, relative to the tile's first cell, so differences are exact
+//    integer subtractions, and W is stored in fixed point with one unit per
+//    cell (WDot).  A product costs an FP64 multiply-add 64 lane slots (GB300's
+//    FP64 rate is 1/64 of its FP32 rate) and a pair multiply-add 12 FP32
+//    instructions; here it costs three wide integer multiply-adds (FP64 path;
+//    each holds its pipe for about 5 clocks a warp) or one and two FP32
+//    multiply-adds (pairs), and the sums are accurate to the bits of the
+//    result;
+//  - the smoothness indicators feed only the cutoff decision.  beta = |a|^2
+//    for the coefficients a = G d; the part of a in the row space of Psi' is
+//    a linear image T y of the values y = W d that are known anyway, so only
+//    the rows Q2' G of its orthogonal complement (m - 3 N_q of m) are stored
+//    and summed, in FP32, with a rigorous error bound: 6,100 bytes a cell at
+//    TENO6, where W with all rows and their bounds took 8,046.  Where the
+//    bound does not separate chi from C_T the coefficients and beta are
+//    recomputed (pairs, or FP64) and the decision is taken in FP64;
+//  - directional values (cells where the large stencil is cut) are evaluated
+//    from the (hi, lo) or FP64 matrices.
+// The last two are lists a warp works off apart from its tiles: one undecided
+// cell at a time by all lanes, 32 directional cells one per lane, so that their
+// chains of loads stall the warp once and not per cell and slot.
+// Bound: HBM at large meshes (1.6 GB a launch at 262,088 cells TENO6: 326 us,
+// 4.9 TB/s; with pair products, all rows and per-tile block barriers 470 us),
+// the FP64 path by its integer products (131,072 cells: 234 us; FP64
+// multiply-adds 608 us), small meshes by the time of one tile (2,046 cells
+// TENO5: 39 us, 52 before).
 
-template <int M, int NS, int NQ3, int kLPS, int kSPS>
+// Variables a consumer warp takes: two on the pair path, where the sums of
+// both share every shared-memory read of W and of the rows (262,088 cells,
+// TENO6: 326 us against 364 with one); one on the FP64 path, whose integer
+// sums need the registers (131,072 cells: 234 us against 256 with two).
+template <typename HT>
+constexpr int w_vars() {
+  return std::is_same<HT, double>::value ? 1 : 2;
+}
+
+template <int M, int NS, int NQ3, typename HT>
 struct WPlan {
-  static constexpr int kG = M + 1, kGs = kSmallM + 1;
-  static constexpr int kSlotG = kG * kTile * 4, kSlotW = NQ3 * kTile * 8;
-  static constexpr int kSlotS = kGs * kTile * 4;
-  static constexpr int kSlotN = kTile * 2;  // halo positions (uint16) of one slot
-  static constexpr int kNL = (NS + kLPS - 1) / kLPS;
-  static constexpr int kPerSmall = kSmallN / kSPS;
-  static constexpr int kStages = kNL + kSmallK * kPerSmall;
-  static constexpr int kMaxSlots = kLPS > kSPS ? kLPS : kSPS;
-  // ring buffer: [FP32 rows][W pairs][halo positions]
-  static constexpr int kGReg = kLPS * kSlotG > kSPS * kSlotS ? kLPS * kSlotG : kSPS * kSlotS;
-  static constexpr int kWOff = kGReg, kNOff = kGReg + kLPS * kSlotW;
-  static constexpr int kMat = kNOff + kMaxSlots * kSlotN;
-  static constexpr int kE32 = NS * kG + kSmallK * kSmallN * kGs;  // floats per lane per tile
-  static constexpr int kEW = NS * NQ3;                            // pairs per lane per tile
+  static constexpr int kVW = w_vars<HT>(), kWWarps = 4 / kVW;
+  static constexpr int kMC = wform_rows(M, NQ3);  // complement rows of a large slot
+  static constexpr int kLPS = wform_lps(NS);      // large slots a stage
+  static constexpr int kNG = kLPS * kMC, kNW = kLPS * NQ3;  // rows and W entries of a stage
+  static constexpr int kGB = kNG * kTile * 4, kWB = kNW * kTile * 8;
+  static constexpr int kSB = kSmallN * kSmallM * kTile * 4;  // rows of a directional stencil
+  static constexpr int kSlotN = kTile * 2;  // halo offsets (uint16) of one slot
+  static constexpr int kNL = NS / kLPS;
+  static constexpr int kStages = kSmallK + kNL;  // the directional stencils first
+  static constexpr int kStatBytes = kWStat * kTile * 4;
+  // ring buffer of a large stage: [FP32 rows][W][halo offsets][cell words];
+  // of a directional stage: [FP32 rows][halo offsets]
+  static constexpr int kWOff = kGB, kNOff = kWOff + kWB;
+  static constexpr int kXOff = kNOff + kLPS * kSlotN;
+  static constexpr int kBufL = kXOff + kStatBytes, kBufS = kSB + kSmallN * kSlotN;
+  static constexpr int kBuf = (kBufL > kBufS ? kBufL : kBufS);
+  static constexpr int kE32 = NS * kMC + kSmallK * kSmallN * kSmallM;  // floats per lane
+  static constexpr int kEW = NS * NQ3;                                 // W entries per lane
   static constexpr int kSL = NS + kSmallSlots;
-  static constexpr size_t kHaloBytes = (size_t)2 * 4 * kHaloMax * sizeof(float2);
-  // output stage of the Gauss-point pairs of one tile (float2 elements)
-  static constexpr size_t kOut = TENO_STAGE_OUT_W ? out_stage_bytes<NQ3 * 4, float2>() : 0;
-  static constexpr size_t kFixed = kHaloBytes + 2 * 4 * 8 + 16 + kOut;
-  // blocks of 160 threads per SM (228 KB of shared memory, 1 KB reserved per
-  // block): four with a 3-deep ring where that fits, else three (4-deep
-  // ring if it fits)
-  static constexpr bool kFour = kWBlocks != 3 &&
-                                4 * ((size_t)3 * kMat + kFixed + 1024) <= (size_t)228 * 1024;
-  static constexpr int kRingW =
-      kFour ? 3 : (3 * ((size_t)4 * kMat + kFixed + 1024) <= (size_t)228 * 1024 ? 4 : 3);
-  static constexpr int kBlocks = kFour ? 4 : 3;
-  static constexpr size_t kOutOff = (size_t)kRingW * kMat + kHaloBytes + 2 * kRingW * 8 + 16;
-  static constexpr size_t kSmem = kOutOff + kOut;
-  static_assert(kSmallN % kSPS == 0, "directional stencil split");
-  static_assert(kSlotG % 16 == 0 && kSlotW % 16 == 0 && kSlotS % 16 == 0 && kMat % 16 == 0,
-                "bulk-copy sizes");
-  // stage j: slots [slot0, slot0 + nslot) of stencil k (-1: large); byte
-  // offsets / sizes of its FP32 block (og, bg) and W block (ow, bw) in the tile
-  __device__ static void stage(int j, int& slot0, int& nslot, int& k, int& og, int& bg, int& ow,
-                               int& bw) {
-    if (j < kNL) {
-      slot0 = j * kLPS;
-      nslot = (NS - slot0) < kLPS ? (NS - slot0) : kLPS;
-      k = -1;
-      og = slot0 * kSlotG;
-      bg = nslot * kSlotG;
-      ow = slot0 * kSlotW;
-      bw = nslot * kSlotW;
-    } else {
-      const int i = j - kNL;
-      k = i / kPerSmall;
-      const int s0 = (i % kPerSmall) * kSPS;
-      slot0 = NS + k * kSmallN + s0;
-      nslot = kSPS;
-      og = NS * kSlotG + (k * kSmallN + s0) * kSlotS;
-      bg = kSPS * kSlotS;
-      ow = 0;
-      bw = 0;
-    }
-  }
+  static constexpr int kTileBytes = kWTile * 4;
+  static constexpr int kHaloRow = kHaloMax + kTile;     // halo states, then the tile's own
+  static constexpr int kHalo = 2 * 4 * kHaloRow * 8;    // double-buffered, per variable
+  static constexpr int kListN = (kVW + 1) * kTile;      // deferred cells of a warp
+  static constexpr int kScratch = kSL * 8;              // differences of one cell, per warp
+  static constexpr int kFixed =
+      kHalo + 2 * kTileBytes + kWWarps * (kListN * 8 + kScratch) + 16 * 8 + 16;
+  // four blocks per SM (96 threads of up to 168 registers, or 160 of 96); the
+  // ring takes what is left of their quarter of the 227 KB of shared memory
+  static constexpr int kRoom = (227 * 1024 / 4 - 1024 - kFixed) / kBuf;
+  static constexpr int kRingW = kRoom < 2 ? 2 : (kRoom > 5 ? 5 : kRoom);
+  static constexpr size_t kSmem = (size_t)kRingW * kBuf + kFixed;
+  static_assert(NS % kLPS == 0, "whole stages");
+  static_assert(kBuf % 16 == 0 && kWOff % 16 == 0 && kNOff % 16 == 0 && kXOff % 16 == 0 &&
+                    kSB % 16 == 0 && kTileBytes % 16 == 0,
+                "bulk-copy alignment");
 };
 
-// Upper bound of |beta_fp32 - beta| relative to beta_fp32 + eps for m FP32
-// coefficients a32_l from n-term FP32 dot products.  Coefficient l errs by at
-// most e_l = (n + 7) u S_l with S_l = sum_s |G_ls| |d_s| (u = 2^-24; the
-// stored matrix rounding and a difference conversion of up to 2u -- the FP64
-// path truncates -- included), and sum_l S_l = e_abs = sum_s colsum_s |d_s|.
-// With E = sum_l e_l, Cauchy-Schwarz gives
-// |sum a32^2 - sum a^2| <= sum e_l (2 |a32_l| + e_l) <= 2 E sqrt(beta32) + E^2;
-// the FP32 sum of squares adds (m + 2) u beta32.  Returns a value >= 1 when
-// the bound is not informative.
-__device__ __forceinline__ float beta_rel_bound(float beta32, float e_abs, int n, int m,
-                                                float eps) {
+// Upper bound of |beta32 - beta| relative to beta32 + eps, for beta32 the FP32
+// sum of squares of m coefficients whose absolute errors sum to at most E:
+// |sum a32^2 - sum a^2| <= sum e_l (2 |a32_l| + e_l) <= 2 E sqrt(beta32) + E^2,
+// and the FP32 sum of squares adds (m + 2) u beta32 (u = 2^-24).  Returns a
+// value >= 1 when the bound is not informative.
+__device__ __forceinline__ float beta_rel_bound(float beta32, float E, int m, float eps) {
   const float u = 5.9604645e-8f;
-  const float E = (float)(n + 7) * u * e_abs * 1.0001f;
-  const float eb = (float)(m + 2) * u * beta32 + E * (2.f * sqrtf(beta32) + E);
+  const float eb = (float)(m + 2) * u * beta32 + E * (2.0001f * sqrt_approx(beta32) + E);
   const float t = beta32 + eps;
   if (!(eb < 0.5f * t)) return 1.f;
-  return eb / (t - eb);
+  return 1.0002f * eb * rcp_approx(t - eb);
+}
+// The coefficients of n differences known to 2u relative plus one unit q each:
+// coefficient l errs by at most (n + 7) u S_l + q sum_s |G_ls| with
+// S_l = sum_s |G_ls| |d_s|, and sum_l S_l = sum_s colsum_s |d_s| <=
+// |colsum|_2 |d|_2 (norm: |colsum|_2, rounded up; dd: sum of the squared FP32
+// differences).
+__device__ __forceinline__ float dot_bound(float norm, float dd, float q, int n) {
+  const float u = 5.9604645e-8f;
+  const float len = sqrt_approx(dd) * 1.0002f;
+  return norm * ((float)(n + 7) * u * len + 7.f * q) * 1.0001f;  // sqrt(n) <= 7
 }
 
-// FP64 -> FP32 by truncation of the significand, in integer instructions
-// (the conversion instruction would take a slot of the FP64 pipe, which bounds
-// the FP64 path's reconstruction).  Relative error below 2^-23 for results in
-// the normal FP32 range; magnitudes below it give a signed zero (an absolute
-// error under 1.2e-38), magnitudes above it, infinities and NaN give an
-// infinity, which the cutoff screen sends to its FP64 fallback.
-__device__ __forceinline__ float d2f_trunc(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned sign = hi & 0x80000000u;
-  const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;
-  if (e <= 0) return __uint_as_float(sign);
-  if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
-  return __uint_as_float(sign | ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+// 2^e as FP32 (zero below the normal range, infinity above it)
+__device__ __forceinline__ float exp2i(int e) {
+  return e < -126 ? 0.f : (e > 127 ? __int_as_float(0x7f800000) : __int_as_float((e + 127) << 23));
+}
+// m 2^sh rounded to the nearest integer, m >= 0
+__device__ __forceinline__ int64_t shift_round(int64_t m, int sh) {
+  if (sh >= 0) return m << sh;
+  if (sh < -62) return 0;
+  return (m + ((int64_t)1 << (-sh - 1))) >> -sh;
+}
+// x 2^k as an integer, rounded (|x| 2^k < 2^62)
+__device__ __forceinline__ int64_t to_fix(float x, int k) {
+  const int b = __float_as_int(x);
+  const int ef = (b >> 23) & 0xff;
+  const int64_t m = (b & 0x7fffff) | (ef ? 0x800000 : 0);
+  const int64_t r = shift_round(m, (ef ? ef : 1) - 150 + k);
+  return b < 0 ? -r : r;
+}
+__device__ __forceinline__ int64_t to_fix(double x, int k) {
+  const int hi = __double2hiint(x);
+  const int ef = (hi >> 20) & 0x7ff;
+  const int64_t m = ((int64_t)((hi & 0xfffff) | (ef ? 0x100000 : 0)) << 32) |
+                    (uint32_t)__double2loint(x);
+  const int64_t r = shift_round(m, (ef ? ef : 1) - 1075 + k);
+  return hi < 0 ? -r : r;
+}
+__device__ __forceinline__ int64_t to_fix(float2 x, int k) { return to_fix(x.x, k) + to_fix(x.y, k); }
+// magnitude bits of a state (ordered like |x|) and their unbiased exponent;
+// kFixExpBad marks infinities and NaN
+constexpr int kFixExpBad = 1 << 20;
+__device__ __forceinline__ unsigned mag_bits(float2 x) {
+  return (unsigned)__float_as_int(x.x) & 0x7fffffffu;
+}
+__device__ __forceinline__ unsigned mag_bits(double x) {
+  return (unsigned)__double2hiint(x) & 0x7fffffffu;
+}
+template <typename HT>
+__device__ __forceinline__ int mag_exp(unsigned m) {
+  if constexpr (std::is_same<HT, double>::value) {
+    const int f = (int)(m >> 20);
+    return f == 0x7ff ? kFixExpBad : f - 1023;
+  } else {
+    const int f = (int)(m >> 23);
+    return f == 0xff ? kFixExpBad : (f ? f : 1) - 127;
+  }
+}
+// limbs x = h 2^30 + l with l in [0, 2^30)
+constexpr int kFixB = 30;
+__device__ __forceinline__ void fix_limbs(int64_t x, int& h, int& l) {
+  h = (int)(x >> kFixB);
+  l = (int)x & ((1 << kFixB) - 1);
+}
+// entry e of a stage's W (pairs of entries as 16 bytes a lane, a last odd one
+// as 8) and of its FP32 rows (fours as 16 bytes, the rest one by one)
+template <int N>
+__device__ __forceinline__ int2 w_entry(const unsigned char* wb, int lane, int e) {
+  if (e < N / 2 * 2) {
+    const int4 q = reinterpret_cast<const int4*>(wb)[(e / 2) * kTile + lane];
+    return e & 1 ? make_int2(q.z, q.w) : make_int2(q.x, q.y);
+  }
+  return reinterpret_cast<const int2*>(wb)[e * kTile + lane];
+}
+template <int N>
+__device__ __forceinline__ float g_entry(const unsigned char* gb, int lane, int e) {
+  if (e < N / 4 * 4) {
+    const float4 q = reinterpret_cast<const float4*>(gb)[(e / 4) * kTile + lane];
+    return (e & 3) == 0 ? q.x : ((e & 3) == 1 ? q.y : ((e & 3) == 2 ? q.z : q.w));
+  }
+  return reinterpret_cast<const float*>(gb)[e * kTile + lane];
+}
+__device__ __forceinline__ void mad_wide(int64_t& acc, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
+// (hh, mid) += (w.x 2^30 + w.y) (dh 2^30 + dl), without the low product
+__device__ __forceinline__ void fix_mac(int64_t& hh, int64_t& mid, int2 w, int dh, int dl) {
+  mad_wide(hh, w.x, dh);
+  mad_wide(mid, w.x, dl);
+  mad_wide(mid, w.y, dh);
+}
+__device__ __forceinline__ int64_t fix_sum(int64_t hh, int64_t mid) {
+  return hh + ((mid + ((int64_t)1 << (kFixB - 1))) >> kFixB);
 }
 
-// pair difference U_s - U_0 of a halo cell (FP32 hi/lo splits of the states)
-__device__ __forceinline__ DF halo_dif(const float2* st, int idx, float2 u0s) {
-  const float2 q = st[idx];
+// The sums W d of the two paths: difference parts D, accumulator A.
+template <typename HT>
+struct WDot;
+// FP64 path (kN): integers throughout, as fix_mac.
+template <>
+struct WDot<double> {
+  static constexpr int kBits = 57;      // |Y| < 2^57
+  // bound of the sum's error: kErr units 2^exp, plus kErrD 2^-kc |d|_2
+  static constexpr float kErr = 256.f, kErrD = 0.f;
+  // an integer of |x| 2^sc < 2^57
+  __device__ __forceinline__ static int64_t fix(double x, int sc, double) { return to_fix(x, sc); }
+  struct D {
+    int h, l;
+  };
+  struct A {
+    int64_t hh = 0, mid = 0;
+  };
+  struct W {
+    int2 m;
+  };
+  __device__ __forceinline__ static W entry(int2 m) { return {m}; }
+  __device__ __forceinline__ static float c(int sc) { return exp2i(kFixB - sc); }
+  // the parts and the FP32 value (c = 2^(30 - sc)) of a difference
+  __device__ __forceinline__ static float split(int64_t d, float c, D& o) {
+    fix_limbs(d, o.h, o.l);
+    return fmaf((float)o.h, c, (float)o.l * (c * (1.f / 1073741824.f)));
+  }
+  __device__ __forceinline__ static void mac(A& a, W w, D d) {
+    fix_mac(a.hh, a.mid, w.m, d.h, d.l);
+  }
+  __device__ __forceinline__ static int64_t sum(const A& a) { return fix_sum(a.hh, a.mid); }
+  __device__ __forceinline__ static int exp(int kc, int sc) { return 2 * kFixB - kc - sc; }
+};
+// Pairs: w = wh + wl with wh a 32-bit integer (sum_s |w_ps| < 2^31) and wl an
+// FP32 fraction, d = (dh + dl) 2^B likewise (|dh| <= 2^30): sum wh dh is exact
+// in 64 bits and wl dh + wh dl, 2^-31 of it, is an FP32 sum (two FP32
+// multiply-adds in the place of two wide ones; a wide multiply-add holds its
+// pipe for 5 clocks).  Accurate to about 2^-53 of |W|_1 times the tile's state
+// range, beyond the 48 bits of the pair it becomes.
+template <int kB>
+struct WPairDot {
+  static constexpr int kBits = kB + 29;
+  // the FP32 sum's 2 n roundings, each 2^-25 of |x| <= sum (|wl| |dh| + |wh| |dl|) <=
+  // (sqrt(n) |dh|_2 + 2^31) / 2
+  static constexpr float kErr = 8192.f, kErrD = 2e-5f;
+  // an integer of |x| 2^sc < 2^51, from the low bits of 1.5 2^52 + x 2^sc (c = 2^sc)
+  __device__ __forceinline__ static int64_t fix(double x, int, double c) {
+    return __double_as_longlong(fma(x, c, 6755399441055744.0)) - 0x4338000000000000LL;
+  }
+  struct D {
+    int h;
+    float hf, lf;
+  };
+  struct A {
+    int64_t hh = 0;
+    float x = 0.f;
+  };
+  struct W {
+    int h;
+    float hf, lf;
+  };
+  __device__ __forceinline__ static W entry(int2 m) {
+    return {m.x, (float)m.x, __int_as_float(m.y)};
+  }
+  __device__ __forceinline__ static float c(int sc) { return exp2i(kB - sc); }
+  __device__ __forceinline__ static float split(int64_t d, float c, D& o) {
+    o.h = (int)((d + (1 << (kB - 1))) >> kB);
+    o.hf = (float)o.h;
+    o.lf = (float)(((int)d << (32 - kB)) >> (32 - kB)) * (1.f / (1 << kB));
+    return (o.hf + o.lf) * c;
+  }
+  __device__ __forceinline__ static void mac(A& a, W w, D d) {
+    mad_wide(a.hh, w.h, d.h);
+    a.x = fmaf(w.hf, d.lf, a.x);
+    a.x = fmaf(w.lf, d.hf, a.x);
+  }
+  // (sum wh dh + x) 2^exp
+  __device__ __forceinline__ static DF value(const A& a, float s2, float s1, float s0) {
+    const float h = (float)(int)(a.hh >> 42) * s2;
+    const float m = (float)(int)((a.hh >> 21) & 0x1fffff) * s1;
+    const float l = ((float)(int)(a.hh & 0x1fffff) + a.x) * s0;
+    const DF r = fast_two_sum(h, m);
+    return two_sum(r.h, r.l + l);
+  }
+  __device__ __forceinline__ static double value_d(const A& a) {
+    return (double)a.hh + (double)a.x;
+  }
+  __device__ __forceinline__ static int exp(int kc, int sc) { return kB - kc - sc; }
+};
+// (the low bits of an FP64 sum give 51-bit differences)
+template <>
+struct WDot<float2> : WPairDot<22> {};
+// x 2^e as a pair (|x| < 2^62; e within the FP32 range less 42)
+__device__ __forceinline__ DF fix_to_df(int64_t x, float s2, float s1, float s0) {
+  const float h = (float)(int)(x >> 42) * s2;
+  const float m = (float)(int)((x >> 21) & 0x1fffff) * s1;
+  const float l = (float)(int)(x & 0x1fffff) * s0;
+  DF r = fast_two_sum(h, m);
+  r.l += l;
+  return fast_two_sum(r.h, r.l);
+}
+
+// pair difference U_s - U_0 of a neighbour (FP32 hi/lo splits of the states)
+__device__ __forceinline__ DF pair_dif(float2 q, float2 u0s) {
   DF t = two_sum(q.x, -u0s.x);
   t.l += q.y - u0s.y;
   return two_sum(t.h, t.l);
 }
 
-// Rare paths of the W-form kernel, kept out of line so that their registers
-// do not weigh on the main loop.  A: the cell's (hi, lo) matrices at its lane,
-// nb: its halo positions, st: the tile's halo of its variable.
-//
-// Cutoff decision in FP64 from coefficients and beta in pairs.
-template <int M, int NS>
-__device__ __noinline__ uint8_t w_select_pairs(const float2* A, const uint16_t* nb,
-                                               const float2* st, float2 u0s, int present,
-                                               double ct, double eps) {
-  DF al[M];
-#pragma unroll
-  for (int l = 0; l < M; ++l) al[l] = DF{0.f, 0.f};
-  for (int s = 0; s < NS; ++s) {
-    const DF d = halo_dif(st, nb[s * kTile] & kHaloPosMask, u0s);
-#pragma unroll
-    for (int l = 0; l < M; ++l) df_mac(al[l], __ldg(A + (int64_t)(s * M + l) * kTile), d);
+// Arithmetic of the deferred evaluations: pairs (float2 states) or FP64.
+template <typename HT>
+struct WArith;
+template <>
+struct WArith<float2> {
+  using Acc = DF;
+  __device__ __forceinline__ static DF zero() { return DF{0.f, 0.f}; }
+  __device__ __forceinline__ static DF dif(float2 q, float2 u0) { return pair_dif(q, u0); }
+  __device__ __forceinline__ static void mac(DF& acc, float2 m, DF d) { df_mac(acc, m, d); }
+  __device__ __forceinline__ static DF norm(DF x) { return df_norm(x); }
+  __device__ __forceinline__ static float2 entry(DF x) { return make_float2(x.h, x.l); }
+  __device__ __forceinline__ static DF shfl(DF x, int l) {
+    return DF{__shfl_sync(0xffffffffu, x.h, l), __shfl_sync(0xffffffffu, x.l, l)};
   }
+  __device__ __forceinline__ static DF add(DF a, DF b) {
+    DF q = two_sum(a.h, b.h);
+    q.l += a.l + b.l;
+    return two_sum(q.h, q.l);
+  }
+  __device__ __forceinline__ static DF div(DF a, int n) {  // exact remainder correction
+    const float fn = (float)n, qh = a.h / fn, r = fmaf(-qh, fn, a.h);
+    return two_sum(qh, (r + a.l) / fn);
+  }
+  __device__ __forceinline__ static float2 value(float2 u0, DF x) {
+    const DF r = DF{u0.x, u0.y} + x;
+    return make_float2(r.h, r.l);
+  }
+};
+template <>
+struct WArith<double> {
+  using Acc = double;
+  __device__ __forceinline__ static double zero() { return 0.0; }
+  __device__ __forceinline__ static double dif(double q, double u0) { return q - u0; }
+  __device__ __forceinline__ static void mac(double& acc, double m, double d) {
+    acc = fma(m, d, acc);
+  }
+  __device__ __forceinline__ static double norm(double x) { return x; }
+  __device__ __forceinline__ static double entry(double x) { return x; }
+  __device__ __forceinline__ static double shfl(double x, int l) {
+    return __shfl_sync(0xffffffffu, x, l);
+  }
+  __device__ __forceinline__ static double add(double a, double b) { return a + b; }
+  __device__ __forceinline__ static double div(double a, int n) { return a / (double)n; }
+  __device__ __forceinline__ static double value(double u0, double x) { return u0 + x; }
+};
+
+// Cutoff decision of one cell in FP64, by the whole warp (the cells it is
+// needed for are few and far between, so one lane per cell would leave the
+// warp waiting for a chain of loads).  A: the cell's matrices at its lane,
+// nb: its stencil cells, st: the states of the variable, dsc: the warp's
+// scratch.  The differences are gathered one slot per lane, then lane q forms
+// coefficient q (of the large stencil's m and the directional 15), and beta
+// and the decision follow in every lane.
+template <int M, int NS, typename HT>
+__device__ __noinline__ int w_select(const HT* A, const int32_t* nb, const HT* st, HT u0,
+                                     int present, double ct, double eps, HT* dsc) {
+  using Ar = WArith<HT>;
+  using Acc = typename Ar::Acc;
+  constexpr int SL = NS + kSmallSlots, NC = M + kSmallK * kSmallM;
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < (SL + kTile - 1) / kTile; ++i) {
+    const int s = lane + i * kTile;
+    if (s < SL) dsc[s] = Ar::entry(Ar::dif(__ldg(st + __ldg(nb + s * kTile)), u0));
+  }
+  __syncwarp();
+  auto coef = [&](int q) {
+    Acc acc = Ar::zero();
+    const bool lg = q < M;
+    const int k = lg ? 0 : (q - M) / kSmallM, l = lg ? q : (q - M) % kSmallM;
+    const int n = q >= NC ? 0 : (lg ? NS : kSmallN);
+    const int rows = lg ? M : kSmallM;
+    const HT* Aq = A + (int64_t)(lg ? l : M * NS + k * kSmallN * kSmallM + l) * kTile;
+    const HT* dq = dsc + (lg ? 0 : NS + k * kSmallN);
+#pragma unroll 6
+    for (int s = 0; s < n; ++s) {
+      const HT d = dq[s];
+      if constexpr (std::is_same<HT, double>::value)
+        Ar::mac(acc, __ldg(Aq + (int64_t)s * rows * kTile), d);
+      else
+        Ar::mac(acc, __ldg(Aq + (int64_t)s * rows * kTile), DF{d.x, d.y});
+    }
+    return Ar::norm(acc);
+  };
+  const Acc c0 = coef(lane);
+  Acc c1 = Ar::zero();
+  if constexpr (NC > kTile) c1 = coef(lane + kTile);
+  __syncwarp();
+  auto sum_sq = [&](int q0, int n) {
+    Acc b = Ar::zero();
+#pragma unroll 1
+    for (int q = q0; q < q0 + n; ++q) {
+      const Acc x = Ar::shfl(q < kTile ? c0 : c1, q & 31);
+      Ar::mac(b, Ar::entry(x), x);
+    }
+    return to_d(Ar::norm(b));
+  };
   double beta[kSmallK + 1];
-  {
-    DF bl = {0.f, 0.f};
+  beta[kSmallK] = sum_sq(0, M);
 #pragma unroll
-    for (int l = 0; l < M; ++l) {
-      const DF x = df_norm(al[l]);
-      df_mac(bl, make_float2(x.h, x.l), x);
-    }
-    beta[kSmallK] = df_to_double(df_norm(bl));
-  }
-#pragma unroll
-  for (int k = 0; k < kSmallK; ++k) {
-    DF as[kSmallM];
-#pragma unroll
-    for (int l = 0; l < kSmallM; ++l) as[l] = DF{0.f, 0.f};
-    if ((present >> k) & 1) {
-      for (int s = 0; s < kSmallN; ++s) {
-        const DF d = halo_dif(st, nb[(NS + k * kSmallN + s) * kTile] & kHaloPosMask, u0s);
-        const float2* As = A + (int64_t)(M * NS + (k * kSmallN + s) * kSmallM) * kTile;
-#pragma unroll
-        for (int l = 0; l < kSmallM; ++l) df_mac(as[l], __ldg(As + l * kTile), d);
-      }
-    }
-    DF q = {0.f, 0.f};
-#pragma unroll
-    for (int l = 0; l < kSmallM; ++l) {
-      const DF x = df_norm(as[l]);
-      df_mac(q, make_float2(x.h, x.l), x);
-    }
-    beta[k] = df_to_double(df_norm(q));
-  }
+  for (int k = 0; k < kSmallK; ++k)
+    beta[k] = (present >> k) & 1 ? sum_sq(M + k * kSmallM, kSmallM) : 0.0;
   return select_fp64(beta, present, ct, eps);
 }
 
 // Gauss-point values of the equally weighted kept directional polynomials
-// (step ii of the selection), in pairs; psi: the [point][kMaxM] table of
-// Psi' as pairs.
-template <int M, int NS, int NQ3, int NV>
-__device__ __noinline__ void w_small_values(const float2* A, const uint16_t* nb, const float2* st,
-                                            float2 u0s, uint8_t sel, const float2* psi,
-                                            float2* out) {
-  DF sum[kSmallM];
+// (step ii of the selection), one cell and variable per lane; psi: the
+// [point][kMaxM] table of Psi'.  A stencil's cells and states are requested
+// together, its matrix entries four slots at a time.
+template <int M, int NS, int NQ3, int NV, typename HT>
+__device__ __noinline__ void w_small(const HT* A, const int32_t* nb, const HT* st, HT u0, int sel,
+                                     const HT* psi, HT* out) {
+  using Ar = WArith<HT>;
+  using Acc = typename Ar::Acc;
+  Acc sum[kSmallM];
 #pragma unroll
-  for (int l = 0; l < kSmallM; ++l) sum[l] = DF{0.f, 0.f};
+  for (int l = 0; l < kSmallM; ++l) sum[l] = Ar::zero();
+#pragma unroll 1
   for (int k = 0; k < kSmallK; ++k) {
     if (!((sel >> k) & 1)) continue;
-    DF as[kSmallM];
+    const int32_t* nk = nb + (NS + k * kSmallN) * kTile;
+    const HT* Ak = A + (int64_t)(M * NS + k * kSmallN * kSmallM) * kTile;
+    int id[kSmallN];
+    HT q[kSmallN];
 #pragma unroll
-    for (int l = 0; l < kSmallM; ++l) as[l] = DF{0.f, 0.f};
+    for (int s = 0; s < kSmallN; ++s) id[s] = __ldg(nk + s * kTile);
+#pragma unroll
+    for (int s = 0; s < kSmallN; ++s) q[s] = __ldg(st + id[s]);
+    Acc as[kSmallM];
+#pragma unroll
+    for (int l = 0; l < kSmallM; ++l) as[l] = Ar::zero();
+#pragma unroll
     for (int s = 0; s < kSmallN; ++s) {
-      const DF d = halo_dif(st, nb[(NS + k * kSmallN + s) * kTile] & kHaloPosMask, u0s);
-      const float2* As = A + (int64_t)(M * NS + (k * kSmallN + s) * kSmallM) * kTile;
+      const Acc d = Ar::dif(q[s], u0);
 #pragma unroll
-      for (int l = 0; l < kSmallM; ++l) df_mac(as[l], __ldg(As + l * kTile), d);
+      for (int l = 0; l < kSmallM; ++l) Ar::mac(as[l], __ldg(Ak + (s * kSmallM + l) * kTile), d);
     }
 #pragma unroll
-    for (int l = 0; l < kSmallM; ++l) {
-      const DF x = df_norm(as[l]);
-      DF q = two_sum(sum[l].h, x.h);
-      q.l += sum[l].l + x.l;
-      sum[l] = two_sum(q.h, q.l);
-    }
+    for (int l = 0; l < kSmallM; ++l) sum[l] = Ar::add(sum[l], Ar::norm(as[l]));
   }
-  // divide by the number of kept stencils (exact remainder correction)
   const int nd = (sel & 1) + ((sel >> 1) & 1) + ((sel >> 2) & 1);
-  const float fn = (float)(nd ? nd : 1);
-  DF cf[kSmallM];
+  Acc cf[kSmallM];
 #pragma unroll
-  for (int l = 0; l < kSmallM; ++l) {
-    const float qh = sum[l].h / fn;
-    const float r = fmaf(-qh, fn, sum[l].h);
-    cf[l] = nd ? two_sum(qh, (r + sum[l].l) / fn) : DF{0.f, 0.f};
-  }
-  const DF u0 = {u0s.x, u0s.y};
+  for (int l = 0; l < kSmallM; ++l) cf[l] = nd ? Ar::div(sum[l], nd) : Ar::zero();
+#pragma unroll 1
   for (int p = 0; p < NQ3; ++p) {
-    DF sp = {0.f, 0.f};
+    Acc sp = Ar::zero();
 #pragma unroll
-    for (int l = 0; l < kSmallM; ++l) df_mac(sp, __ldg(psi + p * kMaxM + l), cf[l]);
-    const DF r = u0 + df_norm(sp);
+    for (int l = 0; l < kSmallM; ++l) Ar::mac(sp, __ldg(psi + p * kMaxM + l), cf[l]);
+    out[p * NV] = Ar::value(u0, Ar::norm(sp));
+  }
+}
+
+// Large-stencil values of a cell whose tile holds an infinity, a NaN or a
+// magnitude outside the fixed-point range: U_0 + W d in floating point.
+template <int NS, int NQ3, int NV>
+__device__ __noinline__ void w_direct(const int2* W, int lane, int kc, const int32_t* nb,
+                                      const float2* st, float2 u0s, float2* out) {
+#pragma unroll 1
+  for (int p = 0; p < NQ3; ++p) {
+    DF acc = {0.f, 0.f};
+#pragma unroll 1
+    for (int s = 0; s < NS; ++s) {
+      const int2 w = W[wform_w_index(NS, NQ3, s, p, lane)];
+      const DF q = d_to_df(ldexp((double)w.x + (double)__int_as_float(w.y), -kc));
+      df_mac(acc, make_float2(q.h, q.l), pair_dif(st[nb[s * kTile]], u0s));
+    }
+    const DF r = DF{u0s.x, u0s.y} + df_norm(acc);
     out[p * NV] = make_float2(r.h, r.l);
   }
 }
-
-// The same two rare paths on the FP64 pipe (native FP64 W form): A is the
-// cell's FP64 matrices at its lane, st the tile's halo of FP64 states.
-template <int M, int NS>
-__device__ __noinline__ uint8_t w_select_native(const double* A, const uint16_t* nb,
-                                                const double* st, double u0, int present,
-                                                double ct, double eps) {
-  double al[M];
-#pragma unroll
-  for (int l = 0; l < M; ++l) al[l] = 0.0;
-  for (int s = 0; s < NS; ++s) {
-    const double d = st[nb[s * kTile] & kHaloPosMask] - u0;
-#pragma unroll
-    for (int l = 0; l < M; ++l) al[l] = fma(__ldg(A + (int64_t)(s * M + l) * kTile), d, al[l]);
-  }
-  double beta[kSmallK + 1];
-  {
-    double b = 0.0;
-#pragma unroll
-    for (int l = 0; l < M; ++l) b = fma(al[l], al[l], b);
-    beta[kSmallK] = b;
-  }
-#pragma unroll
-  for (int k = 0; k < kSmallK; ++k) {
-    double as[kSmallM];
-#pragma unroll
-    for (int l = 0; l < kSmallM; ++l) as[l] = 0.0;
-    if ((present >> k) & 1) {
-      for (int s = 0; s < kSmallN; ++s) {
-        const double d = st[nb[(NS + k * kSmallN + s) * kTile] & kHaloPosMask] - u0;
-        const double* As = A + (int64_t)(M * NS + (k * kSmallN + s) * kSmallM) * kTile;
-#pragma unroll
-        for (int l = 0; l < kSmallM; ++l) as[l] = fma(__ldg(As + l * kTile), d, as[l]);
-      }
-    }
-    double q = 0.0;
-#pragma unroll
-    for (int l = 0; l < kSmallM; ++l) q = fma(as[l], as[l], q);
-    beta[k] = q;
-  }
-  return select_fp64(beta, present, ct, eps);
-}
-
-template <int M, int NS, int NQ3, int NV>
-__device__ __noinline__ void w_small_native(const double* A, const uint16_t* nb, const double* st,
-                                            double u0, uint8_t sel, const double* psi,
-                                            double* out) {
-  double sum[kSmallM];
-#pragma unroll
-  for (int l = 0; l < kSmallM; ++l) sum[l] = 0.0;
-  for (int k = 0; k < kSmallK; ++k) {
-    if (!((sel >> k) & 1)) continue;
-    double as[kSmallM];
-#pragma unroll
-    for (int l = 0; l < kSmallM; ++l) as[l] = 0.0;
-    for (int s = 0; s < kSmallN; ++s) {
-      const double d = st[nb[(NS + k * kSmallN + s) * kTile] & kHaloPosMask] - u0;
-      const double* As = A + (int64_t)(M * NS + (k * kSmallN + s) * kSmallM) * kTile;
-#pragma unroll
-      for (int l = 0; l < kSmallM; ++l) as[l] = fma(__ldg(As + l * kTile), d, as[l]);
-    }
-#pragma unroll
-    for (int l = 0; l < kSmallM; ++l) sum[l] += as[l];
-  }
-  const int nd = (sel & 1) + ((sel >> 1) & 1) + ((sel >> 2) & 1);
-  double cf[kSmallM];
-#pragma unroll
-  for (int l = 0; l < kSmallM; ++l) cf[l] = nd ? sum[l] / (double)nd : 0.0;
+template <int NS, int NQ3, int NV>
+__device__ __noinline__ void w_direct(const int2* W, int lane, int kc, const int32_t* nb,
+                                      const double* st, double u0, double* out) {
+#pragma unroll 1
   for (int p = 0; p < NQ3; ++p) {
-    double sp = 0.0;
-#pragma unroll
-    for (int l = 0; l < kSmallM; ++l) sp = fma(__ldg(psi + p * kMaxM + l), cf[l], sp);
-    out[p * NV] = u0 + sp;
+    double acc = 0.0;
+#pragma unroll 1
+    for (int s = 0; s < NS; ++s) {
+      const int2 w = W[wform_w_index(NS, NQ3, s, p, lane)];
+      const double x = ldexp((double)w.x * 1073741824.0 + (double)w.y, -kc);
+      acc = fma(x, st[nb[s * kTile]] - u0, acc);
+    }
+    out[p * NV] = u0 + acc;
   }
 }
 
-// kN = false: the FP64 path in pairs (halo, W and Gauss values as (hi, lo)
-// FP32 pairs); kN = true: the native FP64 path (FP64 halo, W and values, the
-// multiply-adds on the FP64 pipe).  The FP32 cutoff screen is the same.
-template <int M, int NS, int NQ, bool kN>
-__global__ void __launch_bounds__(kTile * (kConsumers + 1), (WPlan<M, NS, 3 * NQ, 3, 4>::kBlocks))
-    recon_tma_w_kernel(const ReconArgs a, const HaloArgs h, const void* __restrict__ psi_v,
-                       const float* __restrict__ g32, const void* __restrict__ wq, int* err) {
-  // 8-byte elements either way: halo states, W entries, Gauss-point values
-  using HT = typename std::conditional<kN, double, float2>::type;
-  using Acc = typename std::conditional<kN, double, DF>::type;
-  constexpr int NQ3 = 3 * NQ;
-  using P = WPlan<M, NS, NQ3, 3, 4>;
-  constexpr int kR = P::kRingW;
-  constexpr int NV = 4;
-  constexpr int SL = NS + kSmallSlots;
-  constexpr int E = M * NS + kSmallEntries;
-  constexpr int kPer = NQ3 * NV;  // Gauss-point pairs per cell
+// position in a ring of kN buffers: the buffer, and the parity of its phase
+template <int kN>
+struct RingPos {
+  int b = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next() {
+    if (++b == kN) b = 0, ph ^= 1;
+  }
+};
+
+// The cutoff screen's decisions from the FP32 indicators t known within the
+// factor f of chi: the selection, | 256 where C_T lies within that factor of
+// some chi.  Out of line: few cells need it.
+__device__ __noinline__ int w_screen(float t0, float t1, float t2, float tK, int present, float ct,
+                                     float f) {
+  const float t[kSmallK + 1] = {t0, t1, t2, tK};
+  bool near = false;
+  int sel = 8;
+  if (!chi_keep32_bound(t, kSmallK, present | 8, ct, f, &near)) {
+    sel = 0;
+#pragma unroll
+    for (int k = 0; k < kSmallK; ++k)
+      if (((present >> k) & 1) && chi_keep32_bound(t, k, present & 7, ct, f, &near)) sel |= 1 << k;
+  }
+  return sel | (near ? 256 : 0);
+}
+
+// deferred cells: the cell in the low word; the high word's flags, and the
+// selection where it is decided
+constexpr int kDefNear = 1, kDefDirect = 2, kDefSel = 8;  // selection from bit 3
+constexpr int kDefVar = 256;                              // variable from bit 8
+
+// the values of two variables of a point, 16 bytes
+__device__ __forceinline__ void st_two(float2* p, float2 x, float2 y) {
+  *reinterpret_cast<float4*>(p) = make_float4(x.x, x.y, y.x, y.y);
+}
+__device__ __forceinline__ void st_two(double* p, double x, double y) {
+  *reinterpret_cast<double2*>(p) = make_double2(x, y);
+}
+
+struct WArgs {
+  const void* psi;    // Psi' as pairs or FP64
+  const float* g32;   // FP32 rows of the complement and the directional stencils
+  const int2* w;      // W in fixed point
+  const uint16_t* pos;  // [tile][slot][32] byte offsets of the stencil cells in a halo row
+  const int32_t* tile;  // [tile][kWTile] halo cells, lanes that hold a cell, halo ids
+  const int32_t* st;  // [tile][kWStat][32]: column-sum norms of the four stencils (FP32), then
+                      // the exponent of W's unit (low half) and the stencil mask (bit 16)
+  WTable t;
+};
+
+// Works off n <= 32 deferred cells: the undecided ones one by one, then one
+// per lane.
+template <int M, int NS, int NQ, typename HT>
+__device__ __noinline__ void w_deferred(const ReconArgs& a, const WArgs& wa, const int2* list,
+                                        int n, HT* dsc) {
+  constexpr int NQ3 = 3 * NQ, NV = 4, E = M * NS + kSmallEntries, SL = NS + kSmallSlots;
+  const int lane = threadIdx.x & 31;
+  const int2 mine = lane < n ? list[lane] : make_int2(0, 0);
+  auto states = [&](int v) {
+    if constexpr (std::is_same<HT, double>::value)
+      return a.U + (int64_t)v * a.n_pad;
+    else
+      return a.Us + (int64_t)v * a.n_pad;
+  };
+  auto matrices = [&](int64_t c) {
+    return reinterpret_cast<const HT*>(a.ahat) + c / kTile * (int64_t)E * kTile + c % kTile;
+  };
+  auto cells = [&](int64_t c) { return a.nbr + c / kTile * (int64_t)SL * kTile + c % kTile; };
+  int sel = (mine.y >> 3) & 15;
+  unsigned near = __ballot_sync(0xffffffffu, lane < n && (mine.y & kDefNear));
+  for (; near; near &= near - 1) {
+    const int src = __ffs(near) - 1;
+    const int64_t c = __shfl_sync(0xffffffffu, mine.x, src);
+    const HT* st = states(__shfl_sync(0xffffffffu, mine.y / kDefVar, src));
+    const int r = w_select<M, NS, HT>(matrices(c), cells(c), st, st[c], a.smask[c], a.ct, a.eps, dsc);
+    if (lane == src) sel = r;
+  }
+  if (lane >= n) return;
+  const int64_t c = mine.x;
+  const int v = mine.y / kDefVar;
+  const HT* st = states(v);
+  if ((mine.y & kDefNear) && a.sel_out) a.sel_out[(int64_t)v * a.n_pad + c] = (uint8_t)sel;
+  HT* out = reinterpret_cast<HT*>(a.Uq) + c * (NQ3 * NV) + v;
+  if (!(sel & 8)) {
+    w_small<M, NS, NQ3, NV, HT>(matrices(c), cells(c), st, st[c], sel,
+                                reinterpret_cast<const HT*>(wa.psi), out);
+  } else if (mine.y & kDefDirect) {
+    const int64_t tile = c / kTile;
+    const int cl = (int)(c % kTile);
+    const int kc = (int16_t)(wa.st[(tile * kWStat + kWStat - 1) * kTile + cl] & 0xffff);
+    w_direct<NS, NQ3, NV>(wa.w + tile * (int64_t)(NS * NQ3) * kTile, cl, kc, cells(c), st, st[c],
+                          out);
+  }
+}
+
+// HT = float2: the FP64 path in pairs (Gauss values as (hi, lo) FP32 pairs);
+// HT = double: the native FP64 path.  Persistent blocks of consumer warps
+// (kVW variables each) and a producer lane that streams the tiles' matrices in
+// ring stages, and their halo ids, with bulk copies; each consumer warp
+// gathers its variables' halo states of the next tile with cp.async.  Every
+// hand-over is an mbarrier with bounded waits and no warp reads what another
+// consumer wrote, so the consumer warps run without block barriers.
+template <int M, int NS, int NQ, typename HT>
+__global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
+    recon_tma_w_kernel(const ReconArgs a, const WArgs wa, int* err) {
+  constexpr bool kN = std::is_same<HT, double>::value;
+  constexpr int NQ3 = 3 * NQ, NV = 4;
+  using P = WPlan<M, NS, NQ3, HT>;
+  using Dot = WDot<HT>;
+  constexpr int kVW = P::kVW, kWWarps = P::kWWarps;
+  constexpr int kR = P::kRingW, MC = P::kMC, R = M < NQ3 ? M : NQ3;
+  constexpr int kPer = NQ3 * NV;  // Gauss-point values per cell
   extern __shared__ __align__(128) unsigned char smem[];
-  HT* halo = reinterpret_cast<HT*>(smem + (size_t)kR * P::kMat);  // [2][NV][kHaloMax]
-  HT* ostg = reinterpret_cast<HT*>(smem + P::kOutOff);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)kR * P::kMat + P::kHaloBytes);
+  double* halo = reinterpret_cast<double*>(smem + (size_t)kR * P::kBuf);  // [2][NV][kHaloRow]
+  int32_t* tblk = reinterpret_cast<int32_t*>(halo + 2 * NV * P::kHaloRow);  // [2][kWTile]
+  int2* list = reinterpret_cast<int2*>(tblk + 2 * kWTile);  // [kWWarps][kListN]
+  HT* scratch = reinterpret_cast<HT*>(list + kWWarps * P::kListN);  // [kWWarps][kSL]
+  uint64_t* full = reinterpret_cast<uint64_t*>(scratch + kWWarps * P::kSL);
   uint64_t* empty = full + kR;
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + kR);
+  uint64_t* tfull = empty + kR;
+  uint64_t* tempty = tfull + 2;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(full + 16);
+  static_assert(2 * kR + 4 <= 16, "mbarriers");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_tiles = (a.n_cell + kTile - 1) / kTile;
   if (threadIdx.x == 0) {
     *abort_flag = 0;
     for (int i = 0; i < kR; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], kConsumers);
+      mbar_init(&empty[i], kWWarps);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], kWWarps);
     }
     mbar_fence_init();
   }
   __syncthreads();
-  if (warp == kConsumers) {
-    // ---- producer lane: FP32 and W blocks of every tile
+  if (warp == kWWarps) {
+    // ---- producer lane: the halo ids two tiles ahead, the ring stages of
+    // every tile
     if (lane == 0) {
-      int64_t g = 0;
-      for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const unsigned char* sg =
-            reinterpret_cast<const unsigned char*>(g32) + tile * (int64_t)P::kE32 * kTile * 4;
-        const unsigned char* sw =
-            reinterpret_cast<const unsigned char*>(wq) + tile * (int64_t)P::kEW * kTile * 8;
-        const unsigned char* sn =
-            reinterpret_cast<const unsigned char*>(h.nbr_loc) + tile * (int64_t)P::kSL * P::kSlotN;
-        for (int j = 0; j < P::kStages; ++j, ++g) {
-          const int b = (int)(g % kR);
-          if (g >= kR) {
-            const int w = mbar_wait_or_abort(&empty[b], (uint32_t)((g / kR) - 1) & 1, abort_flag);
-            if (w != 1) {
-              if (w == 0) {
-                atomicOr(err, 2);
-                *abort_flag = 1;
-              }
-              for (int64_t i = g - kR; i < g; ++i) mbar_wait(&full[i % kR], (uint32_t)(i / kR) & 1);
-              return;
-            }
-          }
-          int slot0, nslot, k, og, bg, ow, bw;
-          P::stage(j, slot0, nslot, k, og, bg, ow, bw);
-          unsigned char* dst = smem + (size_t)b * P::kMat;
-          const uint32_t bn = (uint32_t)(nslot * P::kSlotN);
-          mbar_expect_tx(&full[b], (uint32_t)(bg + bw) + bn);
-          bulk_g2s(dst, sg + og, (uint32_t)bg, &full[b]);
-          if (bw) bulk_g2s(dst + P::kWOff, sw + ow, (uint32_t)bw, &full[b]);
-          bulk_g2s(dst + P::kNOff, sn + slot0 * P::kSlotN, bn, &full[b]);
-        }
-      }
-      // the block must not exit while a copy it issued is in flight
-      for (int64_t i = g > kR ? g - kR : 0; i < g; ++i)
-        mbar_wait(&full[i % kR], (uint32_t)(i / kR) & 1);
-    }
-    return;
-  }
-  // ---- consumers (the halo pipeline of recon_tma_kernel measured slower
-  // here: this kernel is at its register limit)
-  const int v = warp, tid = threadIdx.x;
-  auto prefetch = [&](int64_t tile, int hb) {
-    const int h0 = h.off[tile], H = h.off[tile + 1] - h0;
-    for (int i = tid; i < H; i += kConsumers * kTile) {
-      const int id = __ldg(h.ids + h0 + i);
-#pragma unroll
-      for (int w = 0; w < NV; ++w) {
-        const void* src;
-        if constexpr (kN)
-          src = a.U + (int64_t)w * a.n_pad + id;
-        else
-          src = a.Us + (int64_t)w * a.n_pad + id;
-        cp_async8(&halo[(hb * NV + w) * kHaloMax + i], src);
-      }
-    }
-    cp_async_commit();
-  };
-  int64_t g = 0;
-  int hb = 0;
-  bool dead = false;  // a bounded wait of this block gave up: skip all work
-  if ((int64_t)blockIdx.x < n_tiles) prefetch(blockIdx.x, 0);
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, hb ^= 1) {
-    consumer_sync();  // every consumer is done with the other halo buffer
-    const int64_t nxt = tile + gridDim.x;
-    if (nxt < n_tiles)
-      prefetch(nxt, hb ^ 1);
-    else
-      cp_async_commit();
-    cp_async_wait<1>();
-    consumer_sync();
-    const HT* st = halo + (hb * NV + v) * kHaloMax;
-    const uint16_t* nb = h.nbr_loc + tile * (int64_t)SL * kTile + lane;
-    const int64_t c = tile * kTile + lane;  // may be a pad lane of the last tile
-    HT u0s;
-    if constexpr (kN)
-      u0s = a.U[(int64_t)v * a.n_pad + (c < a.n_cell ? c : 0)];
-    else
-      u0s = a.Us[(int64_t)v * a.n_pad + (c < a.n_cell ? c : 0)];
-    auto dif = [&](int idx) -> Acc {  // d_s = U_s - U_0 (pairs, or FP64)
-      if constexpr (kN) {
-        return st[idx] - u0s;
-      } else {
-        const float2 q = st[idx];
-        DF t = two_sum(q.x, -u0s.x);
-        t.l += q.y - u0s.y;
-        return two_sum(t.h, t.l);
-      }
-    };
-    float a32[M], s32[kSmallK][kSmallM], eL = 0.f, eS[kSmallK];
-    Acc uq[NQ3];
-#pragma unroll
-    for (int l = 0; l < M; ++l) a32[l] = 0.f;
-#pragma unroll
-    for (int k = 0; k < kSmallK; ++k) {
-      eS[k] = 0.f;
-#pragma unroll
-      for (int l = 0; l < kSmallM; ++l) s32[k][l] = 0.f;
-    }
-#pragma unroll
-    for (int p = 0; p < NQ3; ++p) uq[p] = Acc{};
-    // selection and Gauss-point values of cell c (after all stages of its tile)
-    auto finish_cell = [&](int64_t tile, int64_t c) {
-      const int present = a.smask[c];
-      const HT* A = reinterpret_cast<const HT*>(a.ahat) + tile * (int64_t)E * kTile + lane;
-      uint8_t sel;
-      if (a.sel_in) {
-        sel = a.sel_in[(int64_t)v * a.n_pad + c];
-      } else if (a.linear) {
-        sel = 8;
-      } else {
-        float t[kSmallK + 1];
-        float rho = 0.f;
-        {
-          float bsum = 0.f;
-#pragma unroll
-          for (int l = 0; l < M; ++l) bsum = fmaf(a32[l], a32[l], bsum);
-          t[kSmallK] = bsum + (float)a.eps;
-          rho = beta_rel_bound(bsum, eL, NS, M, (float)a.eps);
-#pragma unroll
-          for (int k = 0; k < kSmallK; ++k) {
-            float q = 0.f;
-#pragma unroll
-            for (int l = 0; l < kSmallM; ++l) q = fmaf(s32[k][l], s32[k][l], q);
-            t[k] = q + (float)a.eps;
-            if ((present >> k) & 1)
-              rho = fmaxf(rho, beta_rel_bound(q, eS[k], kSmallN, kSmallM, (float)a.eps));
-          }
-        }
-        // chi lies within the factor f of its FP32 value under the beta bounds
-        bool near = a.force_near || !(rho < 0.25f);
-        const float q = (1.f + rho) / (1.f - fminf(rho, 0.5f));
-        const float q2 = q * q;
-        const float f = q2 * q2 * q2 * 1.0001f;
-        const float ct = (float)a.ct;
-        if (chi_keep32_bound(t, kSmallK, present | 8, ct, f, &near)) {
-          sel = 8;
-        } else {
-          sel = 0;
-#pragma unroll
-          for (int k = 0; k < kSmallK; ++k)
-            if (((present >> k) & 1) && chi_keep32_bound(t, k, present & 7, ct, f, &near))
-              sel |= (uint8_t)(1u << k);
-        }
-        if (near) {
-          if constexpr (kN)
-            sel = w_select_native<M, NS>(A, nb, st, u0s, present, a.ct, a.eps);
-          else
-            sel = w_select_pairs<M, NS>(A, nb, st, u0s, present, a.ct, a.eps);
-        }
-      }
-      if (a.sel_out) a.sel_out[(int64_t)v * a.n_pad + c] = sel;
-      // Gauss-point values ((hi, lo) pairs or FP64), to the output stage or to Uq
-      HT* __restrict__ out = TENO_STAGE_OUT_W ? ostg + lane * (kPer + 1) + v
-                                              : reinterpret_cast<HT*>(a.Uq) + c * kPer + v;
-      if (sel & 8) {
-        if constexpr (kN) {
-#pragma unroll
-          for (int p = 0; p < NQ3; ++p) out[p * NV] = u0s + uq[p];
-        } else {
-          const DF u0 = {u0s.x, u0s.y};
-#pragma unroll
-          for (int p = 0; p < NQ3; ++p) {
-            const DF r = u0 + df_norm(uq[p]);
-            out[p * NV] = make_float2(r.h, r.l);
-          }
-        }
-      } else {
-        if constexpr (kN)
-          w_small_native<M, NS, NQ3, NV>(A, nb, st, u0s, sel,
-                                         reinterpret_cast<const double*>(psi_v), out);
-        else
-          w_small_values<M, NS, NQ3, NV>(A, nb, st, u0s, sel,
-                                         reinterpret_cast<const float2*>(psi_v), out);
-      }
-    };
-    for (int j = 0; j < P::kStages; ++j, ++g) {
-      const int b = (int)(g % kR);
-      int slot0, nslot, k, og, bg, ow, bw;
-      P::stage(j, slot0, nslot, k, og, bg, ow, bw);
-      if (!dead) {
-        const int w = mbar_wait_or_abort(&full[b], (uint32_t)(g / kR) & 1, abort_flag, a.wait_polls);
+      RingPos<kR> rp;
+      bool lap = false;  // every buffer has been filled once
+      int it = 0;
+      // the block must not exit while a copy it issued is in flight: the last
+      // kR stages (buffers before rp.b are one phase ahead) and id blocks
+      auto drain = [&](int n_blk) {
+        for (int b = 0; b < kR; ++b)
+          if (b < rp.b || lap) mbar_wait(&full[b], b < rp.b ? rp.ph : rp.ph ^ 1);
+        for (int i = n_blk > 2 ? n_blk - 2 : 0; i < n_blk; ++i)
+          mbar_wait(&tfull[i & 1], (uint32_t)(i >> 1) & 1);
+      };
+      auto gave_up = [&](int w, int n_blk) {
         if (w == 0) {
           atomicOr(err, 2);
           *abort_flag = 1;
         }
-        dead = __any_sync(0xffffffffu, w != 1);
+        drain(n_blk);
+      };
+      auto block = [&](int64_t tile, int i) {
+        if (tile >= n_tiles) return;
+        mbar_expect_tx(&tfull[i & 1], P::kTileBytes);
+        bulk_g2s(tblk + (i & 1) * kWTile, wa.tile + tile * kWTile, P::kTileBytes, &tfull[i & 1]);
+      };
+      int n_blk = 0;  // halo-id blocks issued
+      for (; n_blk < 2 && blockIdx.x + (int64_t)n_blk * gridDim.x < n_tiles; ++n_blk)
+        block(blockIdx.x + (int64_t)n_blk * gridDim.x, n_blk);
+      for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+        const unsigned char* sg =
+            reinterpret_cast<const unsigned char*>(wa.g32) + tile * (int64_t)P::kE32 * kTile * 4;
+        const unsigned char* sw =
+            reinterpret_cast<const unsigned char*>(wa.w) + tile * (int64_t)P::kEW * kTile * 8;
+        const unsigned char* sn =
+            reinterpret_cast<const unsigned char*>(wa.pos) + tile * (int64_t)P::kSL * P::kSlotN;
+        for (int j = 0; j < P::kStages; ++j) {
+          const int b = rp.b;
+          if (lap) {
+            const int w = mbar_wait_or_abort(&empty[b], rp.ph ^ 1, abort_flag);
+            if (w != 1) return gave_up(w, n_blk);
+          }
+          unsigned char* dst = smem + b * P::kBuf;
+          if (j < kSmallK) {
+            mbar_expect_tx(&full[b], P::kSB + kSmallN * P::kSlotN);
+            bulk_g2s(dst, sg + P::kNL * P::kGB + j * P::kSB, P::kSB, &full[b]);
+            bulk_g2s(dst + P::kSB, sn + (NS + j * kSmallN) * P::kSlotN, kSmallN * P::kSlotN,
+                     &full[b]);
+          } else {
+            const int i = j - kSmallK;
+            const bool last = j == P::kStages - 1;
+            mbar_expect_tx(&full[b], P::kGB + P::kWB + P::kLPS * P::kSlotN +
+                                         (last ? P::kStatBytes : 0));
+            if constexpr (MC > 0) bulk_g2s(dst, sg + i * P::kGB, P::kGB, &full[b]);
+            bulk_g2s(dst + P::kWOff, sw + i * P::kWB, P::kWB, &full[b]);
+            bulk_g2s(dst + P::kNOff, sn + i * P::kLPS * P::kSlotN, P::kLPS * P::kSlotN, &full[b]);
+            if (last) bulk_g2s(dst + P::kXOff, wa.st + tile * kWStat * kTile, P::kStatBytes, &full[b]);
+          }
+          rp.next();
+          lap |= rp.b == 0;
+        }
+        const int64_t nxt = tile + 2 * (int64_t)gridDim.x;
+        if (nxt < n_tiles) {
+          const int w =
+              mbar_wait_or_abort(&tempty[it & 1], (uint32_t)(it >> 1) & 1, abort_flag);
+          if (w != 1) return gave_up(w, n_blk);
+          block(nxt, n_blk++);
+        }
       }
-      const unsigned char* buf = smem + (size_t)b * P::kMat;
-      const uint16_t* nl = reinterpret_cast<const uint16_t*>(buf + P::kNOff) + lane;
-      if (dead) {
-        // skip the stage
-      } else if (k < 0) {
-        const float* gm = reinterpret_cast<const float*>(buf) + lane;
-        const HT* wm = reinterpret_cast<const HT*>(buf + P::kWOff) + lane;
+      drain(n_blk);
+    }
+    return;
+  }
+  // ---- consumers (warp w: kVW variables from kVW w)
+  constexpr int kPerLane = kHaloMax / kTile;
+  const int v0 = warp * kVW;
+  int2* mylist = list + warp * P::kListN;
+  HT* dsc = scratch + warp * P::kSL;
+  int n_def = 0, it = 0;
+  RingPos<kR> rp;
+  // the wait of one consumer warp; false: some wait of the block gave up
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    const int w = mbar_wait_or_abort(bar, parity, abort_flag, a.wait_polls);
+    if (w == 0) {
+      atomicOr(err, 2);
+      *abort_flag = 1;
+    }
+    return !__any_sync(0xffffffffu, w != 1);
+  };
+  // the halo and own states of this block's i-th tile, one commit group (an
+  // empty one past the end); H and held: its halo cells, the lanes that hold
+  // a cell (a partition's layout has gaps)
+  auto gather = [&](int64_t tile, int i, int& H, unsigned& held) {
+    bool ok = true;
+    if (tile < n_tiles) {
+      ok = wait(&tfull[i & 1], (uint32_t)(i >> 1) & 1);
+      if (ok) {
+        const int32_t* tb = tblk + (i & 1) * kWTile;
+        const double* src = a.U + (int64_t)v0 * a.n_pad;
+        double* dst = halo + ((i & 1) * NV + v0) * P::kHaloRow;
+        H = tb[0];
+        held = (unsigned)tb[1];
 #pragma unroll
-        for (int s = 0; s < 3; ++s) {
-          if (s < nslot) {
-            const Acc d = dif(nl[s * kTile] & kHaloPosMask);
-            float dh;
-            if constexpr (kN)
-              dh = d2f_trunc(d);
-            else
-              dh = d.h;
+        for (int k = 0; k < kPerLane; ++k)
+          if (lane + k * kTile < H) {
+            const int id = tb[4 + lane + k * kTile];
 #pragma unroll
-            for (int l = 0; l < M; ++l) a32[l] = fmaf(gm[(s * P::kG + l) * kTile], dh, a32[l]);
-            eL = fmaf(gm[(s * P::kG + M) * kTile], fabsf(dh), eL);
+            for (int w = 0; w < kVW; ++w)
+              cp_async8(dst + w * P::kHaloRow + lane + k * kTile, src + w * a.n_pad + id);
+          }
+        const int64_t c = tile * kTile + lane;
 #pragma unroll
-            for (int p = 0; p < NQ3; ++p) {
-              if constexpr (kN)
-                uq[p] = fma(wm[(s * NQ3 + p) * kTile], d, uq[p]);
-              else
-                df_mac(uq[p], wm[(s * NQ3 + p) * kTile], d);
-            }
+        for (int w = 0; w < kVW; ++w)
+          cp_async8(dst + w * P::kHaloRow + kHaloMax + lane,
+                    src + w * a.n_pad + (c < a.n_cell ? c : 0));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[i & 1]);
+      }
+    }
+    cp_async_commit();
+    return ok;
+  };
+  int H, Hn = 0;
+  unsigned held, heldn = 0u;
+  if (!gather(blockIdx.x, 0, Hn, heldn)) {
+    cp_async_wait<0>();
+    return;
+  }
+  bool alive = true;
+  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+    const int64_t c = tile * kTile + lane;  // may be a pad lane of the last tile
+    H = Hn;
+    held = heldn;
+    __syncwarp();  // every lane is done with the other halo buffer
+    if (!(alive = gather(tile + gridDim.x, it + 1, Hn, heldn))) break;
+    cp_async_wait<1>();
+    __syncwarp();
+    double* hv = halo + ((it & 1) * NV + v0) * P::kHaloRow;
+    const bool mine = (held >> lane) & 1;
+    // ---- the halo states relative to the tile's first cell in fixed point,
+    // in place (Dot::kBits of the largest difference).  The unit depends on
+    // the set of the tile's cells and halo only, so a partition, which keeps
+    // whole tiles, gets the same bits
+    int64_t y0[kVW];
+    int sc[kVW];       // the units are 2^-sc
+    bool direct[kVW];  // the tile's states of this variable have no such unit
+    {
+      const int n_mine = (H - lane + kTile - 1) / kTile;  // this lane's halo cells
+      unsigned mx[kVW];
+      double ref[kVW];
+#pragma unroll
+      for (int w = 0; w < kVW; ++w) {
+        const double u0 = hv[w * P::kHaloRow + kHaloMax + lane];
+        ref[w] = __shfl_sync(0xffffffffu, u0, 0);
+        mx[w] = mine ? mag_bits(u0 - ref[w]) : 0u;
+      }
+#pragma unroll 2
+      for (int i = 0; i < n_mine; ++i)
+#pragma unroll
+        for (int w = 0; w < kVW; ++w)
+          mx[w] = max(mx[w], mag_bits(hv[w * P::kHaloRow + lane + i * kTile] - ref[w]));
+      double cf[kVW];
+#pragma unroll
+      for (int w = 0; w < kVW; ++w) {
+        mx[w] = __reduce_max_sync(0xffffffffu, mx[w]);
+        // |U - U_ref| < 2^(e + 1); a difference below 2^-900 counts as none
+        const int e = max(mx[w] ? mag_exp<double>(mx[w]) : 0, -900);
+        direct[w] = e > 100;
+        sc[w] = direct[w] ? 0 : Dot::kBits - 1 - e;
+        cf[w] = __hiloint2double((sc[w] + 1023) << 20, 0);
+        const double u0 = hv[w * P::kHaloRow + kHaloMax + lane];
+        y0[w] = mine && !direct[w] ? Dot::fix(u0 - ref[w], sc[w], cf[w]) : 0;
+      }
+#pragma unroll 2
+      for (int i = 0; i < n_mine; ++i)
+#pragma unroll
+        for (int w = 0; w < kVW; ++w) {
+          double* q = hv + w * P::kHaloRow + lane + i * kTile;
+          *q = __longlong_as_double(direct[w] ? 0 : Dot::fix(*q - ref[w], sc[w], cf[w]));
+        }
+      __syncwarp();
+    }
+    float cd[kVW], cu[kVW];  // FP32 scale of a difference, and one unit
+#pragma unroll
+    for (int w = 0; w < kVW; ++w) cd[w] = Dot::c(sc[w]), cu[w] = 80.f * exp2i(-sc[w]);
+    // difference parts of the cell at a byte offset of the halo row, and the
+    // difference in FP32 (error 3u relative plus 2^6 units).  The 64-bit
+    // conversion would take the FP64 pipe.
+    const unsigned char* st = reinterpret_cast<const unsigned char*>(hv);
+    auto dif = [&](int w, int off, typename Dot::D& d) {
+      return Dot::split(*reinterpret_cast<const int64_t*>(st + w * (P::kHaloRow * 8) + off) - y0[w],
+                        cd[w], d);
+    };
+    // ---- directional stencils: FP32 smoothness indicators
+    float ts[kVW][kSmallK], ds[kVW][kSmallK];
+#pragma unroll
+    for (int w = 0; w < kVW; ++w)
+#pragma unroll
+      for (int k = 0; k < kSmallK; ++k) ts[w][k] = ds[w][k] = 0.f;
+#pragma unroll 1
+    for (int k = 0; k < kSmallK; ++k, rp.next()) {
+      if (!(alive = wait(&full[rp.b], rp.ph))) break;
+      const unsigned char* buf = smem + rp.b * P::kBuf;
+      const uint16_t* nl = reinterpret_cast<const uint16_t*>(buf + P::kSB) + lane;
+      float s[kVW][kSmallM], dd[kVW];
+#pragma unroll
+      for (int w = 0; w < kVW; ++w) {
+        dd[w] = 0.f;
+#pragma unroll
+        for (int l = 0; l < kSmallM; ++l) s[w][l] = 0.f;
+      }
+      // four slots (five fours of rows) at a time
+#pragma unroll 1
+      for (int i = 0; i < kSmallN; i += 4) {
+        float f[kVW][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int off = nl[(i + j) * kTile];
+#pragma unroll
+          for (int w = 0; w < kVW; ++w) {
+            typename Dot::D d;
+            f[w][j] = dif(w, off, d);
+            dd[w] = fmaf(f[w][j], f[w][j], dd[w]);
           }
         }
-      } else {
-        const float* gm = reinterpret_cast<const float*>(buf) + lane;
 #pragma unroll
-        for (int kk = 0; kk < kSmallK; ++kk) {
-          if (kk != k) continue;
+        for (int e = 0; e < 4 * kSmallM; ++e) {
+          const float m = g_entry<4 * kSmallM>(buf + i * kSmallM * kTile * 4, lane, e);
 #pragma unroll
-          for (int s = 0; s < 4; ++s) {
-            const HT q = st[nl[s * kTile] & kHaloPosMask];
-            float dh;
-            if constexpr (kN)
-              dh = d2f_trunc(q - u0s);
-            else
-              dh = (q.x - u0s.x) + (q.y - u0s.y);
-#pragma unroll
-            for (int l = 0; l < kSmallM; ++l)
-              s32[kk][l] = fmaf(gm[(s * P::kGs + l) * kTile], dh, s32[kk][l]);
-            eS[kk] = fmaf(gm[(s * P::kGs + kSmallM) * kTile], fabsf(dh), eS[kk]);
-          }
+          for (int w = 0; w < kVW; ++w)
+            s[w][e % kSmallM] = fmaf(m, f[w][e / kSmallM], s[w][e % kSmallM]);
         }
       }
       __syncwarp();
-      if (lane == 0 && !dead) mbar_arrive(&empty[b]);
+      if (lane == 0) mbar_arrive(&empty[rp.b]);
+#pragma unroll
+      for (int w = 0; w < kVW; ++w) {
+        float q = 0.f;
+#pragma unroll
+        for (int l = 0; l < kSmallM; ++l) q = fmaf(s[w][l], s[w][l], q);
+#pragma unroll
+        for (int i = 0; i < kSmallK; ++i)
+          if (i == k) ts[w][i] = q, ds[w][i] = dd[w];
+      }
     }
-    if (!dead && c < a.n_cell) finish_cell(tile, c);
-    if constexpr (TENO_STAGE_OUT_W != 0) {
-      consumer_sync();  // the tile's values are staged
-      if (!dead)
-        store_out_stage<kPer>(ostg, reinterpret_cast<HT*>(a.Uq) + tile * kTile * kPer,
-                              (int)min((int64_t)kTile, a.n_cell - tile * kTile), tid);
+    if (!alive) break;
+    // ---- large stencil: W d in fixed point, complement rows in FP32
+    typename Dot::A acc[kVW][NQ3];
+    float a32[kVW][MC > 0 ? MC : 1], dL[kVW], norm[kSmallK + 1];
+    int stat = 0;
+#pragma unroll
+    for (int w = 0; w < kVW; ++w) {
+      dL[w] = 0.f;
+#pragma unroll
+      for (int l = 0; l < MC; ++l) a32[w][l] = 0.f;
+    }
+#pragma unroll 1
+    for (int j = 0; j < P::kNL; ++j, rp.next()) {
+      if (!(alive = wait(&full[rp.b], rp.ph))) break;
+      const unsigned char* buf = smem + rp.b * P::kBuf;
+      const uint16_t* nl = reinterpret_cast<const uint16_t*>(buf + P::kNOff) + lane;
+      typename Dot::D d[kVW][P::kLPS];
+      float f[kVW][P::kLPS];
+#pragma unroll
+      for (int s = 0; s < P::kLPS; ++s) {
+        const int off = nl[s * kTile];
+#pragma unroll
+        for (int w = 0; w < kVW; ++w) {
+          f[w][s] = dif(w, off, d[w][s]);
+          dL[w] = fmaf(f[w][s], f[w][s], dL[w]);
+        }
+      }
+      if constexpr (MC > 0) {
+#pragma unroll
+        for (int e = 0; e < P::kNG; ++e) {
+          const float m = g_entry<P::kNG>(buf, lane, e);
+#pragma unroll
+          for (int w = 0; w < kVW; ++w) a32[w][e % MC] = fmaf(m, f[w][e / MC], a32[w][e % MC]);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < P::kNW; ++e) {
+        const typename Dot::W m = Dot::entry(w_entry<P::kNW>(buf + P::kWOff, lane, e));
+#pragma unroll
+        for (int w = 0; w < kVW; ++w) Dot::mac(acc[w][e % NQ3], m, d[w][e / NQ3]);
+      }
+      if (j == P::kNL - 1) {
+        const int32_t* xs = reinterpret_cast<const int32_t*>(buf + P::kXOff) + lane;
+#pragma unroll
+        for (int k = 0; k <= kSmallK; ++k) norm[k] = __int_as_float(xs[k * kTile]);
+        stat = xs[kSmallK * kTile + kTile];
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[rp.b]);
+    }
+    if (!alive) break;
+    // ---- selection
+    const int present = (stat >> 16) & 7, kc = (int)(int16_t)(stat & 0xffff);
+    int eT[kVW], sel[kVW];  // W d = (the sum) 2^eT
+    bool near[kVW];
+    HT val[kVW][NQ3];
+#pragma unroll
+    for (int w = 0; w < kVW; ++w) {
+      const int v = v0 + w;
+      eT[w] = Dot::exp(kc, sc[w]);
+      const float s0 = exp2i(eT[w]);
+      // Gauss-point values, and W d in FP32 (y)
+      float y[NQ3];
+      const double u0d = hv[w * P::kHaloRow + kHaloMax + lane];
+      if constexpr (kN) {
+        const double sT = __hiloint2double((eT[w] + 1023) << 20, 0);
+#pragma unroll
+        for (int p = 0; p < NQ3; ++p) {
+          const int64_t T = Dot::sum(acc[w][p]);
+          y[p] = fmaf((float)(int)(T >> 31), s0 * 2147483648.f, (float)(int)(T & 0x7fffffff) * s0);
+          val[w][p] = fma((double)T, sT, u0d);
+        }
+      } else {
+        const float s2 = exp2i(eT[w] + 42), s1 = exp2i(eT[w] + 21);
+        const DF u0 = d_to_df(u0d);  // the split the state kernels write
+#pragma unroll
+        for (int p = 0; p < NQ3; ++p) {
+          const DF x = Dot::value(acc[w][p], s2, s1, s0);
+          y[p] = x.h;
+          const DF r = u0 + x;
+          val[w][p] = make_float2(r.h, r.l);
+        }
+        if (eT[w] < -120) {  // units below the FP32 range (states near 1e-30): FP64
+          const double sT = ldexp(1.0, eT[w]);
+#pragma unroll
+          for (int p = 0; p < NQ3; ++p) {
+            const DF r = d_to_df(fma(Dot::value_d(acc[w][p]), sT, u0d));
+            val[w][p] = make_float2(r.h, r.l);
+          }
+        }
+      }
+      sel[w] = 8;
+      near[w] = false;
+      if (!mine) {
+        // no cell: large stencil, nothing to decide
+      } else if (a.sel_in) {
+        sel[w] = a.sel_in[(int64_t)v * a.n_pad + c];
+      } else if (!a.linear) {
+        const float eps = (float)a.eps;
+        float t[kSmallK + 1], rho = 0.f;
+        // the coefficients in the row space of Psi' are T y, y within 2u
+        // relative plus Dot::kErr units of the fixed-point sum
+        float bsum = 0.f, E = 0.f;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          float q = 0.f;
+#pragma unroll
+          for (int p = 0; p < (NQ3 <= M ? i + 1 : NQ3); ++p)
+            q = fmaf(wa.t.t[i * NQ3 + p], y[p], q);
+          bsum = fmaf(q, q, bsum);
+        }
+#pragma unroll
+        for (int p = 0; p < NQ3; ++p) E = fmaf(wa.t.cs[p], fabsf(y[p]), E);
+        const float l2 = sqrt_approx(dL[w]) * 1.0002f;
+        E = (NQ3 + 5) * 5.9604645e-8f * 1.0001f * E +
+            wa.t.cs_all * fmaf(Dot::kErr, s0, Dot::kErrD * l2 * exp2i(-kc));
+#pragma unroll
+        for (int l = 0; l < MC; ++l) bsum = fmaf(a32[w][l], a32[w][l], bsum);
+        if constexpr (MC > 0) E += dot_bound(norm[kSmallK], dL[w], cu[w], NS);
+        t[kSmallK] = bsum + eps;
+        rho = beta_rel_bound(bsum, E * 1.0001f, M, eps);
+#pragma unroll
+        for (int k = 0; k < kSmallK; ++k) {
+          t[k] = ts[w][k] + eps;
+          if ((present >> k) & 1)
+            rho = fmaxf(rho, beta_rel_bound(ts[w][k],
+                                            dot_bound(norm[k], ds[w][k], cu[w], kSmallN),
+                                            kSmallM, eps));
+        }
+        // chi lies within the factor f of its FP32 value under the beta bounds
+        // (an eps below the squares of flushed differences decides nothing here)
+        near[w] = a.force_near || direct[w] || !(rho < 0.25f) || (sc[w] > 120 && eps < 1e-30f);
+        const float q = (1.f + rho) * rcp_approx(1.f - fminf(rho, 0.5f));
+        const float q2 = q * q;
+        const float f = q2 * q2 * q2 * 1.0002f;
+        const float ct = (float)a.ct;
+        // most cells keep the large stencil by far: chi_K >= 1 / (1 + 3 r^6) with
+        // r the ratio to the smallest directional indicator (2 % for rounding)
+        float tm = t[kSmallK];
+#pragma unroll
+        for (int k = 0; k < kSmallK; ++k)
+          if ((present >> k) & 1) tm = fminf(tm, t[k]);
+        const float rr = t[kSmallK] * rcp_approx(tm), r2 = rr * rr;
+        if (!(fmaf(3.06f * r2, r2 * r2, 1.02f) * (ct * f) < 1.f)) {
+          const int x = w_screen(t[0], t[1], t[2], t[kSmallK], present, ct, f);
+          near[w] |= (x & 256) != 0;
+          sel[w] = x & 15;
+        }
+      }
+    }
+    // ---- Gauss-point values of the large polynomial, both variables of a
+    // point in one store where both keep it (or may)
+    bool put[kVW], both = c < a.n_cell;
+#pragma unroll
+    for (int w = 0; w < kVW; ++w) {
+      if (c < a.n_cell && a.sel_out && !near[w])
+        a.sel_out[(int64_t)(v0 + w) * a.n_pad + c] = (uint8_t)sel[w];
+      put[w] = c < a.n_cell && !direct[w] && (near[w] || (sel[w] & 8));
+      both &= put[w];
+    }
+    {
+      HT* __restrict__ out = reinterpret_cast<HT*>(a.Uq) + c * kPer + v0;
+      if (kVW == 2 && both) {
+#pragma unroll
+        for (int p = 0; p < NQ3; ++p) st_two(out + p * NV, val[0][p], val[kVW - 1][p]);
+      } else {
+#pragma unroll
+        for (int w = 0; w < kVW; ++w)
+          if (put[w])
+#pragma unroll
+            for (int p = 0; p < NQ3; ++p) out[p * NV + w] = val[w][p];
+      }
+    }
+    // ---- defer what the fixed-point values do not settle
+#pragma unroll
+    for (int w = 0; w < kVW; ++w) {
+      const bool def = mine && (near[w] || direct[w] || !(sel[w] & 8));
+      const unsigned bal = __ballot_sync(0xffffffffu, def);
+      if (def)
+        mylist[n_def + __popc(bal & ((1u << lane) - 1u))] =
+            make_int2((int)c, (near[w] ? kDefNear : 0) | (direct[w] ? kDefDirect : 0) |
+                                  sel[w] * kDefSel | (v0 + w) * kDefVar);
+      n_def += __popc(bal);
+    }
+    __syncwarp();
+    while (n_def >= kTile) {
+      n_def -= kTile;
+      w_deferred<M, NS, NQ, HT>(a, wa, mylist + n_def, kTile, dsc);
+      __syncwarp();
     }
   }
   cp_async_wait<0>();
+  if (alive && n_def) w_deferred<M, NS, NQ, HT>(a, wa, mylist, n_def, dsc);
 }
 
 // ------------------------------------ characteristic variables (charvar)
@@ -3498,10 +3978,6 @@ __global__ void __launch_bounds__(128) recon_vjp_kernel(const TS* __restrict__ a
 // Double-float version for the FP64 path (matrices stored as (hi, lo)
 // pairs): the transposed matvecs run on the FP32 pipe; d_bar is written as
 // pairs, u_self in FP64.
-__device__ __forceinline__ DF d_to_df(double x) {
-  const float h = (float)x;
-  return {h, (float)(x - (double)h)};
-}
 __device__ __forceinline__ DF df_div_small(DF a, int n) {  // a / n for n in 1..3
   const float fn = (float)n;
   const float qh = a.h / fn;
@@ -3593,20 +4069,23 @@ __global__ void __launch_bounds__(128) recon_vjp_df_kernel(const float2* __restr
 // cell instead of every stencil slot that holds it.  The tile's Uq_bar block is prefetched
 // with cp.async one tile ahead.
 constexpr int kRingV = 4;
+constexpr int kVjpNone = -(1 << 16);  // an exponent below every value's
 constexpr int kUbStride = 38;  // doubles per cell in the Uq_bar stage (16-byte rows)
 constexpr int kHaccStride = kHaloMax + 4;  // pairs per variable row (conflict-free transpose)
 
 template <int M, int NS, int NQ3>
 struct VjpPlan {
   static constexpr int kLPS = 4, kSPS = 4;
-  static constexpr int kSlotW = NQ3 * kTile * 8;      // W pairs of one large slot
+  static constexpr int kLay = wform_lps(NS);          // slots of a layout stage
+  static_assert(kLPS % kLay == 0, "whole layout stages");
+  static constexpr int kSlotW = NQ3 * kTile * 8;      // W of one large slot
   static constexpr int kSlotS = kSmallM * kTile * 8;  // matrix pairs of one directional slot
   static constexpr int kSlotN = kTile * 2;            // halo positions (uint16) of one slot
   static constexpr int kNL = (NS + kLPS - 1) / kLPS;
   static constexpr int kPerSmall = kSmallN / kSPS;
   static constexpr int kStages = kNL + kSmallK * kPerSmall;
   static constexpr int kNOff = kLPS * kSlotW > kSPS * kSlotS ? kLPS * kSlotW : kSPS * kSlotS;
-  static constexpr int kMat = kNOff + 4 * kSlotN;
+  static constexpr int kMat = kNOff + (kLPS > kSPS ? kLPS : kSPS) * kSlotN;
   static constexpr int kSL = NS + kSmallSlots;
   static constexpr int64_t kTileW = (int64_t)NS * NQ3 * kTile * 8;
   static constexpr int64_t kTileA = (int64_t)(M * NS + kSmallEntries) * kTile * 8;
@@ -3615,7 +4094,7 @@ struct VjpPlan {
   static constexpr size_t kHaccOff = kUbOff + kUbBytes;
   static constexpr size_t kHaccBytes = (size_t)4 * kHaccStride * 8;
   static constexpr size_t kBarOff = kHaccOff + kHaccBytes;
-  static constexpr size_t kSmem = kBarOff + 2 * kRingV * 8 + 16 + 16;
+  static constexpr size_t kSmem = kBarOff + 2 * kRingV * 8 + 16 + 32 + 4 * 8 * 4;
   static_assert(NQ3 * 4 <= kUbStride, "Uq_bar row");
   static_assert(kSmallN % kSPS == 0, "directional stencil split");
   static_assert(kMat % 16 == 0 && kUbOff % 16 == 0 && kHaccOff % 16 == 0 && kBarOff % 8 == 0,
@@ -3650,20 +4129,23 @@ __device__ __forceinline__ bool vjp_needs_small(uint8_t sel) {
 
 template <int M, int NS, int NQ>
 __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
-    recon_vjp_tma_kernel(const float2* __restrict__ ahat, const float2* __restrict__ wq,
-                         const HaloArgs h, const uint8_t* __restrict__ sel_in,
+    recon_vjp_tma_kernel(const float2* __restrict__ ahat, const int2* __restrict__ wq,
+                         const int32_t* __restrict__ wstat, const HaloArgs h, const uint8_t* __restrict__ sel_in,
                          const double* __restrict__ Uq_bar, float2* __restrict__ part,
                          double* __restrict__ u_self, int64_t n_cell, int64_t n_pad,
                          const DFTable ev, int* err) {
   constexpr int NV = 4, NQ3 = 3 * NQ, kPer = NQ3 * NV;
   using VP = VjpPlan<M, NS, NQ3>;
+  using Dot = WPairDot<26>;
   extern __shared__ __align__(128) unsigned char smem[];
   double* ubs = reinterpret_cast<double*>(smem + VP::kUbOff);     // [2][32][kUbStride]
-  float2* hacc = reinterpret_cast<float2*>(smem + VP::kHaccOff);  // [NV][kHaccStride]
+  int64_t* hacc = reinterpret_cast<int64_t*>(smem + VP::kHaccOff);  // [NV][kHaccStride]
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + VP::kBarOff);
   uint64_t* empty = full + kRingV;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + kRingV);
   int* need = const_cast<int*>(abort_flag) + 4;  // [NV] per-variable small-stencil flags
+  int* unit = need + NV;                         // [NV] exponents of the accumulators' units
+  unsigned* nanm = reinterpret_cast<unsigned*>(unit + NV);  // [NV][8] halo cells that take a NaN
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_tiles = (n_cell + kTile - 1) / kTile;
   if (threadIdx.x == 0) {
@@ -3752,18 +4234,20 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
     }
     cp_async_commit();
   };
-  float2* hrow = hacc + v * kHaccStride;
+  int64_t* hrow = hacc + v * kHaccStride;
   // add t at the halo position of code (bits 0-7); lanes with equal
-  // positions in the order of their precomputed ranks (bits 8-12)
-  auto accumulate = [&](bool act, int code, DF t) {
+  // positions in turn, by their precomputed ranks (bits 8-12); a lane whose
+  // cotangents hold an infinity or a NaN marks the halo cell instead
+  auto accumulate = [&](bool act, bool bad, int code, int64_t t) {
     const int hp = code & kHaloPosMask;
     const unsigned rank = (unsigned)code >> 8;
     const unsigned rmax = __reduce_max_sync(0xffffffffu, act ? rank : 0u);
     for (unsigned r = 0; r <= rmax; ++r) {
       if (act && rank == r) {
-        const float2 q = hrow[hp];
-        const DF s = DF{q.x, q.y} + t;
-        hrow[hp] = make_float2(s.h, s.l);
+        if (bad)
+          atomicOr(&nanm[v * 8 + (hp >> 5)], 1u << (hp & 31));
+        else
+          hrow[hp] += t;
       }
       __syncwarp();
     }
@@ -3772,19 +4256,21 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
   int hb = 0;
   bool dead = false;
   if ((int64_t)blockIdx.x < n_tiles) prefetch(blockIdx.x, 0);
-  // the halo offsets and the selection byte of a tile, loaded a tile ahead
-  auto pre = [&](int64_t tile, int& h0, int& H, uint8_t& sl) {
-    h0 = 0, H = 0, sl = 0;
+  // the halo offsets, the selection byte and the exponent of W's unit of a
+  // tile, loaded a tile ahead
+  auto pre = [&](int64_t tile, int& h0, int& H, uint8_t& sl, int& kc) {
+    h0 = 0, H = 0, sl = 0, kc = 0;
     if (tile < n_tiles) {
       h0 = h.off[tile];
       H = h.off[tile + 1] - h0;
       const int64_t cc = tile * kTile + lane;
       if (cc < n_cell) sl = sel_in[(int64_t)v * n_pad + cc];
+      kc = (int)(int16_t)(wstat[(tile * kWStat + kWStat - 1) * kTile + lane] & 0xffff);
     }
   };
-  int h0n, Hn;
+  int h0n, Hn, kcn;
   uint8_t seln;
-  pre(blockIdx.x, h0n, Hn, seln);
+  pre(blockIdx.x, h0n, Hn, seln, kcn);
   for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, hb ^= 1) {
     consumer_sync();  // the previous tile's accumulator, flags and Uq_bar stage are released
     const int64_t nxt = tile + gridDim.x;
@@ -3792,10 +4278,11 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
       prefetch(nxt, hb ^ 1);
     else
       cp_async_commit();
-    const int h0 = h0n, H = Hn;
+    const int h0 = h0n, H = Hn, kc = kcn;
     const uint8_t sel = seln;
-    pre(nxt, h0n, Hn, seln);
-    for (int i = lane; i < H; i += kTile) hrow[i] = make_float2(0.f, 0.f);
+    pre(nxt, h0n, Hn, seln, kcn);
+    for (int i = lane; i < H; i += kTile) hrow[i] = 0;
+    if (lane < 8) nanm[v * 8 + lane] = 0u;
     const int64_t c = tile * kTile + lane;
     const bool valid = c < n_cell;
     const bool vs = __any_sync(0xffffffffu, valid && vjp_needs_small(sel));
@@ -3804,35 +4291,72 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
     consumer_sync();  // the tile's Uq_bar has landed; the flags are set
     const bool small = need[0] | need[1] | need[2] | need[3];
     const int n_stages = small ? VP::kStages : VP::kNL;
-    // Uq_bar of (c, v) at the Gauss points (stored as pairs); the dU_0 term
-    DF ub[NQ3];
-    DF u0b = {0.f, 0.f};
+    const bool large = valid && (sel & 8);
+    const int nd = (sel & 1) + ((sel >> 1) & 1) + ((sel >> 2) & 1);
+    // Uq_bar of (c, v) at the Gauss points: in fixed point, 53 bits of the
+    // largest, unit 2^-sb; and the coefficient adjoints of the directional
+    // polynomials (first kSmallM basis functions) in pairs, where the block
+    // needs them
+    typename Dot::D bd[NQ3];
+    int sb = 0;
+    int64_t u0b = 0;
+    bool bad = false;
+    DF cbs[kSmallM];
+    int ec = kVjpNone;  // |directional contribution| < 2^ec
+#pragma unroll
+    for (int l = 0; l < kSmallM; ++l) cbs[l] = {0.f, 0.f};
     {
       const float2* us = reinterpret_cast<const float2*>(ubs) +
                          (size_t)hb * kTile * kUbStride + lane * kUbStride + v;
+      float2 q[NQ3];
+      unsigned mx = 0u;
 #pragma unroll
       for (int p = 0; p < NQ3; ++p) {
-        const float2 q = us[p * NV];
-        ub[p] = valid ? DF{q.x, q.y} : DF{0.f, 0.f};
-        u0b = u0b + ub[p];
+        q[p] = valid ? us[p * NV] : make_float2(0.f, 0.f);
+        mx = max(mx, mag_bits(q[p]));
       }
+      if (small && valid && !large && nd) {
+#pragma unroll
+        for (int p = 0; p < NQ3; ++p)
+#pragma unroll
+          for (int l = 0; l < kSmallM; ++l)
+            df_mac(cbs[l], ev.psi[p * kMaxM + l], DF{q[p].x, q[p].y});
+        float cm = 0.f, nm = 0.f;
+#pragma unroll
+        for (int l = 0; l < kSmallM; ++l) {
+          cbs[l] = df_norm(cbs[l]);
+          cm = fmaxf(cm, fabsf(cbs[l].h));
+        }
+#pragma unroll
+        for (int k = 0; k < kSmallK; ++k)
+          nm = fmaxf(nm, __int_as_float(wstat[(tile * kWStat + k) * kTile + lane]));
+        // |sum_l G_ls cb_l| <= max|cb| times the largest column sum
+        ec = mag_exp<float2>((unsigned)__float_as_int(cm)) +
+             mag_exp<float2>((unsigned)__float_as_int(nm)) + 3;
+      }
+      const int e = mag_exp<float2>(mx);
+      bad = e == kFixExpBad || ec >= kFixExpBad / 2;
+      sb = bad ? 0 : 52 - e;
+      if (bad) ec = kVjpNone;
+#pragma unroll
+      for (int p = 0; p < NQ3; ++p) {
+        const int64_t x = bad ? 0 : to_fix(q[p], sb);
+        Dot::split(x, 0.f, bd[p]);
+        u0b += x;
+      }
+      if (mx == 0u) sb = -kVjpNone;  // nothing to add: no claim on the unit
     }
-    const bool large = valid && (sel & 8);
-    const int nd = (sel & 1) + ((sel >> 1) & 1) + ((sel >> 2) & 1);
-    // coefficient adjoints of the directional polynomials (first kSmallM
-    // basis functions), only where some lane of the block needs them
-    DF cbs[kSmallM];
-#pragma unroll
-    for (int l = 0; l < kSmallM; ++l) cbs[l] = {0.f, 0.f};
-    if (small && valid && !large) {
-#pragma unroll
-      for (int p = 0; p < NQ3; ++p)
-#pragma unroll
-        for (int l = 0; l < kSmallM; ++l) df_mac(cbs[l], ev.psi[p * kMaxM + l], ub[p]);
-#pragma unroll
-      for (int l = 0; l < kSmallM; ++l) cbs[l] = df_norm(cbs[l]);
-    }
-    DF tot = {0.f, 0.f};
+    // the tile's accumulator unit 2^Ec of this variable: every contribution
+    // (W^T Uq_bar: |T| < 9 2^31 2^27 < 2^61.2 in units of 2^(26 - kc - sb)) stays below
+    // 2^56.2 units, so the at most 96 that meet in one halo cell, and a cell's
+    // own sum over its slots, stay below 2^63
+    const int uT = Dot::exp(kc, sb);
+    int Ec = bad ? kVjpNone : max(4 - sb, ec - 56);
+    if (large && !bad) Ec = max(Ec, uT + 5);
+    Ec = __reduce_max_sync(0xffffffffu, Ec);
+    if (lane == 0) unit[v] = Ec;
+    const int shT = Ec - uT;  // >= 5 on large lanes
+    int64_t tot = 0;
     for (int j = 0; j < n_stages; ++j, ++g) {
       const int b = (int)(g % kRingV);
       int slot0, nslot, k, bytes;
@@ -3846,62 +4370,75 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
         }
         dead = __any_sync(0xffffffffu, w != 1);
       }
-      const float2* mat = reinterpret_cast<const float2*>(smem + (size_t)b * VP::kMat) + lane;
-      const uint16_t* nl =
-          reinterpret_cast<const uint16_t*>(smem + (size_t)b * VP::kMat + VP::kNOff) + lane;
+      const unsigned char* buf = smem + (size_t)b * VP::kMat;
+      const uint16_t* nl = reinterpret_cast<const uint16_t*>(buf + VP::kNOff) + lane;
       if (dead) {
         // skip the stage
       } else if (k < 0) {
         if (__any_sync(0xffffffffu, large)) {
           // the stage's slot values first (independent chains), then their
           // accumulation slot by slot
-          DF ts[VP::kLPS];
+          int64_t ts[VP::kLPS];
 #pragma unroll
           for (int s = 0; s < VP::kLPS; ++s) {
-            ts[s] = {0.f, 0.f};
-            if (large && s < nslot) {
+            typename Dot::A acc;
 #pragma unroll
-              for (int p = 0; p < NQ3; ++p) df_mac(ts[s], mat[(s * NQ3 + p) * kTile], ub[p]);
-              ts[s] = df_norm(ts[s]);
-            }
+            for (int p = 0; p < NQ3; ++p)
+              Dot::mac(
+                  acc,
+                  Dot::entry(w_entry<VP::kLay * NQ3>(
+                      buf + s / VP::kLay * VP::kLay * VP::kSlotW, lane, s % VP::kLay * NQ3 + p)),
+                  bd[p]);
+            // (|x| < 2^35: rounded to 16 units)
+            const int64_t T = acc.hh + (int64_t)__float2int_rn(acc.x * 0.0625f) * 16;
+            ts[s] = large && s < nslot && !bad && shT < 63 ? (T + ((int64_t)1 << (shT - 1))) >> shT : 0;
           }
 #pragma unroll
           for (int s = 0; s < VP::kLPS; ++s) {
             if (s < nslot) {
-              accumulate(large, nl[s * kTile], ts[s]);
-              const DF q = two_sum(tot.h, ts[s].h);  // running sum, renormalised at the end
-              tot.h = q.h;
-              tot.l += q.l + ts[s].l;
+              accumulate(large, bad, nl[s * kTile], ts[s]);
+              tot += ts[s];
             }
           }
         }
       } else {
         const bool on = valid && !large && ((sel >> k) & 1);
         if (__any_sync(0xffffffffu, on)) {
+          const float2* mat = reinterpret_cast<const float2*>(buf) + lane;
 #pragma unroll
           for (int s = 0; s < VP::kSPS; ++s) {
-            DF t = {0.f, 0.f};
-            if (on) {
+            int64_t t = 0;
+            if (on && !bad) {
+              DF q = {0.f, 0.f};
 #pragma unroll
-              for (int l = 0; l < kSmallM; ++l) df_mac(t, mat[(s * kSmallM + l) * kTile], cbs[l]);
-              t = df_div_small(df_norm(t), nd);
+              for (int l = 0; l < kSmallM; ++l) df_mac(q, mat[(s * kSmallM + l) * kTile], cbs[l]);
+              q = df_div_small(df_norm(q), nd);
+              t = to_fix(make_float2(q.h, q.l), -Ec);
             }
-            accumulate(on, nl[s * kTile], t);
-            const DF q = two_sum(tot.h, t.h);
-            tot.h = q.h;
-            tot.l += q.l + t.l;
+            accumulate(on, bad, nl[s * kTile], t);
+            tot += t;
           }
         }
       }
       __syncwarp();
       if (lane == 0 && !dead) mbar_arrive(&empty[b]);
     }
-    if (valid && !dead) u_self[(int64_t)v * n_pad + c] = to_d(u0b - df_norm(tot));
+    if (valid && !dead) {
+      // sum_p Uq_bar_p - sum_s d_bar_s (the first in units of 2^-sb)
+      const int sh = Ec + sb;
+      const int64_t own = !bad && sh < 63 ? (u0b + ((int64_t)1 << (sh - 1))) >> sh : 0;
+      u_self[(int64_t)v * n_pad + c] =
+          bad ? __longlong_as_double(0x7ff8000000000000LL) : ldexp((double)(own - tot), Ec);
+    }
     consumer_sync();  // every variable's accumulator is complete
     if (!dead) {
       float2* dst = part + (int64_t)h0 * NV;
-      for (int e = tid; e < H * NV; e += kConsumers * kTile)
-        dst[e] = hacc[(e & 3) * kHaccStride + (e >> 2)];
+      for (int e = tid; e < H * NV; e += kConsumers * kTile) {
+        const int w = e & 3, i = e >> 2, Ew = unit[w];
+        DF r = fix_to_df(hacc[w * kHaccStride + i], exp2i(Ew + 42), exp2i(Ew + 21), exp2i(Ew));
+        if ((nanm[w * 8 + (i >> 5)] >> (i & 31)) & 1) r = DF{__int_as_float(0x7fffffff), 0.f};
+        dst[e] = make_float2(r.h, r.l);
+      }
     }
   }
   cp_async_wait<0>();
@@ -4041,12 +4578,12 @@ cudaError_t launch_recon_tma(const ReconArgs& a, const DeviceMesh& dm, int* err,
   return cudaGetLastError();
 }
 
-template <int M, int NS, int NQ, bool kN>
+template <int M, int NS, int NQ, typename HT>
 cudaError_t launch_recon_tma_w(const ReconArgs& a, const DeviceMesh& dm, int* err,
                                cudaStream_t st) {
-  using P = WPlan<M, NS, 3 * NQ, 3, 4>;
-  auto kern = recon_tma_w_kernel<M, NS, NQ, kN>;
-  const int threads = kTile * (kConsumers + 1);
+  using P = WPlan<M, NS, 3 * NQ, HT>;
+  auto kern = recon_tma_w_kernel<M, NS, NQ, HT>;
+  const int threads = kTile * (P::kWWarps + 1);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)P::kSmem);
   if (e != cudaSuccess) return e;
@@ -4060,8 +4597,15 @@ cudaError_t launch_recon_tma_w(const ReconArgs& a, const DeviceMesh& dm, int* er
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int64_t tiles = (a.n_cell + kTile - 1) / kTile;
   const int64_t grid = std::min<int64_t>(tiles, (int64_t)per_sm * sms);
-  const void* psi = kN ? (const void*)dm.psi_d : (const void*)dm.psi_df;
-  kern<<<(unsigned)grid, threads, P::kSmem, st>>>(a, dm.halo, psi, dm.g32, dm.wq, err);
+  WArgs wa;
+  wa.psi = std::is_same<HT, double>::value ? (const void*)dm.psi_d : (const void*)dm.psi_df;
+  wa.g32 = dm.g32;
+  wa.w = dm.wq;
+  wa.pos = dm.wpos;
+  wa.tile = dm.wtile;
+  wa.st = dm.wstat;
+  wa.t = dm.wt;
+  kern<<<(unsigned)grid, threads, P::kSmem, st>>>(a, wa, err);
   return cudaGetLastError();
 }
 
@@ -4128,7 +4672,7 @@ cudaError_t launch_recon(const DeviceMesh& dm, const double* U, const float2* Us
       const bool wn = NV == 4 && dm.variant == 2 && dm.err_flag && dm.halo.off && !ext &&
                       dm.precision == TENO_FP64_NATIVE && dm.g32 && dm.wq && dm.psi_d;
       if constexpr (NV == 4) {
-        if (wn) return launch_recon_tma_w<M, NS, NQ, true>(a, dm, dm.err_flag, st);
+        if (wn) return launch_recon_tma_w<M, NS, NQ, double>(a, dm, dm.err_flag, st);
       }
       const bool tma = NV == 4 && dm.variant == 2 && dm.err_flag && dm.halo.off &&
                        dm.precision != TENO_FP64_NATIVE;
@@ -4147,7 +4691,7 @@ cudaError_t launch_recon(const DeviceMesh& dm, const double* U, const float2* Us
       if constexpr (NV == 4) {
         if (tma) {
           if (dm.precision == TENO_FP64 && dm.scheme == 0 && dm.g32 && dm.wq && dm.psi_df)
-            return launch_recon_tma_w<M, NS, NQ, false>(a, dm, dm.err_flag, st);
+            return launch_recon_tma_w<M, NS, NQ, float2>(a, dm, dm.err_flag, st);
           if (ext) {
             if (dm.precision == TENO_FP64)
               return launch_recon_tma<M, NS, NQ, true, true>(a, dm, dm.err_flag, st);
@@ -4530,8 +5074,8 @@ cudaError_t launch_recon_vjp_tma_t(const DeviceMesh& dm, const uint8_t* sel, con
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int64_t tiles = (dm.n_recon + kTile - 1) / kTile;
   const int64_t grid = std::min<int64_t>(tiles, (int64_t)per_sm * sms);
-  kern<<<(unsigned)grid, threads, VP::kSmem, st>>>((const float2*)dm.ahat, dm.wq, dm.halo, sel,
-                                                   Uq_bar, part, u_self, dm.n_recon, dm.n_pad,
+  kern<<<(unsigned)grid, threads, VP::kSmem, st>>>((const float2*)dm.ahat, dm.wq, dm.wstat,
+                                                   dm.halo, sel, Uq_bar, part, u_self, dm.n_recon, dm.n_pad,
                                                    dm.eval_df, dm.err_flag);
   return cudaGetLastError();
 }
