@@ -770,6 +770,43 @@ __device__ __forceinline__ void ghost_state(int tag, const T* UL, double nx, dou
   for (int k = 0; k < 4; ++k) UR[k] = UL[k];
 }
 
+// Groups of NV = 4 values (the states at one Gauss point, the flux of one
+// face) as 16-byte accesses; the arrays are cudaMalloc'd and indexed in whole
+// groups, so every group starts on a 16-byte boundary.
+template <int NV, typename T>
+__device__ __forceinline__ void ld_group(const T* __restrict__ p, T (&x)[NV]) {
+  if constexpr (NV == 4 && std::is_same<T, float>::value) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+    x[0] = q.x, x[1] = q.y, x[2] = q.z, x[3] = q.w;
+  } else if constexpr (NV == 4 && std::is_same<T, DF>::value) {
+    const float4 q0 = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 q1 = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    x[0] = DF{q0.x, q0.y}, x[1] = DF{q0.z, q0.w}, x[2] = DF{q1.x, q1.y}, x[3] = DF{q1.z, q1.w};
+  } else if constexpr (NV == 4 && std::is_same<T, double>::value) {
+    const double2 q0 = __ldg(reinterpret_cast<const double2*>(p));
+    const double2 q1 = __ldg(reinterpret_cast<const double2*>(p) + 1);
+    x[0] = q0.x, x[1] = q0.y, x[2] = q1.x, x[3] = q1.y;
+  } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) x[v] = p[v];
+  }
+}
+template <int NV, typename T>
+__device__ __forceinline__ void st_group(T* __restrict__ p, const T (&x)[NV]) {
+  if constexpr (NV == 4 && std::is_same<T, float>::value) {
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+  } else if constexpr (NV == 4 && std::is_same<T, DF>::value) {
+    reinterpret_cast<float4*>(p)[0] = make_float4(x[0].h, x[0].l, x[1].h, x[1].l);
+    reinterpret_cast<float4*>(p)[1] = make_float4(x[2].h, x[2].l, x[3].h, x[3].l);
+  } else if constexpr (NV == 4 && std::is_same<T, double>::value) {
+    reinterpret_cast<double2*>(p)[0] = make_double2(x[0], x[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(x[2], x[3]);
+  } else {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) p[v] = x[v];
+  }
+}
+
 struct ReconArgs {
   const void* ahat;
   const int32_t* nbr;
@@ -3251,70 +3288,124 @@ __global__ void __launch_bounds__(128) char_finish_df_kernel(
 // so scaling the point values equals scaling the polynomial's deviation from
 // its mean (the average is unchanged).  Density: theta = (rho_0 - eps) /
 // (rho_0 - rho_q) where rho_q < eps; pressure (concave along the segment from
-// the average): 60 bisection halvings of [0, 1].  FP64; one thread per cell.
+// the average): 60 bisection halvings of [0, 1].  FP64.
 __device__ __forceinline__ double pp_pressure(double g, const double* W) {
   return (g - 1.0) * (W[3] - 0.5 * (W[1] * W[1] + W[2] * W[2]) / W[0]);
 }
 
-template <int NQ, typename TQ>
-__global__ void __launch_bounds__(128) positivity_kernel(const double* __restrict__ U,
-                                                         TQ* __restrict__ Uq, int64_t n_cell,
-                                                         int64_t n_pad, double g) {
-  constexpr int NP = 3 * NQ;
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n_cell) return;
-  double U0[4];
+// Largest theta in [0, 1] (60 halvings) that keeps rho > 0 and p >= ep along
+// U0 + theta (W - U0), where p < ep at theta = 1.
+__device__ __forceinline__ double pp_theta(double g, const double* U0, const double* W, double ep) {
+  double D[4];
 #pragma unroll
-  for (int v = 0; v < 4; ++v) U0[v] = U[v * n_pad + c];
-  const double er = fmin(1e-13, U0[0]), ep = fmin(1e-13, pp_pressure(g, U0));
-  TQ* q0 = Uq + c * NP * 4;
-  double W[NP][4];
+  for (int v = 0; v < 4; ++v) D[v] = W[v] - U0[v];
+  auto holds = [&](double th) {
+    double X[4];
 #pragma unroll
-  for (int q = 0; q < NP; ++q)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) W[q][v] = to_d(q0[q * 4 + v]);
-  bool scaled = false;
-  // pass 0: density
-  double th = 1.0;
-#pragma unroll
-  for (int q = 0; q < NP; ++q)
-    if (W[q][0] < er) th = fmin(th, (U0[0] - er) / (U0[0] - W[q][0]));
-  if (th < 1.0) {
-    scaled = true;
-#pragma unroll
-    for (int q = 0; q < NP; ++q)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) W[q][v] = U0[v] + th * (W[q][v] - U0[v]);
-  }
-  // pass 1: pressure
-  th = 1.0;
-  for (int q = 0; q < NP; ++q) {
-    if (pp_pressure(g, W[q]) >= ep) continue;
-    double lo = 0.0, hi = 1.0;
-    for (int it = 0; it < 60; ++it) {
-      const double sm = 0.5 * (lo + hi);
-      double X[4];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) X[v] = U0[v] + sm * (W[q][v] - U0[v]);
-      if (X[0] > 0.0 && pp_pressure(g, X) >= ep)
-        lo = sm;
-      else
-        hi = sm;
+    for (int v = 0; v < 4; ++v) X[v] = U0[v] + th * D[v];
+    return X[0] > 0.0 && pp_pressure(g, X) >= ep;
+  };
+  double lo = 0.0, hi = 1.0;
+  int it = 0;
+  // The bound is the root r of rho (E - ep / (g - 1)) - |m|^2 / 2, a quadratic
+  // in theta.  The halvings that lead to the smallest dyadic interval around r
+  // +- 2^-30 are skipped: p is concave in theta, so at their midpoints it
+  // stands off ep by at least 2^-30 (p_0 - ep), above its rounding where p_0 is
+  // 2^-16 of the energy or more; below that all 60 are made, and so they are
+  // if the interval's ends do not confirm it.
+  if (pp_pressure(g, U0) - ep > 1.6e-5 * U0[3]) {
+    const double e0 = U0[3] - ep / (g - 1.0);
+    const double A = D[0] * D[3] - 0.5 * (D[1] * D[1] + D[2] * D[2]);
+    const double B = U0[0] * D[3] + D[0] * e0 - (U0[1] * D[1] + U0[2] * D[2]);
+    const double C = U0[0] * e0 - 0.5 * (U0[1] * U0[1] + U0[2] * U0[2]);
+    const double q = sqrt(B * B - 4.0 * A * C);
+    const double r = B <= 0.0 ? 2.0 * C / (q - B) : (-B - q) / (2.0 * A);
+    const double r0 = r - 0x1p-30, r1 = r + 0x1p-30;
+    if (r0 > 0.0 && r1 < 1.0) {
+      // common leading bits of the two ends, as 30-bit fractions
+      const unsigned k0 = (unsigned)(r0 * 0x1p30), k1 = (unsigned)(r1 * 0x1p30);
+      const int n = k0 == k1 ? 30 : __clz(k0 ^ k1) - 2;
+      const double w = 1.0 / (double)(1u << n), l = (double)(k0 >> (30 - n)) * w;
+      if ((l == 0.0 || holds(l)) && (l + w >= 1.0 || !holds(l + w))) {
+        lo = l;
+        hi = l + w;
+        it = n;
+      }
     }
-    th = fmin(th, lo);
   }
-  if (th < 1.0) {
-    scaled = true;
+  for (; it < 60; ++it) {
+    const double sm = 0.5 * (lo + hi);
+    if (holds(sm))
+      lo = sm;
+    else
+      hi = sm;
+  }
+  return lo;
+}
+
+// One thread per (cell, Gauss point), 32 cells a block: a cell's theta is the
+// smallest of its points'.  Bound: the FP64 latency of the points that break
+// the floor, 30 bisection steps of an FP64 division each; one thread per cell
+// that took its points in turn, 60 steps each, left a few lanes of the warps at
+// the shock working for 309 us (double Mach reflection, 32,768 cells; now 62).
+template <int NQ, typename TQ>
+__global__ void __launch_bounds__(32 * 3 * NQ) positivity_kernel(const double* __restrict__ U,
+                                                                 TQ* __restrict__ Uq,
+                                                                 int64_t n_cell, int64_t n_pad,
+                                                                 double g) {
+  constexpr int NP = 3 * NQ;
+  __shared__ double s_th[32 * NP];
+  const int64_t i = (int64_t)blockIdx.x * (32 * NP) + threadIdx.x;
+  const int64_t c = i / NP;
+  const bool in = c < n_cell;
+  const int base = (int)threadIdx.x / NP * NP;
+  double U0[4], W[4], er = 0.0, ep = 0.0;
+  if (in) {
+    TQ x[4];
+    ld_group<4>(Uq + i * 4, x);
 #pragma unroll
-    for (int q = 0; q < NP; ++q)
+    for (int v = 0; v < 4; ++v) U0[v] = U[v * n_pad + c], W[v] = to_d(x[v]);
+    er = fmin(1e-13, U0[0]);
+    ep = fmin(1e-13, pp_pressure(g, U0));
+  }
+  // the cell's smallest theta from its points'
+  auto cell_min = [&](double th) {
+    s_th[threadIdx.x] = th;
+    __syncthreads();
+    double m = 1.0;
 #pragma unroll
-      for (int v = 0; v < 4; ++v) W[q][v] = U0[v] + th * (W[q][v] - U0[v]);
+    for (int q = 0; q < NP; ++q) m = fmin(m, s_th[base + q]);
+    __syncthreads();
+    return m;
+  };
+  auto scale = [&](double th) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) W[v] = U0[v] + th * (W[v] - U0[v]);
+  };
+  bool scaled = false;
+  // density
+  const bool low = in && W[0] < er;
+  if (__syncthreads_or(low)) {
+    const double th = cell_min(low ? fmin(1.0, (U0[0] - er) / (U0[0] - W[0])) : 1.0);
+    if (in && th < 1.0) {
+      scaled = true;
+      scale(th);
+    }
+  }
+  // pressure
+  const bool under = in && !(pp_pressure(g, W) >= ep);
+  if (__syncthreads_or(under)) {
+    const double th = cell_min(under ? pp_theta(g, U0, W, ep) : 1.0);
+    if (in && th < 1.0) {
+      scaled = true;
+      scale(th);
+    }
   }
   if (!scaled) return;
+  TQ x[4];
 #pragma unroll
-  for (int q = 0; q < NP; ++q)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) q0[q * 4 + v] = from_d<TQ>(W[q][v]);
+  for (int v = 0; v < 4; ++v) x[v] = from_d<TQ>(W[v]);
+  st_group<4>(Uq + i * 4, x);
 }
 
 // The outflow layer (cells with a face on an outflow boundary) enters every
@@ -3452,43 +3543,6 @@ __device__ __forceinline__ T gauss_w(double w, float2 w2) {
 // Gauss points of a face unrolled in the flux kernel: the pair-arithmetic
 // solver is large enough that one copy of its code runs faster (fewer
 // instruction-fetch stalls) than three; the FP32 and FP64 ones unroll
-// Groups of NV = 4 values (the states at one Gauss point, the flux of one
-// face) as 16-byte accesses; the arrays are cudaMalloc'd and indexed in whole
-// groups, so every group starts on a 16-byte boundary.
-template <int NV, typename T>
-__device__ __forceinline__ void ld_group(const T* __restrict__ p, T (&x)[NV]) {
-  if constexpr (NV == 4 && std::is_same<T, float>::value) {
-    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
-    x[0] = q.x, x[1] = q.y, x[2] = q.z, x[3] = q.w;
-  } else if constexpr (NV == 4 && std::is_same<T, DF>::value) {
-    const float4 q0 = __ldg(reinterpret_cast<const float4*>(p));
-    const float4 q1 = __ldg(reinterpret_cast<const float4*>(p) + 1);
-    x[0] = DF{q0.x, q0.y}, x[1] = DF{q0.z, q0.w}, x[2] = DF{q1.x, q1.y}, x[3] = DF{q1.z, q1.w};
-  } else if constexpr (NV == 4 && std::is_same<T, double>::value) {
-    const double2 q0 = __ldg(reinterpret_cast<const double2*>(p));
-    const double2 q1 = __ldg(reinterpret_cast<const double2*>(p) + 1);
-    x[0] = q0.x, x[1] = q0.y, x[2] = q1.x, x[3] = q1.y;
-  } else {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) x[v] = p[v];
-  }
-}
-template <int NV, typename T>
-__device__ __forceinline__ void st_group(T* __restrict__ p, const T (&x)[NV]) {
-  if constexpr (NV == 4 && std::is_same<T, float>::value) {
-    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
-  } else if constexpr (NV == 4 && std::is_same<T, DF>::value) {
-    reinterpret_cast<float4*>(p)[0] = make_float4(x[0].h, x[0].l, x[1].h, x[1].l);
-    reinterpret_cast<float4*>(p)[1] = make_float4(x[2].h, x[2].l, x[3].h, x[3].l);
-  } else if constexpr (NV == 4 && std::is_same<T, double>::value) {
-    reinterpret_cast<double2*>(p)[0] = make_double2(x[0], x[1]);
-    reinterpret_cast<double2*>(p)[1] = make_double2(x[2], x[3]);
-  } else {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) p[v] = x[v];
-  }
-}
-
 #ifndef TENO_FLUX_UNROLL_PAIRS
 #define TENO_FLUX_UNROLL_PAIRS 1
 #endif
@@ -4860,11 +4914,12 @@ cudaError_t launch_layer_vjp(const DeviceMesh& dm, double* Uq_bar, double* ubd, 
 cudaError_t launch_positivity(const DeviceMesh& dm, const double* U, void* Uq,
                               cudaStream_t st) {
   if (dm.n_var != 4) return cudaErrorInvalidValue;
-  const unsigned grid = (unsigned)((dm.n_recon + 127) / 128);
+  const unsigned grid = (unsigned)((dm.n_recon + 31) / 32);
   auto go = [&](auto nq, auto tq) -> cudaError_t {
     constexpr int NQ = decltype(nq)::value;
     using TQ = typename decltype(tq)::type;
-    positivity_kernel<NQ, TQ><<<grid, 128, 0, st>>>(U, (TQ*)Uq, dm.n_recon, dm.n_pad, dm.gamma);
+    positivity_kernel<NQ, TQ>
+        <<<grid, 32 * 3 * NQ, 0, st>>>(U, (TQ*)Uq, dm.n_recon, dm.n_pad, dm.gamma);
     return cudaGetLastError();
   };
   auto by_type = [&](auto nq) -> cudaError_t {
