@@ -3540,44 +3540,44 @@ __device__ __forceinline__ T gauss_w(double w, float2 w2) {
     return w2.x;
 }
 
-// Gauss points of a face unrolled in the flux kernel: the pair-arithmetic
-// solver is large enough that one copy of its code runs faster (fewer
-// instruction-fetch stalls) than three; the FP32 and FP64 ones unroll
-#ifndef TENO_FLUX_UNROLL_PAIRS
-#define TENO_FLUX_UNROLL_PAIRS 1
-#endif
-constexpr int kFluxUnrollPairs = TENO_FLUX_UNROLL_PAIRS;
+// One thread per (face, Gauss point), 64 faces a block; the points' fluxes go
+// through shared memory to the face's weighted sum, in the order of the points.
+// Bound: the issue of the Riemann solver (pairs, FP32) or the FP64 pipe at
+// large meshes, the latency of one solve at small ones, where a thread that
+// took a face's points in turn ran three of them in a row (32,768 cells TENO5
+// pairs: 18.6 us for three points a thread, 12.8 now; 262,088 cells TENO6:
+// 63 to 53.6; FP64, 131,072 cells: 199 to 174).
+constexpr int kFluxFaces = 64;
 
 template <int NV, int NQ, int FLUX, typename T>
-__global__ void __launch_bounds__(256) face_flux_kernel(const FaceArgs a, const T* __restrict__ Uq,
-                                                        T* __restrict__ K) {
-  const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= a.n_face) return;
-  const int o = a.f_cells[2 * f], n = a.f_cells[2 * f + 1];
-  const int eo = a.f_edges[2 * f], en = a.f_edges[2 * f + 1];
-  const double nx = a.f_geom[5 * f], ny = a.f_geom[5 * f + 1], len = a.f_geom[5 * f + 2];
-  T acc[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) acc[v] = cst<T>(0.0);
-  RiemannK<T> rk;
-  T tl;
-  face_k<T>(a.f_geom, a.f_geom2, f, a.gamma, a.g2, a.gm12, rk, tl);
-  // (the Gauss values of an outflow-layer cell are its cell average, written
-  // by layer_fill_kernel: at an outflow face both states are that average)
-#pragma unroll (std::is_same<T, DF>::value ? kFluxUnrollPairs : 4)
-  for (int k = 0; k < NQ; ++k) {
+__global__ void __launch_bounds__(kFluxFaces * NQ)
+    face_flux_kernel(const FaceArgs a, const T* __restrict__ Uq, T* __restrict__ K) {
+  __shared__ __align__(16) T sF[kFluxFaces * NQ * NV];
+  const int64_t f0 = (int64_t)blockIdx.x * kFluxFaces;
+  const int k = threadIdx.x % NQ;
+  const int64_t f = f0 + threadIdx.x / NQ;
+  if (f < a.n_face) {
+    const int o = a.f_cells[2 * f], n = a.f_cells[2 * f + 1];
+    const int eo = a.f_edges[2 * f], en = a.f_edges[2 * f + 1];
+    RiemannK<T> rk;
+    T tl;
+    face_k<T>(a.f_geom, a.f_geom2, f, a.gamma, a.g2, a.gm12, rk, tl);
+    // (the Gauss values of an outflow-layer cell are its cell average, written
+    // by layer_fill_kernel: at an outflow face both states are that average)
     T UL[NV], UR[NV], F[NV];
     ld_group<NV>(Uq + ((int64_t)(o * 3 + eo) * NQ + k) * NV, UL);
     if (n >= 0) {
       ld_group<NV>(Uq + ((int64_t)(n * 3 + en) * NQ + (NQ - 1 - k)) * NV, UR);
     } else if constexpr (NV == 4) {
-      double x = a.f_geom[5 * f + 3] - ny * len * a.gt[k];
+      const double nx = a.f_geom[5 * f], ny = a.f_geom[5 * f + 1], len = a.f_geom[5 * f + 2];
+      const double x = a.f_geom[5 * f + 3] - ny * len * a.gt[k];
       ghost_state<T>(en, UL, nx, ny, x, a.time, a.gamma, UR);
     } else {
 #pragma unroll
       for (int v = 0; v < NV; ++v) UR[v] = UL[v];
     }
     if constexpr (NV == 1) {
+      const double nx = a.f_geom[5 * f], ny = a.f_geom[5 * f + 1], len = a.f_geom[5 * f + 2];
       const double xq = a.f_geom[5 * f + 3] - ny * len * a.gt[k];
       const double yq = a.f_geom[5 * f + 4] + nx * len * a.gt[k];
       const double an = adv_normal(a.adv_field, a.adv_x, a.adv_y, a.adv_cx, a.adv_cy,
@@ -3586,13 +3586,21 @@ __global__ void __launch_bounds__(256) face_flux_kernel(const FaceArgs a, const 
     } else {
       euler_riemann<T>(UL, UR, rk, FLUX == TENO_FLUX_HLLC, F);
     }
-    const T wk = gauss_w<T>(a.gw[k], a.gw2[k]);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = madd(wk, F[v], acc[v]);
+    st_group<NV>(sF + threadIdx.x * NV, F);
   }
+  __syncthreads();
+  for (int e = threadIdx.x; e < kFluxFaces * NV; e += kFluxFaces * NQ) {
+    const int lf = e / NV, v = e % NV;
+    if (f0 + lf >= a.n_face) break;
+    RiemannK<T> rk;
+    T tl;
+    face_k<T>(a.f_geom, a.f_geom2, f0 + lf, a.gamma, a.g2, a.gm12, rk, tl);
+    T acc = cst<T>(0.0);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) acc[v] = acc[v] * tl;
-  st_group<NV>(K + f * NV, acc);
+    for (int q = 0; q < NQ; ++q)
+      acc = madd(gauss_w<T>(a.gw[q], a.gw2[q]), sF[(lf * NQ + q) * NV + v], acc);
+    K[f0 * NV + e] = acc * tl;
+  }
 }
 
 // ------------------------------------------------------------------ gather
@@ -4811,17 +4819,17 @@ static FaceArgs face_args(const DeviceMesh& dm, double time) {
 cudaError_t launch_face_flux(const DeviceMesh& dm, const void* Uq, void* K, double time,
                              cudaStream_t st) {
   FaceArgs a = face_args(dm, time);
-  const unsigned grid = (unsigned)((dm.n_face + 255) / 256);
+  const unsigned grid = (unsigned)((dm.n_face + kFluxFaces - 1) / kFluxFaces);
   auto go = [&](auto nvc, auto nqc, auto flc) -> cudaError_t {
     constexpr int NV = decltype(nvc)::value, NQ = decltype(nqc)::value,
                   FL = decltype(flc)::value;
     if (dm.precision == TENO_FP64_NATIVE)
-      face_flux_kernel<NV, NQ, FL, double><<<grid, 256, 0, st>>>(
+      face_flux_kernel<NV, NQ, FL, double><<<grid, kFluxFaces * NQ, 0, st>>>(
           a, (const double*)Uq, (double*)K);
     else if (dm.precision == TENO_FP64)
-      face_flux_kernel<NV, NQ, FL, DF><<<grid, 256, 0, st>>>(a, (const DF*)Uq, (DF*)K);
+      face_flux_kernel<NV, NQ, FL, DF><<<grid, kFluxFaces * NQ, 0, st>>>(a, (const DF*)Uq, (DF*)K);
     else
-      face_flux_kernel<NV, NQ, FL, float><<<grid, 256, 0, st>>>(a, (const float*)Uq, (float*)K);
+      face_flux_kernel<NV, NQ, FL, float><<<grid, kFluxFaces * NQ, 0, st>>>(a, (const float*)Uq, (float*)K);
     return cudaGetLastError();
   };
   using I1 = std::integral_constant<int, 1>;
