@@ -29,6 +29,21 @@
 namespace teno {
 namespace {
 
+// Programmatic dependent launch.  The kernels are launched so that the next one
+// starts when the last block of the one before it exits, and wait here for its
+// completion (and its writes) before the first access to memory that a kernel
+// writes: a launch's latency and prologue overlap the tail before it.  Ten
+// launches of a small step took 80 us and take 61 (2,048 cells, scalar TENO3),
+// a step of 32,768 cells TENO5 195 and 171.  No kernel triggers its successor
+// earlier: blocks that wait on occupied SMs end up unevenly spread (14,792
+// cells, scalar: 109 us a step, 177 with a trigger at the kernel's start).
+// Constant data of the plan may be read before the wait.  What a kernel writes
+// is read with plain loads only: the read-only path (ld.global.nc, const
+// __restrict__) assumes data that no running kernel writes.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 constexpr int kSmallEntries = kSmallK * kSmallN * kSmallM;  // 180
 // stencil slots unrolled together in the reconstruction loops (loads of that
 // many slots can be in flight per thread)
@@ -814,17 +829,17 @@ __device__ __forceinline__ void ghost_state(int tag, const T* UL, double nx, dou
 // face) as 16-byte accesses; the arrays are cudaMalloc'd and indexed in whole
 // groups, so every group starts on a 16-byte boundary.
 template <int NV, typename T>
-__device__ __forceinline__ void ld_group(const T* __restrict__ p, T (&x)[NV]) {
+__device__ __forceinline__ void ld_group(const T* p, T (&x)[NV]) {
   if constexpr (NV == 4 && std::is_same<T, float>::value) {
-    const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 q = *(reinterpret_cast<const float4*>(p));
     x[0] = q.x, x[1] = q.y, x[2] = q.z, x[3] = q.w;
   } else if constexpr (NV == 4 && std::is_same<T, DF>::value) {
-    const float4 q0 = __ldg(reinterpret_cast<const float4*>(p));
-    const float4 q1 = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    const float4 q0 = *(reinterpret_cast<const float4*>(p));
+    const float4 q1 = *(reinterpret_cast<const float4*>(p) + 1);
     x[0] = DF{q0.x, q0.y}, x[1] = DF{q0.z, q0.w}, x[2] = DF{q1.x, q1.y}, x[3] = DF{q1.z, q1.w};
   } else if constexpr (NV == 4 && std::is_same<T, double>::value) {
-    const double2 q0 = __ldg(reinterpret_cast<const double2*>(p));
-    const double2 q1 = __ldg(reinterpret_cast<const double2*>(p) + 1);
+    const double2 q0 = *(reinterpret_cast<const double2*>(p));
+    const double2 q1 = *(reinterpret_cast<const double2*>(p) + 1);
     x[0] = q0.x, x[1] = q0.y, x[2] = q1.x, x[3] = q1.y;
   } else {
 #pragma unroll
@@ -1146,6 +1161,7 @@ __device__ __forceinline__ void plain_finish(const ReconArgs& a, const TT& ev, i
 
 template <int M, int NS, int NQ, int NV, typename TA, typename TT>
 __global__ void __launch_bounds__(128) recon_kernel(const ReconArgs a, const TT ev) {
+  pdl_wait();
   constexpr bool kMixed = std::is_same<TA, float>::value;
   const int lane = threadIdx.x, v = threadIdx.y;
   const int64_t tile = (int64_t)blockIdx.x * blockDim.z + threadIdx.z;
@@ -1153,8 +1169,8 @@ __global__ void __launch_bounds__(128) recon_kernel(const ReconArgs a, const TT 
   if (c >= a.n_cell) return;
   constexpr int E = M * NS + kSmallEntries;
   constexpr int SL = NS + kSmallSlots;
-  const double* __restrict__ Uv = a.U + (int64_t)v * a.n_pad;
-  const float2* __restrict__ Usv = kMixed ? a.Us + (int64_t)v * a.n_pad : nullptr;
+  const double* Uv = a.U + (int64_t)v * a.n_pad;
+  const float2* Usv = kMixed ? a.Us + (int64_t)v * a.n_pad : nullptr;
   double u0 = 0.0;
   float2 u0s = make_float2(0.f, 0.f);
   if constexpr (kMixed)
@@ -1165,10 +1181,10 @@ __global__ void __launch_bounds__(128) recon_kernel(const ReconArgs a, const TT 
   const int32_t* __restrict__ nb = a.nbr + tile * (int64_t)SL * kTile + lane;
   auto diff = [&](int j) -> TA {
     if constexpr (kMixed) {
-      const float2 q = __ldg(Usv + j);
+      const float2 q = Usv[j];
       return (q.x - u0s.x) + (q.y - u0s.y);
     } else {
-      return __ldg(Uv + j) - u0;
+      return Uv[j] - u0;
     }
   };
 
@@ -1338,19 +1354,20 @@ __device__ __forceinline__ void df_finish(const ReconArgs& a, const DFTable& ev,
 
 template <int M, int NS, int NQ, int NV>
 __global__ void __launch_bounds__(128) recon_df_kernel(const ReconArgs a, const DFTable ev) {
+  pdl_wait();
   const int lane = threadIdx.x, v = threadIdx.y;
   const int64_t tile = (int64_t)blockIdx.x * blockDim.z + threadIdx.z;
   const int64_t c = tile * kTile + lane;
   if (c >= a.n_cell) return;
   constexpr int E = M * NS + kSmallEntries;
   constexpr int SL = NS + kSmallSlots;
-  const float2* __restrict__ Usv = a.Us + (int64_t)v * a.n_pad;
+  const float2* Usv = a.Us + (int64_t)v * a.n_pad;
   const float2 u0s = Usv[c];
   const float2* __restrict__ A =
       reinterpret_cast<const float2*>(a.ahat) + tile * (int64_t)E * kTile + lane;
   const int32_t* __restrict__ nb = a.nbr + tile * (int64_t)SL * kTile + lane;
   auto diff = [&](int j) -> DF {
-    const float2 q = __ldg(Usv + j);
+    const float2 q = Usv[j];
     DF s = two_sum(q.x, -u0s.x);
     s.l += q.y - u0s.y;
     return two_sum(s.h, s.l);
@@ -1418,6 +1435,7 @@ struct HaloTraits<2> {
 template <int M, int NS, int NQ, int NV, int kMode>
 __global__ void __launch_bounds__(128) recon_halo_kernel(const ReconArgs a, const HaloArgs h,
                                                          const typename HaloTraits<kMode>::Tab ev) {
+  pdl_wait();
   using TR = HaloTraits<kMode>;
   using TE = typename TR::TE;
   using TS = typename TR::TS;
@@ -1438,9 +1456,9 @@ __global__ void __launch_bounds__(128) recon_halo_kernel(const ReconArgs a, cons
 #pragma unroll
       for (int w = 0; w < NV; ++w) {
         if constexpr (kMode == 2)
-          hs[z][w][i] = __ldg(a.U + (int64_t)w * a.n_pad + id);
+          hs[z][w][i] = a.U[(int64_t)w * a.n_pad + id];
         else
-          hs[z][w][i] = __ldg(a.Us + (int64_t)w * a.n_pad + id);
+          hs[z][w][i] = a.Us[(int64_t)w * a.n_pad + id];
       }
     }
   }
@@ -1839,6 +1857,7 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), (kDF && kExt) ? 2 : 
     return;
   }
   // ---- consumers
+  pdl_wait();  // the states (the producer streams constant data before it)
   const int v = warp, tid = threadIdx.x;
   using Acc = typename TR::Acc;
   HaloPipe hp(h, a.Us, a.n_pad, n_tiles, tid);
@@ -2317,7 +2336,7 @@ __device__ __noinline__ int w_select(const HT* A, const int32_t* nb, const HT* s
 #pragma unroll
   for (int i = 0; i < (SL + kTile - 1) / kTile; ++i) {
     const int s = lane + i * kTile;
-    if (s < SL) dsc[s] = Ar::entry(Ar::dif(__ldg(st + __ldg(nb + s * kTile)), u0));
+    if (s < SL) dsc[s] = Ar::entry(Ar::dif(st[__ldg(nb + s * kTile)], u0));
   }
   __syncwarp();
   auto coef = [&](int q) {
@@ -2381,7 +2400,7 @@ __device__ __noinline__ void w_small(const HT* A, const int32_t* nb, const HT* s
 #pragma unroll
     for (int s = 0; s < kSmallN; ++s) id[s] = __ldg(nk + s * kTile);
 #pragma unroll
-    for (int s = 0; s < kSmallN; ++s) q[s] = __ldg(st + id[s]);
+    for (int s = 0; s < kSmallN; ++s) q[s] = st[id[s]];
     Acc as[kSmallM];
 #pragma unroll
     for (int l = 0; l < kSmallM; ++l) as[l] = Ar::zero();
@@ -2655,6 +2674,7 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
     return;
   }
   // ---- consumers (warp w: kVW variables from kVW w)
+  pdl_wait();  // the states (the producer streams constant data before it)
   constexpr int kPerLane = kHaloMax / kTile;
   const int v0 = warp * kVW;
   int2* mylist = list + warp * P::kListN;
@@ -3043,10 +3063,11 @@ __device__ __forceinline__ TQ from_d(double x) {
 
 template <int M, int NQ, typename TQ>
 __global__ void __launch_bounds__(128) char_finish_kernel(
-    const double* __restrict__ coef, const double* __restrict__ U,
+    const double* coef, const double* U,
     const uint8_t* __restrict__ smask, const int32_t* __restrict__ c_faces,
     const double* __restrict__ f_geom, const EvalTable ev, TQ* __restrict__ Uq, int64_t n_cell,
     int64_t n_pad, double g, double ct, double eps, int linear) {
+  pdl_wait();
   constexpr int C = M + kSmallK * kSmallM;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n_cell * 3) return;
@@ -3170,10 +3191,11 @@ __global__ void __launch_bounds__(128) char_finish_kernel(
 // path) or FP32 (mixed path).
 template <int M, int NQ, typename TQ>
 __global__ void __launch_bounds__(128) char_finish_df_kernel(
-    const float2* __restrict__ coef, const double* __restrict__ U,
+    const float2* coef, const double* U,
     const uint8_t* __restrict__ smask, const int32_t* __restrict__ c_faces,
     const double* __restrict__ f_geom, const DFTable ev, TQ* __restrict__ Uq, int64_t n_cell,
     int64_t n_pad, double g, double ct, double eps, int linear) {
+  pdl_wait();
   constexpr int C = M + kSmallK * kSmallM;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n_cell * 3) return;
@@ -3389,10 +3411,11 @@ __device__ __forceinline__ double pp_theta(double g, const double* U0, const dou
 // that took its points in turn, 60 steps each, left a few lanes of the warps at
 // the shock working for 309 us (double Mach reflection, 32,768 cells; now 62).
 template <int NQ, typename TQ>
-__global__ void __launch_bounds__(32 * 3 * NQ) positivity_kernel(const double* __restrict__ U,
+__global__ void __launch_bounds__(32 * 3 * NQ) positivity_kernel(const double* U,
                                                                  TQ* __restrict__ Uq,
                                                                  int64_t n_cell, int64_t n_pad,
                                                                  double g) {
+  pdl_wait();
   constexpr int NP = 3 * NQ;
   __shared__ double s_th[32 * NP];
   const int64_t i = (int64_t)blockIdx.x * (32 * NP) + threadIdx.x;
@@ -3453,8 +3476,9 @@ __global__ void __launch_bounds__(32 * 3 * NQ) positivity_kernel(const double* _
 // of such a cell takes U_0 (in the Gauss-value type of the path).  One thread
 // per (layer cell, slot).
 template <int NV, int NQ3, typename TQ>
-__global__ void layer_fill_kernel(const double* __restrict__ U, TQ* __restrict__ Uq,
+__global__ void layer_fill_kernel(const double* U, TQ* __restrict__ Uq,
                                   const int32_t* __restrict__ list, int64_t n, int64_t n_pad) {
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * NQ3) return;
   const int64_t c = list[i / NQ3];
@@ -3472,6 +3496,7 @@ __global__ void layer_fill_kernel(const double* __restrict__ U, TQ* __restrict__
 template <int NV, int NQ, bool kPairs>
 __global__ void layer_vjp_kernel(double* __restrict__ Uq_bar, double* __restrict__ ubd,
                                  const int32_t* __restrict__ list, int64_t n) {
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * 3) return;
   const int64_t c = list[i / 3];
@@ -3501,7 +3526,7 @@ __global__ void layer_vjp_kernel(double* __restrict__ Uq_bar, double* __restrict
 // its own context's arrays).  pack: buf[v][i] = U[v][idx[i]]; unpack: the
 // reverse, with the FP32 hi/lo split of the written states when Us is given;
 // add = 1 adds instead (the adjoint's contributions returned to their owner).
-__global__ void halo_pack_kernel(const double* __restrict__ U, int64_t ld,
+__global__ void halo_pack_kernel(const double* U, int64_t ld,
                                  const int32_t* __restrict__ idx, int64_t n, int n_var,
                                  double* __restrict__ buf) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -3526,8 +3551,9 @@ __global__ void halo_unpack_kernel(double* __restrict__ U, int64_t ld,
   }
 }
 
-__global__ void split_kernel(const double* __restrict__ U, float2* __restrict__ Us, int64_t n_cell,
+__global__ void split_kernel(const double* U, float2* __restrict__ Us, int64_t n_cell,
                              int64_t n_pad, int n_var) {
+  pdl_wait();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n_cell) return;
   for (int v = 0; v < n_var; ++v) {
@@ -3591,7 +3617,8 @@ constexpr int kFluxFaces = 64;
 
 template <int NV, int NQ, int FLUX, typename T>
 __global__ void __launch_bounds__(kFluxFaces * NQ)
-    face_flux_kernel(const FaceArgs a, const T* __restrict__ Uq, T* __restrict__ K) {
+    face_flux_kernel(const FaceArgs a, const T* Uq, T* __restrict__ K) {
+  pdl_wait();
   __shared__ __align__(16) T sF[kFluxFaces * NQ * NV];
   const int64_t f0 = (int64_t)blockIdx.x * kFluxFaces;
   const int k = threadIdx.x % NQ;
@@ -3652,13 +3679,14 @@ struct GatherArgs {
 };
 
 template <int NV, typename TK>
-__global__ void __launch_bounds__(256) gather_kernel(const GatherArgs a, const TK* __restrict__ K,
-                                                     const double* __restrict__ Un,
-                                                     const double* __restrict__ Us,
+__global__ void __launch_bounds__(256) gather_kernel(const GatherArgs a, const TK* K,
+                                                     const double* Un,
+                                                     const double* Us,
                                                      double* __restrict__ out, int mode, double cn,
                                                      double cs, double dt_fixed, double cfl,
-                                                     const double* __restrict__ max_lam,
+                                                     const double* max_lam,
                                                      int* flag, float2* __restrict__ split) {
+  pdl_wait();
   // the step size once per block (one FP64 division)
   __shared__ double s_dt;
   if (mode != 0 && threadIdx.x == 0) s_dt = max_lam ? cfl / *max_lam : dt_fixed;
@@ -3734,12 +3762,13 @@ __global__ void __launch_bounds__(256) gather_kernel(const GatherArgs a, const T
 
 // --------------------------------------------------------------- CFL speed
 template <int NV>
-__global__ void __launch_bounds__(256) max_lambda_kernel(const double* __restrict__ U,
+__global__ void __launch_bounds__(256) max_lambda_kernel(const double* U,
                                                          const double* __restrict__ cfl_len,
                                                          int64_t n_cell, int64_t n_pad,
                                                          double gamma, double adv_speed,
                                                          const double* __restrict__ cell_speed,
                                                          unsigned long long* out) {
+  pdl_wait();
   double lam = 0.0;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cell;
        c += (int64_t)gridDim.x * blockDim.x) {
@@ -3776,11 +3805,12 @@ __global__ void __launch_bounds__(256) max_lambda_kernel(const double* __restric
 // in pair arithmetic on the FP32 pipe (relative error ~1e-14, far below what
 // a CFL step needs) with 1/L_c as host-split pairs; the maximum as FP64
 // bits.  Non-physical cells (NaN speed) are skipped as fmax skips them.
-__global__ void __launch_bounds__(256) max_lambda_split_kernel(const float2* __restrict__ Us,
+__global__ void __launch_bounds__(256) max_lambda_split_kernel(const float2* Us,
                                                                const float2* __restrict__ ilen2,
                                                                int64_t n_cell, int64_t n_pad,
                                                                float2 g2, float2 gm12,
                                                                unsigned long long* out) {
+  pdl_wait();
   const DF one = {1.f, 0.f}, half = {0.5f, 0.f}, gg = {g2.x, g2.y}, gm1 = {gm12.x, gm12.y};
   DF lam = {0.f, 0.f};
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cell;
@@ -3812,9 +3842,10 @@ __global__ void __launch_bounds__(256) max_lambda_split_kernel(const float2* __r
 }
 
 // -------------------------------------------------------------- utilities
-__global__ void permute_kernel(const double* __restrict__ src, double* __restrict__ dst,
+__global__ void permute_kernel(const double* src, double* __restrict__ dst,
                                const int32_t* __restrict__ perm, int64_t n, int64_t ld_src,
                                int64_t ld_dst, int to_user) {
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int v = blockIdx.y;
   if (i >= n) return;
@@ -3825,9 +3856,10 @@ __global__ void permute_kernel(const double* __restrict__ src, double* __restric
     dst[v * ld_dst + i] = src[v * ld_src + u];
 }
 
-__global__ void permute_u8_kernel(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst,
+__global__ void permute_u8_kernel(const uint8_t* src, uint8_t* __restrict__ dst,
                                   const int32_t* __restrict__ perm, int64_t n, int64_t ld_src,
                                   int64_t ld_dst, int to_user) {
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int v = blockIdx.y;
   if (i >= n) return;
@@ -3840,6 +3872,7 @@ __global__ void permute_u8_kernel(const uint8_t* __restrict__ src, uint8_t* __re
 
 __global__ void axpby_kernel(double* out, const double* a, double ca, const double* b, double cb,
                              int64_t n) {
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = ca * a[i] + cb * b[i];
 }
@@ -3894,9 +3927,10 @@ __device__ __forceinline__ void store_bar(double* base, int i, S x) {
 template <int NV, int NQ, int FLUX, typename TQ, typename S, int ND>
 __global__ void __launch_bounds__(128, TENO_VJP_MIN_BLOCKS > 0 ? TENO_VJP_MIN_BLOCKS : 1)
     face_flux_vjp_kernel(const VjpArgs a,
-                                                            const TQ* __restrict__ Uq,
-                                                            const double* __restrict__ w,
+                                                            const TQ* Uq,
+                                                            const double* w,
                                                             double* __restrict__ Uq_bar) {
+  pdl_wait();
   static_assert((2 * NV) % ND == 0, "directions per pass must divide 2 NV");
   using D = Dual<ND, S>;
   const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -4011,12 +4045,13 @@ constexpr int kVjpSlotUnroll = TENO_VJP_SLOT_UNROLL;
 // (selection frozen); u_self = sum_p Uq_bar - sum_slot d_bar (dU_0 terms).
 template <int M, int NS, int NQ, int NV, typename TS>
 __global__ void __launch_bounds__(128) recon_vjp_kernel(const TS* __restrict__ ahat,
-                                                        const uint8_t* __restrict__ sel_in,
-                                                        const double* __restrict__ Uq_bar,
+                                                        const uint8_t* sel_in,
+                                                        const double* Uq_bar,
                                                         double* __restrict__ d_bar,
                                                         double* __restrict__ u_self,
                                                         int64_t n_cell, int64_t n_pad,
                                                         const EvalTable ev) {
+  pdl_wait();
   const int lane = threadIdx.x, v = threadIdx.y;
   const int64_t tile = (int64_t)blockIdx.x * blockDim.z + threadIdx.z;
   const int64_t c = tile * kTile + lane;
@@ -4089,12 +4124,13 @@ __device__ __forceinline__ DF df_div_small(DF a, int n) {  // a / n for n in 1..
 
 template <int M, int NS, int NQ, int NV>
 __global__ void __launch_bounds__(128) recon_vjp_df_kernel(const float2* __restrict__ ahat,
-                                                           const uint8_t* __restrict__ sel_in,
-                                                           const double* __restrict__ Uq_bar,
+                                                           const uint8_t* sel_in,
+                                                           const double* Uq_bar,
                                                            DF* __restrict__ d_bar,
                                                            double* __restrict__ u_self,
                                                            int64_t n_cell, int64_t n_pad,
                                                            const DFTable ev) {
+  pdl_wait();
   const int lane = threadIdx.x, v = threadIdx.y;
   const int64_t tile = (int64_t)blockIdx.x * blockDim.z + threadIdx.z;
   const int64_t c = tile * kTile + lane;
@@ -4232,10 +4268,12 @@ __device__ __forceinline__ bool vjp_needs_small(uint8_t sel) {
 template <int M, int NS, int NQ>
 __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
     recon_vjp_tma_kernel(const float2* __restrict__ ahat, const int2* __restrict__ wq,
-                         const int32_t* __restrict__ wstat, const HaloArgs h, const uint8_t* __restrict__ sel_in,
-                         const double* __restrict__ Uq_bar, float2* __restrict__ part,
+                         const int32_t* __restrict__ wstat, const HaloArgs h,
+                         const uint8_t* sel_in,
+                         const double* Uq_bar, float2* __restrict__ part,
                          double* __restrict__ u_self, int64_t n_cell, int64_t n_pad,
                          const DFTable ev, int* err) {
+  pdl_wait();
   constexpr int NV = 4, NQ3 = 3 * NQ, kPer = NQ3 * NV;
   using VP = VjpPlan<M, NS, NQ3>;
   using Dot = WPairDot<26>;
@@ -4277,7 +4315,7 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
 #pragma unroll
           for (int q = 0; q < 2; ++q)
             sw4[2 * w + q] =
-                __ldg(reinterpret_cast<const uint4*>(sel_in + (int64_t)w * n_pad + tile * kTile) + q);
+                *(reinterpret_cast<const uint4*>(sel_in + (int64_t)w * n_pad + tile * kTile) + q);
         bool small = false;
 #pragma unroll
         for (int w = 0; w < NV; ++w)
@@ -4557,11 +4595,12 @@ constexpr int kScatterBatch = TENO_SCATTER_BATCH;
 template <int NV, typename TD>
 __global__ void __launch_bounds__(256) scatter_gather_kernel(const int64_t* __restrict__ rev_off,
                                                              const int32_t* __restrict__ rev_idx,
-                                                             const TD* __restrict__ d_bar,
-                                                             const double* __restrict__ u_self0,
+                                                             const TD* d_bar,
+                                                             const double* u_self0,
                                                              double* __restrict__ out,
                                                              int64_t n_cell, int64_t n_pad,
-                                                             const double* __restrict__ ubd) {
+                                                             const double* ubd) {
+  pdl_wait();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_cell) return;
   const int64_t r0 = rev_off[j], r1 = rev_off[j + 1];
@@ -4590,8 +4629,8 @@ __global__ void __launch_bounds__(256) scatter_gather_kernel(const int64_t* __re
 #pragma unroll
         for (int i = 0; i < kScatterBatch; ++i) {
           const float4* e = reinterpret_cast<const float4*>(d_bar + (int64_t)id[i] * NV);
-          a[i] = __ldg(e);
-          b[i] = __ldg(e + 1);
+          a[i] = e[0];
+          b[i] = e[1];
         }
 #pragma unroll
         for (int i = 0; i < kScatterBatch; ++i) {
@@ -4605,8 +4644,8 @@ __global__ void __launch_bounds__(256) scatter_gather_kernel(const int64_t* __re
     for (; r < r1; ++r) {
       const TD* e = d_bar + (int64_t)rev_idx[r] * NV;
       if constexpr (NV == 4) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(e));
-        const float4 b = __ldg(reinterpret_cast<const float4*>(e) + 1);
+        const float4 a = *reinterpret_cast<const float4*>(e);
+        const float4 b = *(reinterpret_cast<const float4*>(e) + 1);
         acc[0] = acc[0] + DF{a.x, a.y};
         acc[1] = acc[1] + DF{a.z, a.w};
         acc[2] = acc[2] + DF{b.x, b.y};
@@ -4625,8 +4664,8 @@ __global__ void __launch_bounds__(256) scatter_gather_kernel(const int64_t* __re
     for (int64_t r = r0; r < r1; ++r) {
       const TD* e = d_bar + (int64_t)rev_idx[r] * NV;
       if constexpr (NV == 4) {
-        const double2 a = __ldg(reinterpret_cast<const double2*>(e));
-        const double2 b = __ldg(reinterpret_cast<const double2*>(e) + 1);
+        const double2 a = *reinterpret_cast<const double2*>(e);
+        const double2 b = *(reinterpret_cast<const double2*>(e) + 1);
         acc[0] += a.x;
         acc[1] += a.y;
         acc[2] += b.x;
@@ -4650,6 +4689,24 @@ cudaError_t dispatch_order(int order, F&& f) {
     case 6: return f(std::integral_constant<int, 20>{}, std::integral_constant<int, 42>{});
   }
   return cudaErrorInvalidValue;
+}
+
+// launch with the programmatic-serialization attribute (pdl_wait)
+// (the callers return cudaGetLastError())
+template <typename... KA, typename... A>
+void launch(void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+            A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, KA(args)...);
 }
 
 }  // namespace
@@ -4676,7 +4733,7 @@ cudaError_t launch_recon_tma(const ReconArgs& a, const DeviceMesh& dm, int* err,
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int64_t tiles = (a.n_cell + kTile - 1) / kTile;
   const int64_t grid = std::min<int64_t>(tiles, (int64_t)per_sm * sms);
-  kern<<<(unsigned)grid, threads, smem, st>>>(a, dm.halo, dm.eval_df, err);
+  launch(kern, (unsigned)grid, threads, smem, st, a, dm.halo, dm.eval_df, err);
   return cudaGetLastError();
 }
 
@@ -4707,7 +4764,7 @@ cudaError_t launch_recon_tma_w(const ReconArgs& a, const DeviceMesh& dm, int* er
   wa.tile = dm.wtile;
   wa.st = dm.wstat;
   wa.t = dm.wt;
-  kern<<<(unsigned)grid, threads, P::kSmem, st>>>(a, wa, err);
+  launch(kern, (unsigned)grid, threads, P::kSmem, st, a, wa, err);
   return cudaGetLastError();
 }
 
@@ -4722,12 +4779,12 @@ cudaError_t launch_char_finish(const DeviceMesh& dm, const double* U, void* Uq, 
     auto go = [&](auto tq) -> cudaError_t {
       using TQ = typename decltype(tq)::type;
       if constexpr (std::is_same<TQ, double>::value)
-        char_finish_kernel<M, NQ, TQ><<<grid, 128, 0, st>>>(
-            dm.coef_out, U, dm.smask, dm.c_faces, dm.f_geom, dm.eval, (TQ*)Uq, dm.n_recon,
+        launch(char_finish_kernel<M, NQ, TQ>, grid, 128, 0, st, dm.coef_out, U, dm.smask,
+               dm.c_faces, dm.f_geom, dm.eval, (TQ*)Uq, dm.n_recon,
             dm.n_pad, dm.gamma, dm.ct, dm.eps, dm.linear);
       else
-        char_finish_df_kernel<M, NQ, TQ><<<grid, 128, 0, st>>>(
-            reinterpret_cast<const float2*>(dm.coef_out), U, dm.smask, dm.c_faces, dm.f_geom,
+        launch(char_finish_df_kernel<M, NQ, TQ>, grid, 128, 0, st,
+               reinterpret_cast<const float2*>(dm.coef_out), U, dm.smask, dm.c_faces, dm.f_geom,
             dm.eval_df, (TQ*)Uq, dm.n_recon, dm.n_pad, dm.gamma, dm.ct, dm.eps, dm.linear);
       return cudaGetLastError();
     };
@@ -4783,11 +4840,11 @@ cudaError_t launch_recon(const DeviceMesh& dm, const double* U, const float2* Us
         dim3 block(kTile, NV, TZh);
         dim3 grid((unsigned)((tiles + TZh - 1) / TZh));
         if (dm.precision == TENO_FP64)
-          recon_halo_kernel<M, NS, NQ, NV, 0><<<grid, block, 0, st>>>(a, dm.halo, dm.eval_df);
+          launch(recon_halo_kernel<M, NS, NQ, NV, 0>, grid, block, 0, st, a, dm.halo, dm.eval_df);
         else if (dm.precision == TENO_FP32_MIXED)
-          recon_halo_kernel<M, NS, NQ, NV, 1><<<grid, block, 0, st>>>(a, dm.halo, dm.eval_df);
+          launch(recon_halo_kernel<M, NS, NQ, NV, 1>, grid, block, 0, st, a, dm.halo, dm.eval_df);
         else
-          recon_halo_kernel<M, NS, NQ, NV, 2><<<grid, block, 0, st>>>(a, dm.halo, dm.eval);
+          launch(recon_halo_kernel<M, NS, NQ, NV, 2>, grid, block, 0, st, a, dm.halo, dm.eval);
         return cudaGetLastError();
       }
       if constexpr (NV == 4) {
@@ -4808,11 +4865,11 @@ cudaError_t launch_recon(const DeviceMesh& dm, const double* U, const float2* Us
       dim3 block(kTile, NV, TZ);
       dim3 grid((unsigned)((tiles + TZ - 1) / TZ));
       if (dm.precision == TENO_FP64_NATIVE)
-        recon_kernel<M, NS, NQ, NV, double, EvalTable><<<grid, block, 0, st>>>(a, dm.eval);
+        launch(recon_kernel<M, NS, NQ, NV, double, EvalTable>, grid, block, 0, st, a, dm.eval);
       else if (dm.precision == TENO_FP64)
-        recon_df_kernel<M, NS, NQ, NV><<<grid, block, 0, st>>>(a, dm.eval_df);
+        launch(recon_df_kernel<M, NS, NQ, NV>, grid, block, 0, st, a, dm.eval_df);
       else
-        recon_kernel<M, NS, NQ, NV, float, DFTable><<<grid, block, 0, st>>>(a, dm.eval_df);
+        launch(recon_kernel<M, NS, NQ, NV, float, DFTable>, grid, block, 0, st, a, dm.eval_df);
       return cudaGetLastError();
     };
     constexpr int NQd = (M <= 9) ? 2 : 3;
@@ -4864,12 +4921,14 @@ cudaError_t launch_face_flux(const DeviceMesh& dm, const void* Uq, void* K, doub
     constexpr int NV = decltype(nvc)::value, NQ = decltype(nqc)::value,
                   FL = decltype(flc)::value;
     if (dm.precision == TENO_FP64_NATIVE)
-      face_flux_kernel<NV, NQ, FL, double><<<grid, kFluxFaces * NQ, 0, st>>>(
-          a, (const double*)Uq, (double*)K);
+      launch(face_flux_kernel<NV, NQ, FL, double>, grid, kFluxFaces * NQ, 0, st, a,
+             (const double*)Uq, (double*)K);
     else if (dm.precision == TENO_FP64)
-      face_flux_kernel<NV, NQ, FL, DF><<<grid, kFluxFaces * NQ, 0, st>>>(a, (const DF*)Uq, (DF*)K);
+      launch(face_flux_kernel<NV, NQ, FL, DF>, grid, kFluxFaces * NQ, 0, st, a, (const DF*)Uq,
+             (DF*)K);
     else
-      face_flux_kernel<NV, NQ, FL, float><<<grid, kFluxFaces * NQ, 0, st>>>(a, (const float*)Uq, (float*)K);
+      launch(face_flux_kernel<NV, NQ, FL, float>, grid, kFluxFaces * NQ, 0, st, a, (const float*)Uq,
+             (float*)K);
     return cudaGetLastError();
   };
   using I1 = std::integral_constant<int, 1>;
@@ -4892,7 +4951,7 @@ cudaError_t launch_gather(const DeviceMesh& dm, const void* K, const double* Un,
   auto go = [&](auto nvc, auto tkc) {
     constexpr int NV = decltype(nvc)::value;
     using TK = typename decltype(tkc)::type;
-    gather_kernel<NV, TK><<<grid, 256, 0, st>>>(a, (const TK*)K, Un, Us, out, mode, cn, cs,
+    launch(gather_kernel<NV, TK>, grid, 256, 0, st, a, (const TK*)K, Un, Us, out, mode, cn, cs,
                                                 dt_fixed, dm.cfl, max_lam, flag, split);
   };
   using I1 = std::integral_constant<int, 1>;
@@ -4915,13 +4974,13 @@ cudaError_t launch_layer_fill(const DeviceMesh& dm, const double* U, void* Uq, c
   auto go = [&](auto nvc, auto nqc) {
     constexpr int NV = decltype(nvc)::value, NQ3 = 3 * decltype(nqc)::value;
     if (dm.precision == TENO_FP64)
-      layer_fill_kernel<NV, NQ3, DF><<<grid, 256, 0, st>>>(U, (DF*)Uq, dm.fo_list, dm.fo_n,
+      launch(layer_fill_kernel<NV, NQ3, DF>, grid, 256, 0, st, U, (DF*)Uq, dm.fo_list, dm.fo_n,
                                                             dm.n_pad);
     else if (dm.precision == TENO_FP32_MIXED)
-      layer_fill_kernel<NV, NQ3, float><<<grid, 256, 0, st>>>(U, (float*)Uq, dm.fo_list,
+      launch(layer_fill_kernel<NV, NQ3, float>, grid, 256, 0, st, U, (float*)Uq, dm.fo_list,
                                                               dm.fo_n, dm.n_pad);
     else
-      layer_fill_kernel<NV, NQ3, double><<<grid, 256, 0, st>>>(U, (double*)Uq, dm.fo_list,
+      launch(layer_fill_kernel<NV, NQ3, double>, grid, 256, 0, st, U, (double*)Uq, dm.fo_list,
                                                                dm.fo_n, dm.n_pad);
   };
   using I1 = std::integral_constant<int, 1>;
@@ -4943,9 +5002,9 @@ cudaError_t launch_layer_vjp(const DeviceMesh& dm, double* Uq_bar, double* ubd, 
   auto go = [&](auto nvc, auto nqc) {
     constexpr int NV = decltype(nvc)::value, NQ = decltype(nqc)::value;
     if (pairs)
-      layer_vjp_kernel<NV, NQ, true><<<grid, 256, 0, st>>>(Uq_bar, ubd, dm.fo_list, dm.fo_n);
+      launch(layer_vjp_kernel<NV, NQ, true>, grid, 256, 0, st, Uq_bar, ubd, dm.fo_list, dm.fo_n);
     else
-      layer_vjp_kernel<NV, NQ, false><<<grid, 256, 0, st>>>(Uq_bar, ubd, dm.fo_list, dm.fo_n);
+      launch(layer_vjp_kernel<NV, NQ, false>, grid, 256, 0, st, Uq_bar, ubd, dm.fo_list, dm.fo_n);
   };
   using I1 = std::integral_constant<int, 1>;
   using I4 = std::integral_constant<int, 4>;
@@ -4966,8 +5025,8 @@ cudaError_t launch_positivity(const DeviceMesh& dm, const double* U, void* Uq,
   auto go = [&](auto nq, auto tq) -> cudaError_t {
     constexpr int NQ = decltype(nq)::value;
     using TQ = typename decltype(tq)::type;
-    positivity_kernel<NQ, TQ>
-        <<<grid, 32 * 3 * NQ, 0, st>>>(U, (TQ*)Uq, dm.n_recon, dm.n_pad, dm.gamma);
+    launch(positivity_kernel<NQ, TQ>, grid, 32 * 3 * NQ, 0, st, U, (TQ*)Uq, dm.n_recon, dm.n_pad,
+           dm.gamma);
     return cudaGetLastError();
   };
   auto by_type = [&](auto nq) -> cudaError_t {
@@ -4995,7 +5054,7 @@ cudaError_t launch_halo_unpack(double* U, int64_t ld, const int32_t* idx, int64_
 }
 
 cudaError_t launch_split(const DeviceMesh& dm, const double* U, float2* Us, cudaStream_t st) {
-  split_kernel<<<(unsigned)((dm.n_cell + 255) / 256), 256, 0, st>>>(U, Us, dm.n_cell, dm.n_pad,
+  launch(split_kernel, (unsigned)((dm.n_cell + 255) / 256), 256, 0, st, U, Us, dm.n_cell, dm.n_pad,
                                                                     dm.n_var);
   return cudaGetLastError();
 }
@@ -5008,12 +5067,12 @@ cudaError_t launch_max_lambda(const DeviceMesh& dm, const double* U, double* max
   if (blocks > 152 * 8) blocks = 152 * 8;
   const double adv = sqrt(dm.adv_x * dm.adv_x + dm.adv_y * dm.adv_y);
   if (dm.n_var == 1)
-    max_lambda_kernel<1><<<(unsigned)blocks, 256, 0, st>>>(
-        U, dm.cfl_len, dm.n_update, dm.n_pad, dm.gamma, adv, dm.cell_speed,
+    launch(max_lambda_kernel<1>, (unsigned)blocks, 256, 0, st, U, dm.cfl_len, dm.n_update, dm.n_pad,
+           dm.gamma, adv, dm.cell_speed,
         (unsigned long long*)max_lam);
   else
-    max_lambda_kernel<4><<<(unsigned)blocks, 256, 0, st>>>(
-        U, dm.cfl_len, dm.n_update, dm.n_pad, dm.gamma, adv, nullptr,
+    launch(max_lambda_kernel<4>, (unsigned)blocks, 256, 0, st, U, dm.cfl_len, dm.n_update, dm.n_pad,
+           dm.gamma, adv, nullptr,
         (unsigned long long*)max_lam);
   return cudaGetLastError();
 }
@@ -5025,8 +5084,8 @@ cudaError_t launch_max_lambda_split(const DeviceMesh& dm, const float2* Us, doub
   if (e != cudaSuccess) return e;
   int64_t blocks = (dm.n_update + 255) / 256;
   if (blocks > 152 * 8) blocks = 152 * 8;
-  max_lambda_split_kernel<<<(unsigned)blocks, 256, 0, st>>>(
-      Us, dm.cfl_ilen2, dm.n_update, dm.n_pad, split2(dm.gamma), split2(dm.gamma - 1.0),
+  launch(max_lambda_split_kernel, (unsigned)blocks, 256, 0, st, Us, dm.cfl_ilen2, dm.n_update,
+         dm.n_pad, split2(dm.gamma), split2(dm.gamma - 1.0),
       (unsigned long long*)max_lam);
   return cudaGetLastError();
 }
@@ -5035,7 +5094,7 @@ cudaError_t launch_permute(const double* src, double* dst, const int32_t* perm, 
                            int64_t ld_src, int64_t ld_dst, int n_var, int to_user,
                            cudaStream_t st) {
   dim3 grid((unsigned)((n + 255) / 256), n_var);
-  permute_kernel<<<grid, 256, 0, st>>>(src, dst, perm, n, ld_src, ld_dst, to_user);
+  launch(permute_kernel, grid, 256, 0, st, src, dst, perm, n, ld_src, ld_dst, to_user);
   return cudaGetLastError();
 }
 
@@ -5043,13 +5102,13 @@ cudaError_t launch_permute_u8(const uint8_t* src, uint8_t* dst, const int32_t* p
                               int64_t ld_src, int64_t ld_dst, int n_var, int to_user,
                               cudaStream_t st) {
   dim3 grid((unsigned)((n + 255) / 256), n_var);
-  permute_u8_kernel<<<grid, 256, 0, st>>>(src, dst, perm, n, ld_src, ld_dst, to_user);
+  launch(permute_u8_kernel, grid, 256, 0, st, src, dst, perm, n, ld_src, ld_dst, to_user);
   return cudaGetLastError();
 }
 
 cudaError_t launch_axpby(double* out, const double* a, double ca, const double* b, double cb,
                          int64_t n, cudaStream_t st) {
-  axpby_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(out, a, ca, b, cb, n);
+  launch(axpby_kernel, (unsigned)((n + 255) / 256), 256, 0, st, out, a, ca, b, cb, n);
   return cudaGetLastError();
 }
 
@@ -5094,11 +5153,11 @@ cudaError_t launch_face_flux_vjp(const DeviceMesh& dm, const void* Uq, const dou
     // all 2 NV directions of an interior face in one pass
     if constexpr (std::is_same<TQ, DF>::value) {
       constexpr int ND = NV < kVjpDirs ? NV : kVjpDirs;
-      face_flux_vjp_kernel<NV, NQ, FL, TQ, DF, ND><<<grid, 128, 0, st>>>(a, (const TQ*)Uq, w,
+      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, DF, ND>, grid, 128, 0, st, a, (const TQ*)Uq, w,
                                                                         Uq_bar);
     } else {
-      face_flux_vjp_kernel<NV, NQ, FL, TQ, double, 2 * NV><<<grid, 128, 0, st>>>(
-          a, (const TQ*)Uq, w, Uq_bar);
+      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, double, 2 * NV>, grid, 128, 0, st, a,
+             (const TQ*)Uq, w, Uq_bar);
     }
   };
   using I1 = std::integral_constant<int, 1>;
@@ -5138,12 +5197,12 @@ cudaError_t launch_recon_vjp(const DeviceMesh& dm, const uint8_t* sel, const dou
       dim3 block(kTile, NV, TZ);
       const unsigned grid = (unsigned)((tiles + TZ - 1) / TZ);
       if constexpr (std::is_same<TS, float2>::value)
-        recon_vjp_df_kernel<M, NS, NQ, NV><<<grid, block, 0, st>>>(
-            (const float2*)dm.ahat, sel, Uq_bar, (DF*)d_bar, u_self, dm.n_recon, dm.n_pad,
+        launch(recon_vjp_df_kernel<M, NS, NQ, NV>, grid, block, 0, st, (const float2*)dm.ahat, sel,
+               Uq_bar, (DF*)d_bar, u_self, dm.n_recon, dm.n_pad,
             dm.eval_df);
       else
-        recon_vjp_kernel<M, NS, NQ, NV, TS><<<grid, block, 0, st>>>(
-            (const TS*)dm.ahat, sel, Uq_bar, d_bar, u_self, dm.n_recon, dm.n_pad, dm.eval);
+        launch(recon_vjp_kernel<M, NS, NQ, NV, TS>, grid, block, 0, st, (const TS*)dm.ahat, sel,
+               Uq_bar, d_bar, u_self, dm.n_recon, dm.n_pad, dm.eval);
     };
     using I1 = std::integral_constant<int, 1>;
     using I4 = std::integral_constant<int, 4>;
@@ -5177,7 +5236,7 @@ cudaError_t launch_recon_vjp_tma_t(const DeviceMesh& dm, const uint8_t* sel, con
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int64_t tiles = (dm.n_recon + kTile - 1) / kTile;
   const int64_t grid = std::min<int64_t>(tiles, (int64_t)per_sm * sms);
-  kern<<<(unsigned)grid, threads, VP::kSmem, st>>>((const float2*)dm.ahat, dm.wq, dm.wstat,
+  launch(kern, (unsigned)grid, threads, VP::kSmem, st, (const float2*)dm.ahat, dm.wq, dm.wstat,
                                                    dm.halo, sel, Uq_bar, part, u_self, dm.n_recon, dm.n_pad,
                                                    dm.eval_df, dm.err_flag);
   return cudaGetLastError();
@@ -5204,17 +5263,17 @@ cudaError_t launch_scatter_gather(const DeviceMesh& dm, const int64_t* rev_off,
   const bool pairs = dm.precision == TENO_FP64;  // d_bar holds (hi, lo) pairs
   if (dm.n_var == 1) {
     if (pairs)
-      scatter_gather_kernel<1, DF><<<grid, 256, 0, st>>>(rev_off, rev_idx, (const DF*)d_bar,
+      launch(scatter_gather_kernel<1, DF>, grid, 256, 0, st, rev_off, rev_idx, (const DF*)d_bar,
                                                          u_self, v, dm.n_cell, dm.n_pad, ubd);
     else
-      scatter_gather_kernel<1, double><<<grid, 256, 0, st>>>(rev_off, rev_idx, d_bar, u_self, v,
+      launch(scatter_gather_kernel<1, double>, grid, 256, 0, st, rev_off, rev_idx, d_bar, u_self, v,
                                                              dm.n_cell, dm.n_pad, ubd);
   } else {
     if (pairs)
-      scatter_gather_kernel<4, DF><<<grid, 256, 0, st>>>(rev_off, rev_idx, (const DF*)d_bar,
+      launch(scatter_gather_kernel<4, DF>, grid, 256, 0, st, rev_off, rev_idx, (const DF*)d_bar,
                                                          u_self, v, dm.n_cell, dm.n_pad, ubd);
     else
-      scatter_gather_kernel<4, double><<<grid, 256, 0, st>>>(rev_off, rev_idx, d_bar, u_self, v,
+      launch(scatter_gather_kernel<4, double>, grid, 256, 0, st, rev_off, rev_idx, d_bar, u_self, v,
                                                              dm.n_cell, dm.n_pad, ubd);
   }
   return cudaGetLastError();
