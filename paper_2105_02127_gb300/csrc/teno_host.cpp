@@ -905,6 +905,9 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   // Euler TENO on the FP64 paths with the bulk-copy kernel (the W form)
   const bool wform = (store == TENO_FP64 || store == TENO_FP64_NATIVE) && p.n_var == 4 &&
                      p.recon_variant == 2 && p.scheme == 0 && p.charvar == 0;
+  // the tile kernel: TENO on the mixed path
+  const bool tileform = store == TENO_FP32_MIXED && p.recon_variant == 2 && p.scheme == 0 &&
+                        p.charvar == 0;
   // the global tiles whose cells are built: all of them, or those holding a
   // partition's compute set (every lane of such a tile, for its slot colouring)
   PartCells pc;
@@ -1316,8 +1319,9 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   bool halo_ok = true;
   std::vector<int32_t> hoff(ntile + 1, 0), hids;
   std::vector<uint16_t> hloc((size_t)ntile * SL * kTile, 0);
-  std::vector<int32_t> wtile(wform ? (size_t)ntile * kWTile : 0, 0);
-  std::vector<uint16_t> wpos(wform ? (size_t)ntile * SL * kTile : 0, 0);
+  const bool staged = wform || tileform;
+  std::vector<int32_t> wtile(staged ? (size_t)ntile * kWTile : 0, 0);
+  std::vector<uint16_t> wpos(staged ? (size_t)ntile * SL * kTile : 0, 0);
   {
     std::vector<int32_t> ids;
     for (int64_t t = 0; t < ntile && halo_ok; ++t) {
@@ -1340,9 +1344,9 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
           if (ln < nval)
             for (int j = 0; j < ln; ++j) rank += tn[(size_t)s * kTile + j] == tn[i];
           hloc[(size_t)t * SL * kTile + i] = (uint16_t)(pos | (rank << 8));
-          if (wform) wpos[(size_t)t * SL * kTile + i] = (uint16_t)(pos * 8);
+          if (staged) wpos[(size_t)t * SL * kTile + i] = (uint16_t)(pos * 8);
         }
-      if (wform) {
+      if (staged) {
         int32_t* tb = &wtile[(size_t)t * kWTile];
         tb[0] = (int32_t)ids.size();
         uint32_t held = 0;
@@ -1368,6 +1372,31 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
     std::vector<int64_t> pos(cnt.begin(), cnt.end() - 1);
     for (size_t i = 0; i < hids.size(); ++i) ctx->hrev_idx_h[pos[hids[i]]++] = (int32_t)i;
   }
+  // the tile kernel's matrices, in the place of the plain ones (which only
+  // the kernels of the other variants and of meshes without halos read)
+  const bool tile_on = tileform && halo_ok;
+  if (tile_on) {
+    const size_t tn = (size_t)E * kTile;
+    float* mat = reinterpret_cast<float*>(ahat.data());
+#pragma omp parallel
+    {
+      std::vector<float> src(tn);
+#pragma omp for schedule(static)
+      for (int64_t t = 0; t < ntile; ++t) {
+        float* out = mat + (size_t)t * tn;
+        std::copy(out, out + tn, src.begin());
+        for (int ln = 0; ln < kTile; ++ln) {
+          for (int s = 0; s < ns; ++s)
+            for (int l = 0; l < m; ++l)
+              out[tile_l_index(ns, m, s, l, ln)] = src[(size_t)(s * m + l) * kTile + ln];
+          for (int s = 0; s < kSmallK * kSmallN; ++s)
+            for (int l = 0; l < kSmallM; ++l)
+              out[tile_s_index(ns, m, s, l, ln)] =
+                  src[(size_t)(m * ns + s * kSmallM + l) * kTile + ln];
+        }
+      }
+    }
+  }
   int e = upload(ctx, ctx->b_ahat, ahat.data(), ahat.size());
   if (!e) e = upload(ctx, ctx->b_nbr, nbr.data(), nbr.size() * sizeof(int32_t));
   if (!e && halo_ok) e = upload(ctx, ctx->b_halo_off, hoff.data(), hoff.size() * 4);
@@ -1376,8 +1405,8 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   if (!e) e = upload(ctx, ctx->b_smask, smask.data(), smask.size());
   if (!e && wform) e = upload(ctx, ctx->b_g32, g32.data(), g32.size() * sizeof(float));
   if (!e && wform) e = upload(ctx, ctx->b_wq, wq.data(), wq.size() * sizeof(int2));
-  if (!e && wform && halo_ok) e = upload(ctx, ctx->b_wtile, wtile.data(), wtile.size() * 4);
-  if (!e && wform && halo_ok) e = upload(ctx, ctx->b_wpos, wpos.data(), wpos.size() * 2);
+  if (!e && staged && halo_ok) e = upload(ctx, ctx->b_wtile, wtile.data(), wtile.size() * 4);
+  if (!e && staged && halo_ok) e = upload(ctx, ctx->b_wpos, wpos.data(), wpos.size() * 2);
   if (!e && wform) e = upload(ctx, ctx->b_wstat, wstat.data(), wstat.size() * sizeof(int32_t));
   if (e) return e;
   // device mesh descriptor
@@ -1452,9 +1481,10 @@ int run_precompute(teno_ctx* ctx, int32_t n_parts = 1, int32_t part = 0) {
   dm.g32 = wform ? (const float*)ctx->b_g32.p : nullptr;
   dm.wq = wform ? (const int2*)ctx->b_wq.p : nullptr;
   dm.wstat = wform ? (const int32_t*)ctx->b_wstat.p : nullptr;
-  dm.wtile = wform && halo_ok ? (const int32_t*)ctx->b_wtile.p : nullptr;
-  dm.wpos = wform && halo_ok ? (const uint16_t*)ctx->b_wpos.p : nullptr;
+  dm.wtile = staged && halo_ok ? (const int32_t*)ctx->b_wtile.p : nullptr;
+  dm.wpos = staged && halo_ok ? (const uint16_t*)ctx->b_wpos.p : nullptr;
   if (wform) dm.wt = wb.table;
+  dm.tmat = tile_on ? ctx->b_ahat.p : nullptr;
   dm.nbr = (const int32_t*)ctx->b_nbr.p;
   dm.smask = (const uint8_t*)ctx->b_smask.p;
   std::copy(R.psi_t, R.psi_t + kMaxPts * kMaxM, dm.eval.psi);

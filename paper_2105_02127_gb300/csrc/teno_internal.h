@@ -72,6 +72,20 @@ struct WTable {
   float t[81], cs[12], cs_all;
 };
 
+// Tile kernel (TENO on the mixed path): large slots of a ring stage (5 to 8 KB;
+// a directional stencil is one stage), and the positions of an FP32 entry in a
+// tile's matrices, stage by stage in fours of 16 bytes a lane, the rest singly.
+TENO_HD constexpr int tile_lps(int ns) { return ns > 20 ? 3 : (ns > 12 ? 4 : 6); }
+TENO_HD constexpr int tile_l_index(int ns, int m, int s, int l, int lane) {
+  const int per = tile_lps(ns) * m, r = (s % tile_lps(ns)) * m + l;
+  return (s / tile_lps(ns)) * per * 32 +
+         (r < per / 4 * 4 ? ((r / 4) * 32 + lane) * 4 + r % 4 : r * 32 + lane);
+}
+TENO_HD constexpr int tile_s_index(int ns, int m, int slot, int l, int lane) {  // slot: 0 .. 35
+  const int r = (slot % 12) * 5 + l;
+  return (ns * m + (slot / 12) * 60) * 32 + ((r / 4) * 32 + lane) * 4 + r % 4;
+}
+
 // Per-tile stencil halo: the distinct cells of a tile's stencils (internal
 // ids, at most kHaloMax per tile) and the stencil slots as halo-local indices.
 constexpr int kHaloMax = 256;
@@ -136,6 +150,8 @@ struct DeviceMesh {
   const int32_t* wstat = nullptr;
   const int32_t* wtile = nullptr;
   const uint16_t* wpos = nullptr;
+  // tile kernel (else null): the FP32 matrices by tile_*_index
+  const void* tmat = nullptr;
   WTable wt{};
   const float2* psi_df = nullptr;   // device copy of eval_df.psi (pair W form)
   const double* psi_d = nullptr;    // device copy of eval.psi (native W form)

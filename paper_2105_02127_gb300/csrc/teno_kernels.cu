@@ -1626,28 +1626,6 @@ __device__ __forceinline__ void consumer_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(kConsumers * kTile) : "memory");
 }
 
-// Output stage of the TMA kernels.  Each variable warp writes its lanes'
-// Gauss-point values to shared memory laid out [cell][point][variable] with
-// an odd cell stride of kPer + 1 elements (conflict-free), and the consumer
-// threads then store the tile's contiguous block of Uq with coalesced writes
-// instead of one 32-sector store per point and variable.
-#ifndef TENO_STAGE_OUT
-#define TENO_STAGE_OUT 1
-#endif
-template <int kPer, typename TO>
-__device__ __forceinline__ void store_out_stage(const TO* stg, TO* __restrict__ dst, int nvalid,
-                                                int tid) {
-#pragma unroll 3
-  for (int e = tid; e < nvalid * kPer; e += kConsumers * kTile) {
-    const int cl = e / kPer;
-    dst[e] = stg[cl * (kPer + 1) + (e - cl * kPer)];
-  }
-}
-template <int kPer, typename TO>
-constexpr size_t out_stage_bytes() {
-  return ((size_t)kTile * (kPer + 1) * sizeof(TO) + 15) / 16 * 16;
-}
-
 // Stage j of a tile's matrix block: kLPS large-stencil slots, or kSPS slots of
 // one directional stencil.
 template <int M, int NS, int kEsz, int kLPS, int kSPS, int kRingT = kRing>
@@ -1690,21 +1668,6 @@ struct StagePlan {
   }
 };
 
-// Ring depth of the FP32-mixed bulk-copy reconstruction: 4 stages unless
-// they keep the kernel below four blocks per SM, then 3 (TENO6: 3 -> 4 blocks,
-// 7 % faster; TENO5 fits four blocks with 4 stages).  TENO_RING_MIXED > 0
-// overrides.
-#ifndef TENO_RING_MIXED
-#define TENO_RING_MIXED 0
-#endif
-template <int M, int NS, int NQ>
-struct MixedRing {
-  static constexpr size_t kBlock4 = StagePlan<M, NS, 4, 4, 4, 4>::kSmem +
-                                    (TENO_STAGE_OUT ? out_stage_bytes<3 * NQ * 4, float>() : 0) +
-                                    1024;
-  static constexpr int value =
-      TENO_RING_MIXED > 0 ? TENO_RING_MIXED : (4 * kBlock4 <= (size_t)228 * 1024 ? 4 : 3);
-};
 template <bool kDF, int M, int NS, int NQ>
 struct TmaTraits {
   using TE = float2;  // matrix entry: (hi, lo)
@@ -1715,7 +1678,7 @@ template <int M, int NS, int NQ>
 struct TmaTraits<false, M, NS, NQ> {
   using TE = float;
   using Acc = float;
-  static constexpr int kLPS = 4, kSPS = 4, kRing = MixedRing<M, NS, NQ>::value;
+  static constexpr int kLPS = 4, kSPS = 4, kRing = 4;
 };
 
 // Halo prefetch pipeline of the bulk-copy reconstruction kernels (consumer
@@ -1783,11 +1746,14 @@ struct HaloPipe {
 // the tile's stencil halo in a double-buffered shared-memory area, prefetched
 // with cp.async one tile ahead; stencil differences from the halo, matrices
 // from the ring.  kDF: FP64 path (double-float); !kDF: FP32-mixed path.
-// The pair kernel with the CWENO and characteristic branches (kDF && kExt)
-// is held to two blocks per SM: uncapped it took 252 registers at TENO6, one
-// block (five warps) per SM.
-template <int M, int NS, int NQ, bool kDF, bool kExt>
-__global__ void __launch_bounds__(kTile * (kConsumers + 1), (kDF && kExt) ? 2 : 0)
+// CWENO and the characteristic mode only (the other modes of variant 2 have
+// the W form and the tile kernel; with these modes' finish, which takes most of
+// the registers and of a tile's time, the tile kernel's form measured slower at
+// orders 5 and 6 on the pair path: 384 us against 490, 80,000 cells CWENO6).
+// The pair kernel is held to two blocks per SM: uncapped it took 252 registers
+// at TENO6, one block (five warps) per SM.
+template <int M, int NS, int NQ, bool kDF>
+__global__ void __launch_bounds__(kTile * (kConsumers + 1), kDF ? 2 : 0)
     recon_tma_kernel(const ReconArgs a, const HaloArgs h, const DFTable ev, int* err) {
   using TR = TmaTraits<kDF, M, NS, NQ>;
   using TE = typename TR::TE;
@@ -1795,13 +1761,8 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), (kDF && kExt) ? 2 : 
   using P = StagePlan<M, NS, (int)sizeof(TE), TR::kLPS, TR::kSPS, kRing>;
   constexpr int NV = 4;
   constexpr int SL = NS + kSmallSlots;
-  constexpr int kPer = 3 * NQ * NV;  // Gauss-point values per cell
-  // output stage on the FP32-mixed TENO path (the pair path would lose a
-  // block per SM to it)
-  constexpr bool kStage = TENO_STAGE_OUT && !kExt && !kDF;
   extern __shared__ __align__(128) unsigned char smem[];
   float2* halo = reinterpret_cast<float2*>(smem + (size_t)kRing * P::kMat);  // [2][NV][kHaloMax]
-  float* ostg = reinterpret_cast<float*>(smem + P::kSmem);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)kRing * P::kMat + P::kHaloBytes);
   uint64_t* empty = full + kRing;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + kRing);
@@ -1960,19 +1921,11 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), (kDF && kExt) ? 2 : 
         for (int k = 0; k < kSmallK; ++k)
 #pragma unroll
           for (int l = 0; l < kSmallM; ++l) as[k][l] = df_norm(as[k][l]);
-        df_finish<M, NQ, NV, kExt>(a, ev, c, v, acc, as, nullptr, present);
+        df_finish<M, NQ, NV, true>(a, ev, c, v, acc, as, nullptr, present);
       } else {
-        plain_finish<M, NQ, NV, float, DFTable, kExt>(a, ev, c, v, 0.0, u0s, acc, as,
-                                                      kStage ? ostg + lane * (kPer + 1) + v
-                                                             : nullptr,
+        plain_finish<M, NQ, NV, float, DFTable, true>(a, ev, c, v, 0.0, u0s, acc, as, nullptr,
                                                       present);
       }
-    }
-    if constexpr (kStage) {
-      consumer_sync();  // the tile's values are staged
-      if (!dead)
-        store_out_stage<kPer>(ostg, reinterpret_cast<float*>(a.Uq) + tile * kTile * kPer,
-                              (int)min((int64_t)kTile, a.n_cell - tile * kTile), tid);
     }
   }
   cp_async_wait<0>();
@@ -3039,6 +2992,277 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
   }
   cp_async_wait<0>();
   if (alive && n_def) w_deferred<M, NS, NQ, HT>(a, wa, mylist, n_def, dsc);
+}
+
+// ------------------------------------------- FP32-mixed TENO, tile kernel (variant 2)
+// The reconstruction of the mixed path, Euler and scalar: FP32 differences and
+// multiply-adds, slot by slot in stencil order.  The pipeline is the W form's: a
+// producer lane streams a tile's matrices in ring stages and its halo ids with
+// bulk copies; each consumer warp gathers its variables' halo states of the next
+// tile with cp.async and runs through its tiles without block barriers; four
+// matrix entries are read from shared memory at a time, and one read serves both
+// of an Euler warp's variables.
+// Bound: HBM at large meshes (0.71 GB a launch at 262,088 cells TENO5: 150 us,
+// 166 with one variable a warp and two block barriers a tile), the time of a
+// tile at small ones (1,152 cells: Euler TENO3 11.3 us, 12.8 before; scalar
+// TENO3, which read its matrices straight from global memory, 8.9 and 13.4).
+template <int M, int NS, int NQ, int NV>
+struct TPlan {
+  static constexpr int kVW = NV == 4 ? 2 : 1, kWarps = NV / kVW;  // variables a warp
+  static constexpr int kBlocks = NV == 1 ? 6 : 4;
+  static constexpr int kEsz = 4, kVec = 4;
+  static constexpr int kLPS = tile_lps(NS), kSPS = kSmallN;
+  static constexpr int kNL = NS / kLPS;
+  static constexpr int kStages = kSmallK + kNL;  // the directional stencils first
+  static constexpr int kEL = kLPS * M, kES = kSPS * kSmallM;    // entries of a stage, per lane
+  static constexpr int kLB = kEL * kTile * kEsz, kSB = kES * kTile * kEsz;
+  static constexpr int kSlotN = kTile * 2;  // halo offsets (uint16) of one slot
+  static constexpr int kNOff = kLB > kSB ? kLB : kSB;
+  static constexpr int kMaxSlots = kLPS > kSPS ? kLPS : kSPS;
+  static constexpr int kBuf = kNOff + kMaxSlots * kSlotN;
+  static constexpr int64_t kTileMat = (int64_t)(M * NS + kSmallEntries) * kTile * kEsz;
+  static constexpr int kSL = NS + kSmallSlots;
+  static constexpr int kTileBytes = kWTile * 4;
+  static constexpr int kHaloRow = kHaloMax + kTile;  // halo states, then the tile's own
+  static constexpr int kHalo = 2 * NV * kHaloRow * 8;
+  // Euler: a warp's Gauss values [cell][point][variable], odd row
+  static constexpr int kOutRow = 3 * NQ * kVW + 1;
+  static constexpr int kOut = NV == 4 ? kWarps * kTile * kOutRow * 4 : 0;
+  static constexpr int kFixed = kHalo + 2 * kTileBytes + kOut + 16 * 8 + 16;
+  static constexpr int kRoom = (227 * 1024 / kBlocks - 1024 - kFixed) / kBuf;
+  static constexpr int kRing = kRoom < 2 ? 2 : (kRoom > 5 ? 5 : kRoom);
+  static constexpr size_t kSmem = (size_t)kRing * kBuf + kFixed;
+  static_assert(NS % kLPS == 0, "whole stages");
+  static_assert(kBuf % 16 == 0 && kNOff % 16 == 0 && kLB % 16 == 0 && kSB % 16 == 0 &&
+                    kOut % 16 == 0,
+                "bulk-copy alignment");
+};
+
+template <int M, int NS, int NQ, int NV>
+__global__ void __launch_bounds__(kTile*(TPlan<M, NS, NQ, NV>::kWarps + 1),
+                                  (TPlan<M, NS, NQ, NV>::kBlocks))
+    recon_tile_kernel(const ReconArgs a, const uint16_t* __restrict__ pos,
+                      const int32_t* __restrict__ tiles, const DFTable ev, int* err) {
+  using P = TPlan<M, NS, NQ, NV>;
+  using St = float2;  // halo states: the (hi, lo) split
+  constexpr int kR = P::kRing, kVW = P::kVW, kWarps = P::kWarps, NQ3 = 3 * NQ;
+  extern __shared__ __align__(128) unsigned char smem[];
+  St* halo = reinterpret_cast<St*>(smem + (size_t)kR * P::kBuf);            // [2][NV][kHaloRow]
+  int32_t* tblk = reinterpret_cast<int32_t*>(halo + 2 * NV * P::kHaloRow);  // [2][kWTile]
+  float* ostg = reinterpret_cast<float*>(tblk + 2 * kWTile);                // [kWarps][32][kOutRow]
+  uint64_t* full = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(ostg) + P::kOut);
+  uint64_t* empty = full + kR;
+  uint64_t* tfull = empty + kR;
+  uint64_t* tempty = tfull + 2;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(full + 16);
+  static_assert(2 * kR + 4 <= 16, "mbarriers");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t n_tiles = (a.n_cell + kTile - 1) / kTile;
+  if (threadIdx.x == 0) {
+    *abort_flag = 0;
+    for (int i = 0; i < kR; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], kWarps);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], kWarps);
+    }
+    mbar_fence_init();
+  }
+  __syncthreads();
+  if (warp == kWarps) {
+    // ---- producer lane
+    if (lane == 0) {
+      RingPos<kR> rp;
+      bool lap = false;  // every buffer has been filled once
+      int it = 0;
+      // the block must not exit while a copy it issued is in flight: the last
+      // kR stages (buffers before rp.b are one phase ahead) and id blocks
+      auto drain = [&](int n_blk) {
+        for (int b = 0; b < kR; ++b)
+          if (b < rp.b || lap) mbar_wait(&full[b], b < rp.b ? rp.ph : rp.ph ^ 1);
+        for (int i = n_blk > 2 ? n_blk - 2 : 0; i < n_blk; ++i)
+          mbar_wait(&tfull[i & 1], (uint32_t)(i >> 1) & 1);
+      };
+      auto gave_up = [&](int w, int n_blk) {
+        if (w == 0) {
+          atomicOr(err, 2);
+          *abort_flag = 1;
+        }
+        drain(n_blk);
+      };
+      auto block = [&](int64_t tile, int i) {
+        mbar_expect_tx(&tfull[i & 1], P::kTileBytes);
+        bulk_g2s(tblk + (i & 1) * kWTile, tiles + tile * kWTile, P::kTileBytes, &tfull[i & 1]);
+      };
+      int n_blk = 0;  // halo-id blocks issued
+      for (; n_blk < 2 && blockIdx.x + (int64_t)n_blk * gridDim.x < n_tiles; ++n_blk)
+        block(blockIdx.x + (int64_t)n_blk * gridDim.x, n_blk);
+      for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+        const unsigned char* sa = reinterpret_cast<const unsigned char*>(a.ahat) + tile * P::kTileMat;
+        const unsigned char* sn =
+            reinterpret_cast<const unsigned char*>(pos) + tile * (int64_t)P::kSL * P::kSlotN;
+        for (int j = 0; j < P::kStages; ++j) {
+          const int b = rp.b;
+          if (lap) {
+            const int w = mbar_wait_or_abort(&empty[b], rp.ph ^ 1, abort_flag);
+            if (w != 1) return gave_up(w, n_blk);
+          }
+          unsigned char* dst = smem + b * P::kBuf;
+          const int js = j - kSmallK;  // large stage
+          const unsigned char* src = js < 0 ? sa + P::kNL * P::kLB + j * P::kSB : sa + js * P::kLB;
+          const int bytes = js < 0 ? P::kSB : P::kLB;
+          const int slot = js < 0 ? NS + j * P::kSPS : js * P::kLPS;
+          const int nslot = js < 0 ? P::kSPS : P::kLPS;
+          mbar_expect_tx(&full[b], bytes + nslot * P::kSlotN);
+          bulk_g2s(dst, src, bytes, &full[b]);
+          bulk_g2s(dst + P::kNOff, sn + slot * P::kSlotN, nslot * P::kSlotN, &full[b]);
+          rp.next();
+          lap |= rp.b == 0;
+        }
+        const int64_t nxt = tile + 2 * (int64_t)gridDim.x;
+        if (nxt < n_tiles) {
+          const int w = mbar_wait_or_abort(&tempty[it & 1], (uint32_t)(it >> 1) & 1, abort_flag);
+          if (w != 1) return gave_up(w, n_blk);
+          block(nxt, n_blk++);
+        }
+      }
+      drain(n_blk);
+    }
+    return;
+  }
+  // ---- consumers (warp w: kVW variables from kVW w)
+  pdl_wait();  // the states (the producer streams constant data before it)
+  constexpr int kPerLane = kHaloMax / kTile;
+  const int v0 = warp * kVW;
+  int it = 0;
+  RingPos<kR> rp;
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    const int w = mbar_wait_or_abort(bar, parity, abort_flag, a.wait_polls);
+    if (w == 0) {
+      atomicOr(err, 2);
+      *abort_flag = 1;
+    }
+    return !__any_sync(0xffffffffu, w != 1);
+  };
+  auto gather = [&](int64_t tile, int i) {
+    bool ok = true;
+    if (tile < n_tiles) {
+      ok = wait(&tfull[i & 1], (uint32_t)(i >> 1) & 1);
+      if (ok) {
+        const int32_t* tb = tblk + (i & 1) * kWTile;
+        const St* src = a.Us + (int64_t)v0 * a.n_pad;
+        St* dst = halo + ((i & 1) * NV + v0) * P::kHaloRow;
+        const int H = tb[0];
+#pragma unroll
+        for (int k = 0; k < kPerLane; ++k)
+          if (lane + k * kTile < H) {
+            const int id = tb[4 + lane + k * kTile];
+#pragma unroll
+            for (int w = 0; w < kVW; ++w)
+              cp_async8(dst + w * P::kHaloRow + lane + k * kTile, src + w * a.n_pad + id);
+          }
+        const int64_t c = tile * kTile + lane;
+#pragma unroll
+        for (int w = 0; w < kVW; ++w)
+          cp_async8(dst + w * P::kHaloRow + kHaloMax + lane,
+                    src + w * a.n_pad + (c < a.n_cell ? c : 0));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[i & 1]);
+      }
+    }
+    cp_async_commit();
+    return ok;
+  };
+  if (!gather(blockIdx.x, 0)) {
+    cp_async_wait<0>();
+    return;
+  }
+  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+    const int64_t c = tile * kTile + lane;  // may be a pad lane of the last tile
+    __syncwarp();  // every lane is done with the other halo buffer
+    if (!gather(tile + gridDim.x, it + 1)) break;
+    const int present = a.smask[c < a.n_cell ? c : 0];
+    cp_async_wait<1>();
+    __syncwarp();
+    St* hv = halo + ((it & 1) * NV + v0) * P::kHaloRow;
+    float2 u0s[kVW];
+#pragma unroll
+    for (int w = 0; w < kVW; ++w) u0s[w] = hv[w * P::kHaloRow + kHaloMax + lane];
+    const unsigned char* st = reinterpret_cast<const unsigned char*>(hv);
+    auto dif = [&](int w, int off) {
+      const float2 x = *reinterpret_cast<const float2*>(st + w * (P::kHaloRow * 8) + off);
+      return (x.x - u0s[w].x) + (x.y - u0s[w].y);
+    };
+    // one stage's products: entries e = slot * kRows + l of the buffer
+    auto stage = [&](auto nslots, auto rows, const unsigned char* buf, auto& acc) {
+      constexpr int kS = decltype(nslots)::value, kRows = decltype(rows)::value, kN = kS * kRows;
+      const uint16_t* nl = reinterpret_cast<const uint16_t*>(buf + P::kNOff) + lane;
+      float d[kVW][kS];
+#pragma unroll
+      for (int s = 0; s < kS; ++s) {
+        const int off = nl[s * kTile];
+#pragma unroll
+        for (int w = 0; w < kVW; ++w) d[w][s] = dif(w, off);
+      }
+#pragma unroll
+      for (int e = 0; e < kN; ++e) {
+        const float m = g_entry<kN>(buf, lane, e);
+#pragma unroll
+        for (int w = 0; w < kVW; ++w) acc[w][e % kRows] = fmaf(m, d[w][e / kRows], acc[w][e % kRows]);
+      }
+    };
+    float as[kSmallK][kVW][kSmallM] = {}, acc[kVW][M] = {};
+    bool alive = true;
+#pragma unroll
+    for (int k = 0; alive && k < kSmallK; ++k) {
+      if (!(alive = wait(&full[rp.b], rp.ph))) break;
+      stage(std::integral_constant<int, P::kSPS>{}, std::integral_constant<int, kSmallM>{},
+            smem + rp.b * P::kBuf, as[k]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[rp.b]);
+      rp.next();
+    }
+#pragma unroll 1
+    for (int j = 0; alive && j < P::kNL; ++j) {
+      if (!(alive = wait(&full[rp.b], rp.ph))) break;
+      stage(std::integral_constant<int, P::kLPS>{}, std::integral_constant<int, M>{},
+            smem + rp.b * P::kBuf, acc);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[rp.b]);
+      rp.next();
+    }
+    if (!alive) break;
+    // ---- selection and Gauss-point values
+    if (c < a.n_cell) {
+#pragma unroll
+      for (int w = 0; w < kVW; ++w) {
+        float aw[kSmallK][kSmallM];
+#pragma unroll
+        for (int k = 0; k < kSmallK; ++k)
+#pragma unroll
+          for (int l = 0; l < kSmallM; ++l) aw[k][l] = as[k][w][l];
+        plain_finish<M, NQ, kVW, float, DFTable, false>(
+            a, ev, c, v0 + w, 0.0, u0s[w], acc[w], aw,
+            NV == 4 ? ostg + (warp * kTile + lane) * P::kOutRow + w : nullptr, present);
+      }
+    }
+    // Euler: the warp's values, staged, in rows of consecutive cells
+    if constexpr (P::kOut > 0) {
+      __syncwarp();
+      const int n = (int)min((int64_t)kTile, a.n_cell - tile * kTile) * NQ3;
+      const float* o = ostg + warp * kTile * P::kOutRow;
+      float* dst = reinterpret_cast<float*>(a.Uq) + tile * kTile * (NQ3 * NV) + v0;
+#pragma unroll 3
+      for (int e = lane; e < n; e += kTile) {
+        const float* q = o + e / NQ3 * P::kOutRow + e % NQ3 * kVW;
+        *reinterpret_cast<float2*>(dst + e * NV) = make_float2(q[0], q[1]);
+      }
+      __syncwarp();
+    }
+  }
+  cp_async_wait<0>();
 }
 
 // ------------------------------------ characteristic variables (charvar)
@@ -4712,16 +4936,11 @@ void launch(void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
-template <int M, int NS, int NQ, bool kDF, bool kExt>
-cudaError_t launch_recon_tma(const ReconArgs& a, const DeviceMesh& dm, int* err, cudaStream_t st) {
-  using TR = TmaTraits<kDF, M, NS, NQ>;
-  using P = StagePlan<M, NS, (int)sizeof(typename TR::TE), TR::kLPS, TR::kSPS, TR::kRing>;
-  auto kern = recon_tma_kernel<M, NS, NQ, kDF, kExt>;
-  const int threads = kTile * (kConsumers + 1);
-  constexpr bool kStage = TENO_STAGE_OUT && !kExt && !kDF;
-  const size_t smem = P::kSmem + (kStage ? out_stage_bytes<3 * NQ * 4, float>() : 0);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+// blocks of a persistent kernel: what is resident, at most one per tile
+template <typename K>
+cudaError_t resident_grid(K kern, int threads, size_t smem, int64_t tiles, unsigned* grid) {
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -4731,9 +4950,36 @@ cudaError_t launch_recon_tma(const ReconArgs& a, const DeviceMesh& dm, int* err,
       cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int64_t tiles = (a.n_cell + kTile - 1) / kTile;
-  const int64_t grid = std::min<int64_t>(tiles, (int64_t)per_sm * sms);
-  launch(kern, (unsigned)grid, threads, smem, st, a, dm.halo, dm.eval_df, err);
+  *grid = (unsigned)std::min<int64_t>(tiles, (int64_t)per_sm * sms);
+  return cudaSuccess;
+}
+
+template <int M, int NS, int NQ, int NV>
+cudaError_t launch_recon_tile(const ReconArgs& a, const DeviceMesh& dm, cudaStream_t st) {
+  using P = TPlan<M, NS, NQ, NV>;
+  auto kern = recon_tile_kernel<M, NS, NQ, NV>;
+  const int threads = kTile * (P::kWarps + 1);
+  unsigned grid = 0;
+  const cudaError_t e =
+      resident_grid(kern, threads, P::kSmem, (a.n_cell + kTile - 1) / kTile, &grid);
+  if (e != cudaSuccess) return e;
+  ReconArgs b = a;
+  b.ahat = dm.tmat;
+  launch(kern, grid, threads, P::kSmem, st, b, dm.wpos, dm.wtile, dm.eval_df, dm.err_flag);
+  return cudaGetLastError();
+}
+
+template <int M, int NS, int NQ, bool kDF>
+cudaError_t launch_recon_tma(const ReconArgs& a, const DeviceMesh& dm, cudaStream_t st) {
+  using TR = TmaTraits<kDF, M, NS, NQ>;
+  using P = StagePlan<M, NS, (int)sizeof(typename TR::TE), TR::kLPS, TR::kSPS, TR::kRing>;
+  auto kern = recon_tma_kernel<M, NS, NQ, kDF>;
+  const int threads = kTile * (kConsumers + 1);
+  unsigned grid = 0;
+  const cudaError_t e =
+      resident_grid(kern, threads, P::kSmem, (a.n_cell + kTile - 1) / kTile, &grid);
+  if (e != cudaSuccess) return e;
+  launch(kern, grid, threads, P::kSmem, st, a, dm.halo, dm.eval_df, dm.err_flag);
   return cudaGetLastError();
 }
 
@@ -4743,19 +4989,10 @@ cudaError_t launch_recon_tma_w(const ReconArgs& a, const DeviceMesh& dm, int* er
   using P = WPlan<M, NS, 3 * NQ, HT>;
   auto kern = recon_tma_w_kernel<M, NS, NQ, HT>;
   const int threads = kTile * (P::kWWarps + 1);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)P::kSmem);
+  unsigned grid = 0;
+  const cudaError_t e =
+      resident_grid(kern, threads, P::kSmem, (a.n_cell + kTile - 1) / kTile, &grid);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-    return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, P::kSmem)) !=
-      cudaSuccess)
-    return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int64_t tiles = (a.n_cell + kTile - 1) / kTile;
-  const int64_t grid = std::min<int64_t>(tiles, (int64_t)per_sm * sms);
   WArgs wa;
   wa.psi = std::is_same<HT, double>::value ? (const void*)dm.psi_d : (const void*)dm.psi_df;
   wa.g32 = dm.g32;
@@ -4764,7 +5001,7 @@ cudaError_t launch_recon_tma_w(const ReconArgs& a, const DeviceMesh& dm, int* er
   wa.tile = dm.wtile;
   wa.st = dm.wstat;
   wa.t = dm.wt;
-  launch(kern, (unsigned)grid, threads, P::kSmem, st, a, wa, err);
+  launch(kern, grid, threads, P::kSmem, st, a, wa, err);
   return cudaGetLastError();
 }
 
@@ -4822,20 +5059,26 @@ cudaError_t launch_recon(const DeviceMesh& dm, const double* U, const float2* Us
     constexpr int M = decltype(Mc)::value, NS = decltype(NSc)::value;
     auto go = [&](auto nqc, auto nvc) -> cudaError_t {
       constexpr int NQ = decltype(nqc)::value, NV = decltype(nvc)::value;
-      // the TMA kernel covers Euler on the pair and mixed paths; variant 2
-      // elsewhere takes the halo kernel. CWENO and the characteristic mode
-      // take the TMA or the direct kernels: the halo kernel is compiled for
-      // TENO in conservative variables only.
+      // variant 2 where every tile has its halo: the W form (Euler TENO in FP64
+      // and pairs), the tile kernel (dm.tmat: TENO on the mixed path, scalar
+      // too), and on Euler's mixed and pair paths the bulk-copy kernel of CWENO
+      // and the characteristic mode.  What is left of variant 2 (scalar FP64
+      // and pairs) takes the halo kernel, compiled for TENO in conservative
+      // variables only, or the direct kernels.
       const bool ext = dm.scheme != 0 || dm.charvar != 0;
-      // the native FP64 path has the W-form kernel only (no pair TMA kernel)
-      const bool wn = NV == 4 && dm.variant == 2 && dm.err_flag && dm.halo.off && !ext &&
-                      dm.precision == TENO_FP64_NATIVE && dm.g32 && dm.wq && dm.psi_d;
-      if constexpr (NV == 4) {
-        if (wn) return launch_recon_tma_w<M, NS, NQ, double>(a, dm, dm.err_flag, st);
+      if (dm.variant == 2 && dm.err_flag && dm.halo.off) {
+        if (dm.tmat) return launch_recon_tile<M, NS, NQ, NV>(a, dm, st);
+        if constexpr (NV == 4) {
+          if (dm.wq && dm.psi_d)
+            return launch_recon_tma_w<M, NS, NQ, double>(a, dm, dm.err_flag, st);
+          if (dm.wq && dm.psi_df)
+            return launch_recon_tma_w<M, NS, NQ, float2>(a, dm, dm.err_flag, st);
+          if (ext && dm.precision == TENO_FP64) return launch_recon_tma<M, NS, NQ, true>(a, dm, st);
+          if (ext && dm.precision == TENO_FP32_MIXED)
+            return launch_recon_tma<M, NS, NQ, false>(a, dm, st);
+        }
       }
-      const bool tma = NV == 4 && dm.variant == 2 && dm.err_flag && dm.halo.off &&
-                       dm.precision != TENO_FP64_NATIVE;
-      if (!ext && (dm.variant == 0 || (dm.variant == 2 && !tma)) && dm.halo.off) {
+      if (!ext && dm.variant != 1 && dm.halo.off) {
         constexpr int TZh = 4 / NV;
         dim3 block(kTile, NV, TZh);
         dim3 grid((unsigned)((tiles + TZh - 1) / TZh));
@@ -4846,20 +5089,6 @@ cudaError_t launch_recon(const DeviceMesh& dm, const double* U, const float2* Us
         else
           launch(recon_halo_kernel<M, NS, NQ, NV, 2>, grid, block, 0, st, a, dm.halo, dm.eval);
         return cudaGetLastError();
-      }
-      if constexpr (NV == 4) {
-        if (tma) {
-          if (dm.precision == TENO_FP64 && dm.scheme == 0 && dm.g32 && dm.wq && dm.psi_df)
-            return launch_recon_tma_w<M, NS, NQ, float2>(a, dm, dm.err_flag, st);
-          if (ext) {
-            if (dm.precision == TENO_FP64)
-              return launch_recon_tma<M, NS, NQ, true, true>(a, dm, dm.err_flag, st);
-            return launch_recon_tma<M, NS, NQ, false, true>(a, dm, dm.err_flag, st);
-          }
-          if (dm.precision == TENO_FP64)
-            return launch_recon_tma<M, NS, NQ, true, false>(a, dm, dm.err_flag, st);
-          return launch_recon_tma<M, NS, NQ, false, false>(a, dm, dm.err_flag, st);
-        }
       }
       constexpr int TZ = 4 / NV;  // 128 threads per block
       dim3 block(kTile, NV, TZ);
