@@ -4143,39 +4143,44 @@ __device__ __forceinline__ void store_bar(double* base, int i, S x) {
     base[i] = to_d(x);
 }
 
-// minimum resident blocks of 128 threads per SM for the flux VJP (3: 168
-// registers, measured 13 % faster than no cap; 0: no cap)
-#ifndef TENO_VJP_MIN_BLOCKS
-#define TENO_VJP_MIN_BLOCKS 3
-#endif
+// One thread per (face, Gauss point), 64 faces a block; the faces' cotangents
+// are formed once and shared.  Bound: FP32 issue (pairs) at 168 registers, the
+// latency of one reverse sweep at small meshes, where a thread that took a
+// face's points in turn ran three in a row
+// (8,320 cells TENO6, HLLC: 136 us a residual's adjoint, 122 now).
 template <int NV, int NQ, int FLUX, typename TQ, typename S, int ND>
-__global__ void __launch_bounds__(128, TENO_VJP_MIN_BLOCKS > 0 ? TENO_VJP_MIN_BLOCKS : 1)
-    face_flux_vjp_kernel(const VjpArgs a,
-                                                            const TQ* Uq,
-                                                            const double* w,
-                                                            double* __restrict__ Uq_bar) {
+__global__ void __launch_bounds__(kFluxFaces * NQ, 384 / (kFluxFaces * NQ))
+    face_flux_vjp_kernel(const VjpArgs a, const TQ* Uq, const double* w,
+                         double* __restrict__ Uq_bar) {
   pdl_wait();
   static_assert((2 * NV) % ND == 0, "directions per pass must divide 2 NV");
   using D = Dual<ND, S>;
-  const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ S sK[kFluxFaces * NV];
+  const int64_t f0 = (int64_t)blockIdx.x * kFluxFaces;
+  // Kbar in FP64 from the FP64 weights, once per face in the flux scalar type
+  for (int e = threadIdx.x; e < kFluxFaces * NV; e += kFluxFaces * NQ) {
+    const int64_t f = f0 + e % kFluxFaces;
+    const int v = e / kFluxFaces;
+    if (f >= a.n_face) continue;
+    const int o = a.f_cells[2 * f], n = a.f_cells[2 * f + 1];
+    double kb = -w[v * a.n_pad + o] * a.inv_area[o];
+    if (n >= 0) kb = fma(w[v * a.n_pad + n], a.inv_area[n], kb);
+    sK[e % kFluxFaces * NV + v] = cst<S>(kb);
+  }
+  __syncthreads();
+  const int k = threadIdx.x % NQ;
+  const int64_t f = f0 + threadIdx.x / NQ;
   if (f >= a.n_face) return;
   const int o = a.f_cells[2 * f], n = a.f_cells[2 * f + 1];
   const int eo = a.f_edges[2 * f], en = a.f_edges[2 * f + 1];
   const double nx = a.f_geom[5 * f], ny = a.f_geom[5 * f + 1], len = a.f_geom[5 * f + 2];
-  // Kbar in FP64 from the FP64 weights, once per face in the flux scalar type
-  S Kb[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    double kb = -w[v * a.n_pad + o] * a.inv_area[o];
-    if (n >= 0) kb = fma(w[v * a.n_pad + n], a.inv_area[n], kb);
-    Kb[v] = cst<S>(kb);
-  }
+  const S* Kb = sK + threadIdx.x / NQ * NV;
   const int n_pass = ((n >= 0 ? 2 * NV : NV) + ND - 1) / ND;
   RiemannK<S> rks;
   S tl;  // |A| in the flux scalar type
   face_k<S>(a.f_geom, a.f_geom2, f, a.gamma, a.g2, a.gm12, rks, tl);
   const RiemannK<D> rk = riemann_k_dual<ND, S>(rks);
-  for (int k = 0; k < NQ; ++k) {
+  {
     TQ ul[NV], ur[NV];
     ld_group<NV>(Uq + ((int64_t)(o * 3 + eo) * NQ + k) * NV, ul);
     if (n >= 0) ld_group<NV>(Uq + ((int64_t)(n * 3 + en) * NQ + (NQ - 1 - k)) * NV, ur);
@@ -5373,7 +5378,7 @@ cudaError_t launch_face_flux_vjp(const DeviceMesh& dm, const void* Uq, const dou
     a.gt[k] = dm.gt[k];
     a.gw2[k] = split2(dm.gw[k]);
   }
-  const unsigned grid = (unsigned)((dm.n_face + 127) / 128);
+  const unsigned grid = (unsigned)((dm.n_face + kFluxFaces - 1) / kFluxFaces);
   auto go = [&](auto nvc, auto nqc, auto flc, auto tqc) {
     constexpr int NV = decltype(nvc)::value, NQ = decltype(nqc)::value,
                   FL = decltype(flc)::value;
@@ -5382,10 +5387,10 @@ cudaError_t launch_face_flux_vjp(const DeviceMesh& dm, const void* Uq, const dou
     // all 2 NV directions of an interior face in one pass
     if constexpr (std::is_same<TQ, DF>::value) {
       constexpr int ND = NV < kVjpDirs ? NV : kVjpDirs;
-      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, DF, ND>, grid, 128, 0, st, a, (const TQ*)Uq, w,
-                                                                        Uq_bar);
+      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, DF, ND>, grid, kFluxFaces * NQ, 0, st, a,
+             (const TQ*)Uq, w, Uq_bar);
     } else {
-      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, double, 2 * NV>, grid, 128, 0, st, a,
+      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, double, 2 * NV>, grid, kFluxFaces * NQ, 0, st, a,
              (const TQ*)Uq, w, Uq_bar);
     }
   };
