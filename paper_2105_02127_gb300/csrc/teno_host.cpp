@@ -1913,13 +1913,15 @@ int vjp_internal(teno_ctx* ctx, const double* U, const double* w, double* v, dou
 // its output, which the next stage's reconstruction reads)
 int rk_stage(teno_ctx* ctx, const double* Un, const double* Us, double* out, double cn,
              double cs, double dt, const double* max_lam, double time, bool split_ready,
-             void* uq = nullptr, uint8_t* sel_out = nullptr) {
+             void* uq = nullptr, uint8_t* sel_out = nullptr, double* lam_next = nullptr,
+             double* lam_zero = nullptr) {
   int rc = stage_flux(ctx, Us, sel_out, time, split_ready, uq);
   if (rc) return rc;
   const bool split = ctx->prm.precision != TENO_FP64_NATIVE;
   long pe = prof_begin(ctx, K_GATHER);
   CK(launch_gather(ctx->dm, ctx->b_K.p, Un, Us, out, 1, cn, cs, dt, max_lam,
-                   (int*)ctx->b_flag.p, split ? (float2*)ctx->b_Usplit.p : nullptr, ctx->stream),
+                   (int*)ctx->b_flag.p, split ? (float2*)ctx->b_Usplit.p : nullptr, lam_next, lam_zero,
+                   ctx->stream),
      "gather launch");
   prof_end(ctx, pe);
   return TENO_OK;
@@ -2210,7 +2212,7 @@ int teno_residual(teno_ctx* ctx, double* R, uint8_t* sel, int on_device) {
                   ctx->split_ok);
   if (rc) return rc;
   CK(launch_gather(ctx->dm, ctx->b_K.p, nullptr, nullptr, (double*)ctx->b_R.p, 0, 0, 0, 0,
-                   nullptr, nullptr, nullptr, ctx->stream),
+                   nullptr, nullptr, nullptr, nullptr, nullptr, ctx->stream),
      "gather launch");
   if (sel) {
     const uint8_t* src = ctx->override_on ? (const uint8_t*)ctx->b_sel_ovr.p
@@ -2274,34 +2276,42 @@ int teno_cfl_dt(teno_ctx* ctx, double* dt) {
   return TENO_OK;
 }
 
-static int rk3_once(teno_ctx* ctx, double dt, double* dt_used) {
+// One step.  On the device CFL path (dt <= 0 without a host step) slot: where
+// its maximum lies (0 or 1), reduced here unless ready; next: the last stage
+// reduces the following step's into the other slot.
+static int rk3_once(teno_ctx* ctx, double dt, double* dt_used, int slot = 0, bool ready = false,
+                    bool next = false) {
+  double* lam = (double*)ctx->b_maxlam.p;
   const double* maxlam = nullptr;
   if (dt <= 0.0) {
     if (dt_used || ctx->has_time_bc) {
       int rc = teno_cfl_dt(ctx, &dt);
       if (rc) return rc;
-    } else {
+    } else if (!ready) {
       long pe = prof_begin(ctx, K_CFL);
       // from the (hi, lo) split of U where the FP64 or mixed path holds it
       if (ctx->split_ok && ctx->prm.n_var == 4 && ctx->prm.precision != TENO_FP64_NATIVE)
-        CK(launch_max_lambda_split(ctx->dm, (const float2*)ctx->b_Usplit.p,
-                                   (double*)ctx->b_maxlam.p, ctx->stream),
+        CK(launch_max_lambda_split(ctx->dm, (const float2*)ctx->b_Usplit.p, lam + slot,
+                                   ctx->stream),
            "max lambda launch");
       else
-        CK(launch_max_lambda(ctx->dm, (const double*)ctx->b_U.p, (double*)ctx->b_maxlam.p,
-                             ctx->stream),
+        CK(launch_max_lambda(ctx->dm, (const double*)ctx->b_U.p, lam + slot, ctx->stream),
            "max lambda launch");
       prof_end(ctx, pe);
-      maxlam = (const double*)ctx->b_maxlam.p;
     }
+    if (dt <= 0.0) maxlam = lam + slot;
   }
   double* U = (double*)ctx->b_U.p;
   double* U1 = (double*)ctx->b_U1.p;
   double* U2 = (double*)ctx->b_U2.p;
   const double t = ctx->time;
-  int rc = rk_stage(ctx, U, U, U1, 0.0, 1.0, dt, maxlam, t, ctx->split_ok);
+  double* nxt = next && maxlam ? lam + (slot ^ 1) : nullptr;
+  int rc = rk_stage(ctx, U, U, U1, 0.0, 1.0, dt, maxlam, t, ctx->split_ok, nullptr, nullptr,
+                    nullptr, nxt);
   if (!rc) rc = rk_stage(ctx, U, U1, U2, 0.75, 0.25, dt, maxlam, t + dt, true);
-  if (!rc) rc = rk_stage(ctx, U, U2, U, 1.0 / 3.0, 2.0 / 3.0, dt, maxlam, t + 0.5 * dt, true);
+  if (!rc)
+    rc = rk_stage(ctx, U, U2, U, 1.0 / 3.0, 2.0 / 3.0, dt, maxlam, t + 0.5 * dt, true, nullptr,
+                  nullptr, nxt);
   ctx->split_ok = ctx->prm.precision != TENO_FP64_NATIVE;
   if (rc) return rc;
   ctx->stages_ok = true;
@@ -2337,7 +2347,9 @@ int teno_rk3_steps(teno_ctx* ctx, int32_t n_steps, double dt) {
     return fail(ctx, TENO_EINVAL,
                 "partition: step with teno_group_rk3_step, or teno_rk3_stage and halo exchanges");
   if (n_steps < 0) return fail(ctx, TENO_EINVAL, "rk3_steps: negative count");
-  for (int32_t i = 0; i < n_steps && !rc; ++i) rc = rk3_once(ctx, dt, nullptr);
+  const bool dev_cfl = dt <= 0.0 && !ctx->has_time_bc;
+  for (int32_t i = 0; i < n_steps && !rc; ++i)
+    rc = rk3_once(ctx, dt, nullptr, i & 1, dev_cfl && i > 0, dev_cfl && i + 1 < n_steps);
   return rc;
 }
 

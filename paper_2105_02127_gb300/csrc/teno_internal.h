@@ -192,10 +192,13 @@ cudaError_t launch_layer_fill(const DeviceMesh& dm, const double* U, void* Uq, c
 cudaError_t launch_face_flux(const DeviceMesh& dm, const void* Uq, void* K, double time,
                              cudaStream_t st);
 // mode 0: R = residual; mode 1: U_out = cn*Un + cs*(Us + dt*R), and (split
-// non-null) the FP32 hi/lo split of U_out
+// non-null) the FP32 hi/lo split of U_out; lam_next (or null): the CFL maximum
+// over U_out is merged into it, as launch_max_lambda(_split) forms it; lam_zero
+// (or null): cleared
 cudaError_t launch_gather(const DeviceMesh& dm, const void* K, const double* Un, const double* Us,
                           double* out, int mode, double cn, double cs, double dt_fixed,
-                          const double* max_lam, int* flag, float2* split, cudaStream_t st);
+                          const double* max_lam, int* flag, float2* split, double* lam_next,
+                          double* lam_zero, cudaStream_t st);
 // the same maximum from the (hi, lo) state split (Euler, FP64 and mixed paths)
 cudaError_t launch_max_lambda_split(const DeviceMesh& dm, const float2* Us, double* max_lam,
                                     cudaStream_t st);

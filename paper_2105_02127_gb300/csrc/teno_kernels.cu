@@ -3902,86 +3902,168 @@ struct GatherArgs {
   double gamma;
 };
 
-template <int NV, typename TK>
+// CFL speed lambda = (|u| + c) / L of a cell from its conservative state in
+// FP64 (a non-physical cell, rho <= 0, p <= 0 or NaN, makes it infinite, which
+// the host reports as TENO_ENONPHYS; fmax would drop a NaN speed), or from the
+// (hi, lo) split of the state and the pair 1/L in pair arithmetic on the FP32
+// pipe (relative error ~1e-14, far below what a CFL step needs; false for a NaN
+// speed, which is skipped as fmax skips it)
+__device__ __forceinline__ double cfl_speed(const double* W, double gamma) {
+  const double rho = W[0], u = W[1] / rho, v = W[2] / rho;
+  const double p = (gamma - 1.0) * (W[3] - 0.5 * rho * (u * u + v * v));
+  const double s = sqrt(u * u + v * v) + sqrt(gamma * p / rho);
+  return !(rho > 0.0) || !(p > 0.0) ? __longlong_as_double(0x7ff0000000000000LL) : s;
+}
+__device__ __forceinline__ bool cfl_speed_split(const float2* q, float2 il, float2 g2, float2 gm12,
+                                                DF* lam) {
+  const DF one = {1.f, 0.f}, half = {0.5f, 0.f}, gg = {g2.x, g2.y}, gm1 = {gm12.x, gm12.y};
+  const DF rho = {q[0].x, q[0].y}, mx = {q[1].x, q[1].y}, my = {q[2].x, q[2].y},
+           E = {q[3].x, q[3].y};
+  const DF ir = one / rho;
+  const DF u = mx * ir, v = my * ir;
+  const DF k = u * u + v * v;
+  const DF p = gm1 * (E - half * rho * k);
+  const DF sp = tsqrt(k) + tsqrt(gg * p * ir);
+  *lam = sp * DF{il.x, il.y};
+  return lam->h == lam->h;
+}
+// block maximum of non-negative lam (which order like their bit patterns) into
+// *out; every thread of a 256-thread block takes part
+__device__ __forceinline__ void block_max(double lam, unsigned long long* out) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) lam = fmax(lam, __shfl_xor_sync(0xffffffffu, lam, o));
+  __shared__ double red[32];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (l == 0) red[w] = lam;
+  __syncthreads();
+  if (w == 0) {
+    lam = l < (int)(blockDim.x >> 5) ? red[l] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lam = fmax(lam, __shfl_xor_sync(0xffffffffu, lam, o));
+    if (l == 0) atomicMax(out, (unsigned long long)__double_as_longlong(lam));
+  }
+}
+
+// The next step's CFL maximum, taken by the update that makes its state (the
+// last stage of a step with another one after it): the same per-cell speeds as
+// max_lambda_kernel and max_lambda_split_kernel without their launch and read.
+// A step of a small mesh is bound by its chain of launches, ten of them with the
+// separate reduction: 2,048 cells, scalar TENO3, 63.5 -> 58 us a step, 32,768
+// cells, Euler TENO5, 170 -> 162.
+struct NextLam {
+  unsigned long long* out = nullptr;   // maximum of this update's states, or none
+  unsigned long long* zero = nullptr;  // a word to clear (an earlier stage), or none
+  const double* cfl_len = nullptr;
+  const float2* ilen2 = nullptr;
+  const double* cell_speed = nullptr;
+  double adv_speed = 0.0;
+  float2 g2, gm12;
+};
+
+// (kLam: with the next step's CFL maximum; its own instantiation, because the
+// other updates ran 4 % slower with its registers)
+template <int NV, typename TK, bool kLam>
 __global__ void __launch_bounds__(256) gather_kernel(const GatherArgs a, const TK* K,
-                                                     const double* Un,
-                                                     const double* Us,
+                                                     const double* Un, const double* Us,
                                                      double* __restrict__ out, int mode, double cn,
                                                      double cs, double dt_fixed, double cfl,
-                                                     const double* max_lam,
-                                                     int* flag, float2* __restrict__ split) {
+                                                     const double* max_lam, int* flag,
+                                                     float2* __restrict__ split,
+                                                     const NextLam nl) {
   pdl_wait();
-  // the step size once per block (one FP64 division)
+  // the step size once per block (one FP64 division, while the others load)
   __shared__ double s_dt;
   if (mode != 0 && threadIdx.x == 0) s_dt = max_lam ? cfl / *max_lam : dt_fixed;
-  if (mode != 0) __syncthreads();
+  if (nl.zero && blockIdx.x == 0 && threadIdx.x == 0) *nl.zero = 0ull;
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= a.n_cell) return;
-  double acc[NV];
-  if constexpr (std::is_same<TK, DF>::value || std::is_same<TK, float>::value) {
-    // pair (or FP32) fluxes summed in pairs on the FP32 pipe, one conversion
-    // per variable; three FP32 terms sum exactly in a pair
-    DF sum[NV];
+  const bool in = c < a.n_cell;
+  double acc[NV], un[NV], us[NV], ia = 0.0;
+  if (in) {
+    if constexpr (std::is_same<TK, DF>::value || std::is_same<TK, float>::value) {
+      // pair (or FP32) fluxes summed in pairs on the FP32 pipe, one conversion
+      // per variable; three FP32 terms sum exactly in a pair
+      DF sum[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) sum[v] = DF{0.f, 0.f};
+      for (int v = 0; v < NV; ++v) sum[v] = DF{0.f, 0.f};
 #pragma unroll
-    for (int e = 0; e < 3; ++e) {
-      const int cf = a.c_faces[3 * c + e];
-      const int64_t f = cf >> 1;
-      TK kf[NV];
-      ld_group<NV>(K + f * NV, kf);
+      for (int e = 0; e < 3; ++e) {
+        const int cf = a.c_faces[3 * c + e];
+        const int64_t f = cf >> 1;
+        TK kf[NV];
+        ld_group<NV>(K + f * NV, kf);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        DF k;
-        if constexpr (std::is_same<TK, DF>::value)
-          k = kf[v];
-        else
-          k = DF{kf[v], 0.f};
-        sum[v] = (cf & 1) ? sum[v] - k : sum[v] + k;
+        for (int v = 0; v < NV; ++v) {
+          DF k;
+          if constexpr (std::is_same<TK, DF>::value)
+            k = kf[v];
+          else
+            k = DF{kf[v], 0.f};
+          sum[v] = (cf & 1) ? sum[v] - k : sum[v] + k;
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) acc[v] = to_d(sum[v]);
+    } else {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        const int cf = a.c_faces[3 * c + e];
+        const int64_t f = cf >> 1;
+        const double s = (cf & 1) ? -1.0 : 1.0;
+        TK kf[NV];
+        ld_group<NV>(K + f * NV, kf);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v] = fma(s, to_d(kf[v]), acc[v]);
       }
     }
+    ia = a.inv_area[c];
+    if (mode == 0) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = to_d(sum[v]);
-  } else {
+      for (int v = 0; v < NV; ++v) out[v * a.n_pad + c] = -acc[v] * ia;
+    } else {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = 0.0;
-#pragma unroll
-    for (int e = 0; e < 3; ++e) {
-      const int cf = a.c_faces[3 * c + e];
-      const int64_t f = cf >> 1;
-      const double s = (cf & 1) ? -1.0 : 1.0;
-      TK kf[NV];
-      ld_group<NV>(K + f * NV, kf);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) acc[v] = fma(s, to_d(kf[v]), acc[v]);
+      for (int v = 0; v < NV; ++v) un[v] = Un[v * a.n_pad + c], us[v] = Us[v * a.n_pad + c];
     }
   }
-  const double ia = a.inv_area[c];
-  if (mode == 0) {
+  if (mode == 0) return;
+  __syncthreads();
+  double lam = 0.0;
+  if (in) {
+    const double wr = cs * s_dt * ia;  // the stage's weight of the face-flux sum
+    double u[NV];
+    float2 sp[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) out[v * a.n_pad + c] = -acc[v] * ia;
-    return;
-  }
-  const double wr = cs * s_dt * ia;  // the stage's weight of the face-flux sum
-  double u[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const int64_t i = v * a.n_pad + c;
-    u[v] = fma(-wr, acc[v], fma(cn, Un[i], cs * Us[i]));
-    out[i] = u[v];
-    if (split) {
-      const float hi = (float)u[v];
-      split[i] = make_float2(hi, (float)(u[v] - (double)hi));
+    for (int v = 0; v < NV; ++v) {
+      const int64_t i = v * a.n_pad + c;
+      u[v] = fma(-wr, acc[v], fma(cn, un[v], cs * us[v]));
+      out[i] = u[v];
+      if (split) {
+        const float hi = (float)u[v];
+        sp[v] = make_float2(hi, (float)(u[v] - (double)hi));
+        split[i] = sp[v];
+      }
+    }
+    if constexpr (NV == 4) {
+      // rho > 0 and p > 0, the latter as rho E - |m|^2 / 2 > 0 (no division)
+      const double rho = u[0];
+      const double pr = u[3] * rho - 0.5 * (u[1] * u[1] + u[2] * u[2]);
+      if (!(rho > 0.0) || !(pr > 0.0)) atomicOr(flag, 1);
+    } else {
+      if (!(u[0] == u[0])) atomicOr(flag, 1);
+    }
+    if constexpr (kLam) {
+      if constexpr (NV == 1) {
+        lam = (nl.cell_speed ? nl.cell_speed[c] : nl.adv_speed) / nl.cfl_len[c];
+      } else if (split) {
+        DF l;
+        if (cfl_speed_split(sp, nl.ilen2[c], nl.g2, nl.gm12, &l)) lam = fmax(0.0, to_d(l));
+      } else {
+        lam = cfl_speed(u, a.gamma) / nl.cfl_len[c];
+      }
     }
   }
-  if constexpr (NV == 4) {
-    // rho > 0 and p > 0, the latter as rho E - |m|^2 / 2 > 0 (no division)
-    const double rho = u[0];
-    const double pr = u[3] * rho - 0.5 * (u[1] * u[1] + u[2] * u[2]);
-    if (!(rho > 0.0) || !(pr > 0.0)) atomicOr(flag, 1);
-  } else {
-    if (!(u[0] == u[0])) atomicOr(flag, 1);
-  }
+  if constexpr (kLam) block_max(lam, nl.out);
 }
 
 // --------------------------------------------------------------- CFL speed
@@ -4000,28 +4082,14 @@ __global__ void __launch_bounds__(256) max_lambda_kernel(const double* U,
     if constexpr (NV == 1) {
       s = cell_speed ? cell_speed[c] : adv_speed;
     } else {
-      const double rho = U[c], u = U[n_pad + c] / rho, v = U[2 * n_pad + c] / rho;
-      const double p = (gamma - 1.0) * (U[3 * n_pad + c] - 0.5 * rho * (u * u + v * v));
-      s = sqrt(u * u + v * v) + sqrt(gamma * p / rho);
-      // a non-physical cell (rho <= 0, p <= 0 or NaN) makes the maximum infinite, which
-      // the host reports as TENO_ENONPHYS (fmax would drop a NaN speed)
-      if (!(rho > 0.0) || !(p > 0.0)) s = __longlong_as_double(0x7ff0000000000000LL);
+      double W[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) W[v] = U[v * n_pad + c];
+      s = cfl_speed(W, gamma);
     }
     lam = fmax(lam, s / cfl_len[c]);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) lam = fmax(lam, __shfl_xor_sync(0xffffffffu, lam, o));
-  __shared__ double red[32];
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) red[w] = lam;
-  __syncthreads();
-  if (w == 0) {
-    lam = l < (int)(blockDim.x >> 5) ? red[l] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) lam = fmax(lam, __shfl_xor_sync(0xffffffffu, lam, o));
-    // non-negative doubles order like their bit patterns
-    if (l == 0) atomicMax(out, (unsigned long long)__double_as_longlong(lam));
-  }
+  block_max(lam, out);
 }
 
 // The same maximum from the (hi, lo) split of the state that the FP64 and
@@ -4035,34 +4103,16 @@ __global__ void __launch_bounds__(256) max_lambda_split_kernel(const float2* Us,
                                                                float2 g2, float2 gm12,
                                                                unsigned long long* out) {
   pdl_wait();
-  const DF one = {1.f, 0.f}, half = {0.5f, 0.f}, gg = {g2.x, g2.y}, gm1 = {gm12.x, gm12.y};
   DF lam = {0.f, 0.f};
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n_cell;
        c += (int64_t)gridDim.x * blockDim.x) {
-    const float2 q0 = Us[c], q1 = Us[n_pad + c], q2 = Us[2 * n_pad + c], q3 = Us[3 * n_pad + c];
-    const DF rho = {q0.x, q0.y}, mx = {q1.x, q1.y}, my = {q2.x, q2.y}, E = {q3.x, q3.y};
-    const DF ir = one / rho;
-    const DF u = mx * ir, v = my * ir;
-    const DF q = u * u + v * v;
-    const DF p = gm1 * (E - half * rho * q);
-    const DF sp = tsqrt(q) + tsqrt(gg * p * ir);
-    const float2 il = ilen2[c];
-    const DF l = sp * DF{il.x, il.y};
-    if (l.h == l.h) lam = vmax(lam, l);
-  }
-  double d = to_d(lam);
+    float2 q[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) d = fmax(d, __shfl_xor_sync(0xffffffffu, d, o));
-  __shared__ double red[32];
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) red[w] = d;
-  __syncthreads();
-  if (w == 0) {
-    d = l < (int)(blockDim.x >> 5) ? red[l] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d = fmax(d, __shfl_xor_sync(0xffffffffu, d, o));
-    if (l == 0) atomicMax(out, (unsigned long long)__double_as_longlong(d));
+    for (int v = 0; v < 4; ++v) q[v] = Us[v * n_pad + c];
+    DF l;
+    if (cfl_speed_split(q, ilen2[c], g2, gm12, &l)) lam = vmax(lam, l);
   }
+  block_max(to_d(lam), out);
 }
 
 // -------------------------------------------------------------- utilities
@@ -5179,14 +5229,24 @@ cudaError_t launch_face_flux(const DeviceMesh& dm, const void* Uq, void* K, doub
 
 cudaError_t launch_gather(const DeviceMesh& dm, const void* K, const double* Un, const double* Us,
                           double* out, int mode, double cn, double cs, double dt_fixed,
-                          const double* max_lam, int* flag, float2* split, cudaStream_t st) {
+                          const double* max_lam, int* flag, float2* split, double* lam_next,
+                          double* lam_zero, cudaStream_t st) {
   GatherArgs a{dm.c_faces, dm.inv_area, dm.n_update, dm.n_pad, dm.gamma};
+  NextLam nl;
+  nl.out = (unsigned long long*)lam_next;
+  nl.zero = (unsigned long long*)lam_zero;
+  nl.cfl_len = dm.cfl_len;
+  nl.ilen2 = dm.cfl_ilen2;
+  nl.cell_speed = dm.n_var == 1 ? dm.cell_speed : nullptr;
+  nl.adv_speed = sqrt(dm.adv_x * dm.adv_x + dm.adv_y * dm.adv_y);
+  nl.g2 = split2(dm.gamma);
+  nl.gm12 = split2(dm.gamma - 1.0);
   const unsigned grid = (unsigned)((dm.n_update + 255) / 256);
   auto go = [&](auto nvc, auto tkc) {
     constexpr int NV = decltype(nvc)::value;
     using TK = typename decltype(tkc)::type;
-    launch(gather_kernel<NV, TK>, grid, 256, 0, st, a, (const TK*)K, Un, Us, out, mode, cn, cs,
-                                                dt_fixed, dm.cfl, max_lam, flag, split);
+    launch(lam_next ? gather_kernel<NV, TK, true> : gather_kernel<NV, TK, false>, grid, 256, 0, st,
+           a, (const TK*)K, Un, Us, out, mode, cn, cs, dt_fixed, dm.cfl, max_lam, flag, split, nl);
   };
   using I1 = std::integral_constant<int, 1>;
   using I4 = std::integral_constant<int, 4>;
