@@ -2792,18 +2792,23 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
     {
       const int n_mine = (H - lane + kTile - 1) / kTile;  // this lane's halo cells
       unsigned mx[kVW];
-      double ref[kVW];
+      double ref[kVW], own[kVW];
 #pragma unroll
       for (int w = 0; w < kVW; ++w) {
         const double u0 = hv[w * P::kHaloRow + kHaloMax + lane];
         ref[w] = __shfl_sync(0xffffffffu, u0, 0);
-        mx[w] = mine ? mag_bits(u0 - ref[w]) : 0u;
+        own[w] = u0 - ref[w];
+        mx[w] = mine ? mag_bits(own[w]) : 0u;
       }
 #pragma unroll 2
       for (int i = 0; i < n_mine; ++i)
 #pragma unroll
-        for (int w = 0; w < kVW; ++w)
-          mx[w] = max(mx[w], mag_bits(hv[w * P::kHaloRow + lane + i * kTile] - ref[w]));
+        for (int w = 0; w < kVW; ++w) {
+          double* q = hv + w * P::kHaloRow + lane + i * kTile;
+          const double d = *q - ref[w];
+          *q = d;  // one FP64 operation per state (the FP64 pipe is the slow one)
+          mx[w] = max(mx[w], mag_bits(d));
+        }
       double cf[kVW];
 #pragma unroll
       for (int w = 0; w < kVW; ++w) {
@@ -2813,15 +2818,14 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         direct[w] = e > 100;
         sc[w] = direct[w] ? 0 : Dot::kBits - 1 - e;
         cf[w] = __hiloint2double((sc[w] + 1023) << 20, 0);
-        const double u0 = hv[w * P::kHaloRow + kHaloMax + lane];
-        y0[w] = mine && !direct[w] ? Dot::fix(u0 - ref[w], sc[w], cf[w]) : 0;
+        y0[w] = mine && !direct[w] ? Dot::fix(own[w], sc[w], cf[w]) : 0;
       }
 #pragma unroll 2
       for (int i = 0; i < n_mine; ++i)
 #pragma unroll
         for (int w = 0; w < kVW; ++w) {
           double* q = hv + w * P::kHaloRow + lane + i * kTile;
-          *q = __longlong_as_double(direct[w] ? 0 : Dot::fix(*q - ref[w], sc[w], cf[w]));
+          *q = __longlong_as_double(direct[w] ? 0 : Dot::fix(*q, sc[w], cf[w]));
         }
       __syncwarp();
     }
