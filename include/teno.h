@@ -65,7 +65,8 @@ enum teno_flux { TENO_FLUX_UPWIND = 0, TENO_FLUX_HLL = 1, TENO_FLUX_HLLC = 2 };
  * TENO_FP32_MIXED: matvecs and fluxes in FP32 with FP32 accumulation, the
  *   selection decision (FP64 inside a guard band of C_T) and the residual
  *   accumulation and update in FP64;
- * TENO_FP64_NATIVE: everything in FP64 on the FP64 pipe. */
+ * TENO_FP64_NATIVE: FP64 state, matrices, Gauss values, flux and update; the
+ * default Euler reconstruction forms its products in 60-bit fixed point. */
 enum teno_precision { TENO_FP64 = 0, TENO_FP32_MIXED = 1, TENO_FP64_NATIVE = 2 };
 
 /* Boundary tags of non-periodic meshes (bface[:,2]); the ghost state at each
