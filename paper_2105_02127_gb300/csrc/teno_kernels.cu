@@ -2,7 +2,7 @@
 // sm_103a (GB300).
 //
 // Per RK stage (Sec. 2.1, Eq. fv_governing_equation_semi_discrete):
-//   recon_kernel      stencil differences, coefficient matvecs (Eqs.
+//   recon_*_kernel    stencil differences, coefficient matvecs (Eqs.
 //                     reconstruction_08/09 with |V'_s| folded into the
 //                     matrices), smoothness indicators (Eq. WENO_smoothness in
 //                     a beta-orthonormal basis, so beta = |a'|^2), TENO scale
@@ -2037,7 +2037,7 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), kDF ? 2 : 0)
 //    for the coefficients a = G d; the part of a in the row space of Psi' is
 //    a linear image T y of the values y = W d that are known anyway, so only
 //    the rows Q2' G of its orthogonal complement (m - 3 N_q of m) are stored
-//    and summed, in FP32, with a rigorous error bound: 6,100 bytes a cell at
+//    and summed, in FP32, with a rigorous error bound: 5,770 bytes a cell at
 //    TENO6, where W with all rows and their bounds took 8,046.  Where the
 //    bound does not separate chi from C_T the coefficients and beta are
 //    recomputed (pairs, or FP64) and the decision is taken in FP64;
@@ -2046,15 +2046,15 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), kDF ? 2 : 0)
 // The last two are lists a warp works off apart from its tiles: one undecided
 // cell at a time by all lanes, 32 directional cells one per lane, so that their
 // chains of loads stall the warp once and not per cell and slot.
-// Bound: HBM at large meshes (1.6 GB a launch at 262,088 cells TENO6: 326 us,
-// 4.9 TB/s; with pair products, all rows and per-tile block barriers 470 us),
-// the FP64 path by its integer products (131,072 cells: 234 us; FP64
-// multiply-adds 608 us), small meshes by the time of one tile (2,046 cells
-// TENO5: 39 us, 52 before).
+// Bound: HBM and issue at large meshes (1.56 GB a launch at 262,088 cells TENO6:
+// 318 us; with pair products, all rows and per-tile block barriers 470 us), the
+// FP64 path by issue at four consumer warps a block and four blocks (131,072
+// cells: 234 us; FP64 multiply-adds 608 us), small meshes by the time of one tile
+// (2,046 cells TENO5: 39 us, 52 before).
 
 // Variables a consumer warp takes: two on the pair path, where the sums of
 // both share every shared-memory read of W and of the rows (262,088 cells,
-// TENO6: 326 us against 364 with one); one on the FP64 path, whose integer
+// TENO6: 326 us, 364 with one, before later steps); one on the FP64 path, whose integer
 // sums need the registers (131,072 cells: 234 us against 256 with two).
 template <typename HT>
 constexpr int w_vars() {
@@ -4561,23 +4561,26 @@ __global__ void __launch_bounds__(128) recon_vjp_df_kernel(const float2* __restr
 }
 
 // Tiled reconstruction VJP (FP64 path, Euler, W form).  With the selection
-// frozen, Uq_p = U_0 + sum_s W_ps d_s for the large polynomial (W = Psi' G,
-// the per-cell pairs the forward W-form kernel uses), so d_bar_s =
-// sum_p W_ps Uq_bar_p: NQ3 pair products per slot and no coefficient
-// adjoint.  Directional stencils (cells whose large stencil is cut) take
-// d_bar_s = (G_k^T Psi_k^T Uq_bar)_s / n_kept from their (hi, lo) matrices;
-// their stages are streamed only for tiles where some (cell, variable) keeps
-// a directional stencil, a predicate the producer and the consumers evaluate
-// from the same selection bytes.  Each lane adds its d_bar_s to the tile's
-// halo accumulator in shared memory at the slot's halo position (lanes with
-// equal positions in lane order, by ranks the host stores next to the
-// positions; slots in stencil order: deterministic sums).  The host assigns
-// the large-stencil members to slots so that the lanes of a tile do not
-// share a cell within a slot, and these slots take one round.  At the end of
-// the tile the accumulator is written as one pair per (halo entry,
-// variable), so the reverse gather reads the few halo entries that hold a
-// cell instead of every stencil slot that holds it.  The tile's Uq_bar block is prefetched
-// with cp.async one tile ahead.
+// frozen, Uq_p = U_0 + sum_s W_ps d_s for the large polynomial (W = Psi' G in
+// the forward W-form kernel's fixed point), so d_bar_s = sum_p W_ps Uq_bar_p:
+// NQ3 products per slot and no coefficient adjoint.  Directional stencils
+// (cells whose large stencil is cut) take d_bar_s = (G_k^T Psi_k^T Uq_bar)_s /
+// n_kept from their (hi, lo) matrices; their stages are streamed only for tiles
+// where some (cell, variable) keeps a directional stencil, a predicate the
+// producer and the consumers evaluate from the same selection bytes.  The sums
+// run in fixed point: Uq_bar in units of its largest per cell (53 bits), the
+// contributions in one unit per tile and variable as 64-bit integers, so their
+// order does not matter.  Each lane adds its d_bar_s to the tile's halo
+// accumulator in shared memory at the slot's halo position (lanes with equal
+// positions in turn, by ranks the host stores next to the positions).  The host
+// assigns the large-stencil members to slots so that the lanes of a tile do not
+// share a cell within a slot, and these slots take one round.  At the end of the
+// tile the accumulator is written as one pair per (halo entry, variable), so the
+// reverse gather reads the few halo entries that hold a cell instead of every
+// stencil slot that holds it.  The tile's Uq_bar block is prefetched with
+// cp.async one tile ahead.  Bound: instruction issue (131,072 cells TENO5 153 us,
+// 8,320 cells TENO6 44; without the block barriers at a tile's ends
+// 151, not worth a second copy of the flags).
 constexpr int kRingV = 4;
 constexpr int kVjpNone = -(1 << 16);  // an exponent below every value's
 constexpr int kUbStride = 38;  // doubles per cell in the Uq_bar stage (16-byte rows)
