@@ -4290,7 +4290,9 @@ __device__ __forceinline__ void store_bar(double* base, int i, S x) {
 // are formed once and shared.  Bound: FP32 issue (pairs) at 168 registers, the
 // latency of one reverse sweep at small meshes, where a thread that took a
 // face's points in turn ran three in a row
-// (8,320 cells TENO6, HLLC: 136 us a residual's adjoint, 122 now).
+// (8,320 cells TENO6, HLLC: 136 us a residual's adjoint, 122 now).  The states
+// load while the cotangents are formed (1,048,352 cells TENO6: 706 us, 746 with
+// the loads after the barrier; 32 faces a block 722).
 template <int NV, int NQ, int FLUX, typename TQ, typename S, int ND>
 __global__ void __launch_bounds__(kFluxFaces * NQ, 384 / (kFluxFaces * NQ))
     face_flux_vjp_kernel(const VjpArgs a, const TQ* Uq, const double* w,
@@ -4310,10 +4312,9 @@ __global__ void __launch_bounds__(kFluxFaces * NQ, 384 / (kFluxFaces * NQ))
     if (n >= 0) kb = fma(w[v * a.n_pad + n], a.inv_area[n], kb);
     sK[e % kFluxFaces * NV + v] = cst<S>(kb);
   }
-  __syncthreads();
   const int k = threadIdx.x % NQ;
-  const int64_t f = f0 + threadIdx.x / NQ;
-  if (f >= a.n_face) return;
+  const bool in = f0 + threadIdx.x / NQ < a.n_face;  // (past the end: the last face's loads)
+  const int64_t f = in ? f0 + threadIdx.x / NQ : a.n_face - 1;
   const int o = a.f_cells[2 * f], n = a.f_cells[2 * f + 1];
   const int eo = a.f_edges[2 * f], en = a.f_edges[2 * f + 1];
   const double nx = a.f_geom[5 * f], ny = a.f_geom[5 * f + 1], len = a.f_geom[5 * f + 2];
@@ -4327,6 +4328,8 @@ __global__ void __launch_bounds__(kFluxFaces * NQ, 384 / (kFluxFaces * NQ))
     TQ ul[NV], ur[NV];
     ld_group<NV>(Uq + ((int64_t)(o * 3 + eo) * NQ + k) * NV, ul);
     if (n >= 0) ld_group<NV>(Uq + ((int64_t)(n * 3 + en) * NQ + (NQ - 1 - k)) * NV, ur);
+    __syncthreads();  // the cotangents, while the states load
+    if (!in) return;
     // x of the Gauss point (ghost states and the scalar field only)
     auto xq = [&]() { return a.f_geom[5 * f + 3] - ny * len * a.gt[k]; };
     const S wl = gauss_w<S>(a.gw[k], a.gw2[k]) * tl;
