@@ -2531,6 +2531,8 @@ __device__ __noinline__ int w_screen(float t0, float t1, float t2, float tK, int
 
 // deferred cells: the cell in the low word; the high word's flags, and the
 // selection where it is decided
+// (bits 0-3 of it: a selection override passes a caller's bytes, whose other bits
+// mean nothing and would reach the variable)
 constexpr int kDefNear = 1, kDefDirect = 2, kDefSel = 8;  // selection from bit 3
 constexpr int kDefVar = 256;                              // variable from bit 8
 
@@ -3073,7 +3075,7 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
       if (def)
         mylist[n_def + __popc(bal & ((1u << lane) - 1u))] =
             make_int2((int)c, (near[w] ? kDefNear : 0) | (direct[w] ? kDefDirect : 0) |
-                                  sel[w] * kDefSel | (v0 + w) * kDefVar);
+                                  (sel[w] & 15) * kDefSel | (v0 + w) * kDefVar);
       n_def += __popc(bal);
     }
     __syncwarp();
