@@ -1698,6 +1698,10 @@ __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src)
                : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src)
+               : "memory");
+}
 // 16-byte asynchronous copy (both addresses 16-byte aligned), L2 only
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src)
@@ -2031,8 +2035,12 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), kDF ? 2 : 0)
 //    FP64 rate is 1/64 of its FP32 rate) and a pair multiply-add 12 FP32
 //    instructions; here it costs three wide integer multiply-adds (FP64 path;
 //    each holds its pipe for about 5 clocks a warp) or one and two FP32
-//    multiply-adds (pairs), and the sums are accurate to the bits of the
-//    result;
+//    multiply-adds (pairs).  The states' rounding to the tile's unit is one of
+//    the largest difference in the tile, up to 2^-51 of it (pairs) or 2^-57; where
+//    that is more than some cell's own rounding (the small side of a jump that
+//    the tile holds, own_scale) the tile's integers take the 64 bits there are and
+//    each lane the bits of them that its cell needs, and cells for which these do
+//    not do either are summed in floating point (w_direct);
 //  - the smoothness indicators feed only the cutoff decision.  beta = |a|^2
 //    for the coefficients a = G d; the part of a in the row space of Psi' is
 //    a linear image T y of the values y = W d that are known anyway, so only
@@ -2086,9 +2094,15 @@ struct WPlan {
   static constexpr int kHaloRow = kHaloMax + kTile;     // halo states, then the tile's own
   static constexpr int kHalo = 2 * 4 * kHaloRow * 8;    // double-buffered, per variable
   static constexpr int kListN = (kVW + 1) * kTile;      // deferred cells of a warp
-  static constexpr int kScratch = kSL * 8;              // differences of one cell, per warp
-  static constexpr int kFixed =
-      kHalo + 2 * kTileBytes + kWWarps * (kListN * 8 + kScratch) + 16 * 8 + 16;
+  // per warp: the differences of one cell, or the tile's directional indicators
+  static constexpr int kScratch = kSL * 8 > kVW * kSmallK * 2 * kTile * 4
+                                      ? kSL * 8
+                                      : kVW * kSmallK * 2 * kTile * 4;
+  // what own_scale needs of the tile's cells beyond a warp's own variables, two
+  // buffers a warp: the other one of rho and E (pairs), or both and wstat's last word
+  static constexpr int kOwn2 = (3 - kVW) * kTile * 8 + (kVW == 1 ? kTile * 4 : 0);
+  static constexpr int kFixed = kHalo + 2 * kTileBytes + kWWarps * 2 * kOwn2 +
+                                kWWarps * (kListN * 8 + kScratch) + 16 * 8 + 16;
   // four blocks per SM (96 threads of up to 168 registers, or 160 of 96); the
   // ring takes what is left of their quarter of the 227 KB of shared memory
   static constexpr int kRoom = (227 * 1024 / 4 - 1024 - kFixed) / kBuf;
@@ -2127,9 +2141,11 @@ __device__ __forceinline__ float dot_bound(float norm, float dd, float q, int n)
 __device__ __forceinline__ float exp2i(int e) {
   return e < -126 ? 0.f : (e > 127 ? __int_as_float(0x7f800000) : __int_as_float((e + 127) << 23));
 }
+// 2^e as FP64, |e| <= 1000
+__device__ __forceinline__ double exp2d(int e) { return __hiloint2double((e + 1023) << 20, 0); }
 // m 2^sh rounded to the nearest integer, m >= 0
 __device__ __forceinline__ int64_t shift_round(int64_t m, int sh) {
-  if (sh >= 0) return m << sh;
+  if (sh >= 0) return (int64_t)((uint64_t)m << sh);
   if (sh < -62) return 0;
   return (m + ((int64_t)1 << (-sh - 1))) >> -sh;
 }
@@ -2150,6 +2166,11 @@ __device__ __forceinline__ int64_t to_fix(double x, int k) {
   return hi < 0 ? -r : r;
 }
 __device__ __forceinline__ int64_t to_fix(float2 x, int k) { return to_fix(x.x, k) + to_fix(x.y, k); }
+// x 2^k as an integer modulo 2^64, rounded: differences below 2^63 come out of it
+__device__ __forceinline__ int64_t to_fix_mod(double x, int k) {
+  const int ef = max((__double2hiint(x) >> 20) & 0x7ff, 1);
+  return ef - 1075 + k > 63 ? 0 : to_fix(x, k);
+}
 // magnitude bits of a state (ordered like |x|) and their unbiased exponent;
 // kFixExpBad marks infinities and NaN
 constexpr int kFixExpBad = 1 << 20;
@@ -2171,10 +2192,6 @@ __device__ __forceinline__ int mag_exp(unsigned m) {
 }
 // limbs x = h 2^30 + l with l in [0, 2^30)
 constexpr int kFixB = 30;
-__device__ __forceinline__ void fix_limbs(int64_t x, int& h, int& l) {
-  h = (int)(x >> kFixB);
-  l = (int)x & ((1 << kFixB) - 1);
-}
 // entry e of a stage's W (pairs of entries as 16 bytes a lane, a last odd one
 // as 8) and of its FP32 rows (fours as 16 bytes, the rest one by one)
 template <int N>
@@ -2215,6 +2232,9 @@ struct WDot<double> {
   static constexpr int kBits = 57;      // |Y| < 2^57
   // bound of the sum's error: kErr units 2^exp, plus kErrD 2^-kc |d|_2
   static constexpr float kErr = 256.f, kErrD = 0.f;
+  // own_scale's weight of s (an exponent): the values are rounded to 2^-53 of it, the sum to
+  // |W|_1 < 2^(60 - kc) units
+  __device__ __forceinline__ static int own_weight(int kc) { return kc - 58; }
   // an integer of |x| 2^sc < 2^57
   __device__ __forceinline__ static int64_t fix(double x, int sc, double) { return to_fix(x, sc); }
   struct D {
@@ -2228,9 +2248,10 @@ struct WDot<double> {
   };
   __device__ __forceinline__ static W entry(int2 m) { return {m}; }
   __device__ __forceinline__ static float c(int sc) { return exp2i(kFixB - sc); }
-  // the parts and the FP32 value (c = 2^(30 - sc)) of a difference
-  __device__ __forceinline__ static float split(int64_t d, float c, D& o) {
-    fix_limbs(d, o.h, o.l);
+  // the parts and the FP32 value (c = 2^(30 - sc)) of a difference d 2^-sh
+  __device__ __forceinline__ static float split(int64_t d, int sh, float c, D& o) {
+    o.h = (int)(d >> (kFixB + sh));
+    o.l = (int)(d >> sh) & ((1 << kFixB) - 1);
     return fmaf((float)o.h, c, (float)o.l * (c * (1.f / 1073741824.f)));
   }
   __device__ __forceinline__ static void mac(A& a, W w, D d) {
@@ -2243,14 +2264,18 @@ struct WDot<double> {
 // FP32 fraction, d = (dh + dl) 2^B likewise (|dh| <= 2^30): sum wh dh is exact
 // in 64 bits and wl dh + wh dl, 2^-31 of it, is an FP32 sum (two FP32
 // multiply-adds in the place of two wide ones; a wide multiply-add holds its
-// pipe for 5 clocks).  Accurate to about 2^-53 of |W|_1 times the tile's state
-// range, beyond the 48 bits of the pair it becomes.
+// pipe for 5 clocks).  The states' rounding is half a unit each, so the sum errs
+// by at most |W|_1 units, and by about a third of |W|_2 units as a rule; the FP32
+// part adds about as much.
 template <int kB>
 struct WPairDot {
   static constexpr int kBits = kB + 29;
   // the FP32 sum's 2 n roundings, each 2^-25 of |x| <= sum (|wl| |dh| + |wh| |dl|) <=
   // (sqrt(n) |dh|_2 + 2^31) / 2
   static constexpr float kErr = 8192.f, kErrD = 2e-5f;
+  // (the pairs that the states become in every other kernel of this path are
+  // rounded to 2^-49 of them before the difference, so |W|_1 is on both sides)
+  __device__ __forceinline__ static int own_weight(int) { return 0; }
   // an integer of |x| 2^sc < 2^51, from the low bits of 1.5 2^52 + x 2^sc (c = 2^sc)
   __device__ __forceinline__ static int64_t fix(double x, int, double c) {
     return __double_as_longlong(fma(x, c, 6755399441055744.0)) - 0x4338000000000000LL;
@@ -2271,10 +2296,11 @@ struct WPairDot {
     return {m.x, (float)m.x, __int_as_float(m.y)};
   }
   __device__ __forceinline__ static float c(int sc) { return exp2i(kB - sc); }
-  __device__ __forceinline__ static float split(int64_t d, float c, D& o) {
-    o.h = (int)((d + (1 << (kB - 1))) >> kB);
+  __device__ __forceinline__ static float split(int64_t d, int sh, float c, D& o) {
+    const int z = (int)(d >> sh);
+    o.h = (int)(d >> (kB + sh)) + ((z >> (kB - 1)) & 1);
     o.hf = (float)o.h;
-    o.lf = (float)(((int)d << (32 - kB)) >> (32 - kB)) * (1.f / (1 << kB));
+    o.lf = (float)((z << (32 - kB)) >> (32 - kB)) * (1.f / (1 << kB));
     return (o.hf + o.lf) * c;
   }
   __device__ __forceinline__ static void mac(A& a, W w, D d) {
@@ -2298,6 +2324,18 @@ struct WPairDot {
 // (the low bits of an FP64 sum give 51-bit differences)
 template <>
 struct WDot<float2> : WPairDot<22> {};
+// Whether a cell keeps its own precision in units of 2^-sc: w s or max|d| is at
+// least 2^(kBits - 2) units, for the differences d of its large stencil (es, ed:
+// exponents of s and max|d|, w: own_weight).  That bounds the units' rounding by
+// that of the sums in the path's own arithmetic: 2^-49 of s or |d| for pairs, 2^-53
+// of s and 2^-55 of |d| in FP64.  s is |U_0|, and for a momentum at least 2^-6
+// sqrt(rho E) (sqrt(rho E) >= |m| / 2^(1/2)): the flux rounds to 2^-49 or 2^-53 of
+// sqrt(rho E) however small the momentum is, so a decaying tail of it (15 % of the
+// shear layer's cells by |m| alone) has nothing to keep.
+template <typename Dot>
+__device__ __forceinline__ bool own_scale(int es, int ed, int kc, int sc) {
+  return max(es + Dot::own_weight(kc), ed) >= Dot::kBits - 2 - sc;
+}
 // x 2^e as a pair (|x| < 2^62; e within the FP32 range less 42)
 __device__ __forceinline__ DF fix_to_df(int64_t x, float s2, float s1, float s0) {
   const float h = (float)(int)(x >> 42) * s2;
@@ -2469,7 +2507,8 @@ __device__ __noinline__ void w_small(const HT* A, const int32_t* nb, const HT* s
 }
 
 // Large-stencil values of a cell whose tile holds an infinity, a NaN or a
-// magnitude outside the fixed-point range: U_0 + W d in floating point.
+// magnitude outside the fixed-point range, or too large a difference for the
+// cell's own scale (own_scale): U_0 + W d in floating point.
 template <int NS, int NQ3, int NV>
 __device__ __noinline__ void w_direct(const int2* W, int lane, int kc, const int32_t* nb,
                                       const float2* st, float2 u0s, float2* out) {
@@ -2620,9 +2659,10 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
   extern __shared__ __align__(128) unsigned char smem[];
   double* halo = reinterpret_cast<double*>(smem + (size_t)kR * P::kBuf);  // [2][NV][kHaloRow]
   int32_t* tblk = reinterpret_cast<int32_t*>(halo + 2 * NV * P::kHaloRow);  // [2][kWTile]
-  int2* list = reinterpret_cast<int2*>(tblk + 2 * kWTile);  // [kWWarps][kListN]
-  HT* scratch = reinterpret_cast<HT*>(list + kWWarps * P::kListN);  // [kWWarps][kSL]
-  uint64_t* full = reinterpret_cast<uint64_t*>(scratch + kWWarps * P::kSL);
+  unsigned char* owns = reinterpret_cast<unsigned char*>(tblk + 2 * kWTile);  // [kWWarps][2][kOwn2]
+  int2* list = reinterpret_cast<int2*>(owns + kWWarps * 2 * P::kOwn2);  // [kWWarps][kListN]
+  HT* scratch = reinterpret_cast<HT*>(list + kWWarps * P::kListN);  // [kWWarps][kScratch]
+  uint64_t* full = reinterpret_cast<uint64_t*>(scratch + kWWarps * (P::kScratch / 8));
   uint64_t* empty = full + kR;
   uint64_t* tfull = empty + kR;
   uint64_t* tempty = tfull + 2;
@@ -2722,7 +2762,11 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
   constexpr int kPerLane = kHaloMax / kTile;
   const int v0 = warp * kVW;
   int2* mylist = list + warp * P::kListN;
-  HT* dsc = scratch + warp * P::kSL;
+  HT* dsc = scratch + warp * (P::kScratch / 8);
+  // beta and |d|^2 of the directional stencils, [kSmallK][kVW][2][32]: twelve
+  // registers less in the large stencil's loop
+  float* tsd = reinterpret_cast<float*>(dsc) + lane;
+  unsigned char* own2 = owns + warp * 2 * P::kOwn2;
   int n_def = 0, it = 0;
   RingPos<kR> rp;
   // the wait of one consumer warp; false: some wait of the block gave up
@@ -2760,6 +2804,17 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         for (int w = 0; w < kVW; ++w)
           cp_async8(dst + w * P::kHaloRow + kHaloMax + lane,
                     src + w * a.n_pad + (c < a.n_cell ? c : 0));
+        double* o2 = reinterpret_cast<double*>(own2 + (i & 1) * P::kOwn2) + lane;
+        if constexpr (kN) {
+          if (v0 == 1 || v0 == 2)
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+              cp_async8(o2 + k * kTile, a.U + 3 * k * a.n_pad + (c < a.n_cell ? c : 0));
+          cp_async4(reinterpret_cast<int32_t*>(own2 + (i & 1) * P::kOwn2 + 2 * kTile * 8) + lane,
+                    wa.st + (tile * kWStat + kWStat - 1) * kTile + lane);
+        } else {
+          cp_async8(o2, a.U + (v0 == 0 ? 3 : 0) * a.n_pad + (c < a.n_cell ? c : 0));
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty[i & 1]);
       }
@@ -2788,9 +2843,10 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
     // in place (Dot::kBits of the largest difference).  The unit depends on
     // the set of the tile's cells and halo only, so a partition, which keeps
     // whole tiles, gets the same bits
+    const unsigned char* st = reinterpret_cast<const unsigned char*>(hv);
     int64_t y0[kVW];
-    int sc[kVW];       // the units are 2^-sc
-    bool direct[kVW];  // the tile's states of this variable have no such unit
+    int sc[kVW], sh[kVW];  // units: the cell's 2^-sc, the tile's 2^-(sc + sh)
+    int float_w[kVW];      // 1: the tile's states have no unit, 2: too coarse a one for the cell
     {
       const int n_mine = (H - lane + kTile - 1) / kTile;  // this lane's halo cells
       unsigned mx[kVW];
@@ -2811,43 +2867,113 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
           *q = d;  // one FP64 operation per state (the FP64 pipe is the slow one)
           mx[w] = max(mx[w], mag_bits(d));
         }
-      double cf[kVW];
+      // a cell's scale (own_scale), first without its differences
+      const unsigned char* o2 = own2 + (it & 1) * P::kOwn2;
+      const int kc =
+          kN ? (int)(int16_t)(reinterpret_cast<const int32_t*>(o2 + 2 * kTile * 8)[lane] & 0xffff) : 0;
+      int es[kVW];
+      bool coarse = false;
 #pragma unroll
       for (int w = 0; w < kVW; ++w) {
         mx[w] = __reduce_max_sync(0xffffffffu, mx[w]);
         // |U - U_ref| < 2^(e + 1); a difference below 2^-900 counts as none
         const int e = max(mx[w] ? mag_exp<double>(mx[w]) : 0, -900);
-        direct[w] = e > 100;
-        sc[w] = direct[w] ? 0 : Dot::kBits - 1 - e;
-        cf[w] = __hiloint2double((sc[w] + 1023) << 20, 0);
-        y0[w] = mine && !direct[w] ? Dot::fix(own[w], sc[w], cf[w]) : 0;
+        float_w[w] = e > 100;
+        sc[w] = float_w[w] ? 0 : Dot::kBits - 1 - e;
+        sh[w] = 0;
+        es[w] = mag_exp<double>(mag_bits(hv[w * P::kHaloRow + kHaloMax + lane]));
+        if (v0 + w == 1 || v0 + w == 2) {  // rho and E, in either order
+          const double* x = reinterpret_cast<const double*>(o2) + lane;
+          const double y = kN ? x[kTile] : hv[(kVW - 1 - w) * P::kHaloRow + kHaloMax + lane];
+          es[w] = max(es[w], ((mag_exp<double>(mag_bits(*x)) + mag_exp<double>(mag_bits(y))) >> 1) - 6);
+        }
+        coarse |= mine && mx[w] && !float_w[w] && !own_scale<Dot>(es[w], -5000, kc, sc[w]);
       }
-#pragma unroll 2
-      for (int i = 0; i < n_mine; ++i)
+      bool wide = __any_sync(0xffffffffu, coarse);
+      int ed[kVW];
+      if (wide) {  // then with them
+        unsigned ml[kVW] = {};
+        const uint16_t* gp = wa.pos + tile * (int64_t)(P::kSL * kTile) + lane;
+        __syncwarp();
+        constexpr int kN1 = NS > 30 ? NS / 3 : NS / 2;  // some slots usually show enough
+#pragma unroll 1
+        for (int i0 = 0; wide && i0 < NS; i0 += kN1) {
+#pragma unroll
+          for (int i = 0; i < kN1; ++i) {
+            const int off = __ldg(gp + (i0 + i) * kTile);
+#pragma unroll
+            for (int w = 0; w < kVW; ++w)
+              ml[w] = max(ml[w], mag_bits(*reinterpret_cast<const double*>(
+                                              st + w * (P::kHaloRow * 8) + off) -
+                                          own[w]));
+          }
+          coarse = false;
+#pragma unroll
+          for (int w = 0; w < kVW; ++w) {
+            ed[w] = mag_exp<double>(ml[w]);
+            coarse |= mine && mx[w] && !float_w[w] && !own_scale<Dot>(es[w], ed[w], kc, sc[w]);
+          }
+          wide = __any_sync(0xffffffffu, coarse);
+        }
+      }
+      if (!wide) {
+        double cf[kVW];
 #pragma unroll
         for (int w = 0; w < kVW; ++w) {
-          double* q = hv + w * P::kHaloRow + lane + i * kTile;
-          *q = __longlong_as_double(direct[w] ? 0 : Dot::fix(*q, sc[w], cf[w]));
+          cf[w] = exp2d(sc[w]);
+          y0[w] = mine && !float_w[w] ? Dot::fix(own[w], sc[w], cf[w]) : 0;
         }
+#pragma unroll 2
+        for (int i = 0; i < n_mine; ++i)
+#pragma unroll
+          for (int w = 0; w < kVW; ++w) {
+            double* q = hv + w * P::kHaloRow + lane + i * kTile;
+            *q = __longlong_as_double(float_w[w] ? 0 : Dot::fix(*q, sc[w], cf[w]));
+          }
+      } else {
+        // 62 bits for the largest difference in the tile, from the states themselves
+        // (U - U_ref is rounded to 2^-53 of it), and of these kBits for its own
+        // largest for each cell: pairs reach cells 2^-12 of the tile's largest
+        // difference, FP64 2^-5 or so (|W|_1).  (A second copy of the loops below
+        // with lane units of any size cost the tiles that never enter it 8 to 16 %:
+        // registers.)
+        const int32_t* ids = wa.tile + tile * kWTile + 4 + lane;
+        __syncwarp();
+#pragma unroll 1
+        for (int i = 0; i < n_mine; ++i) {
+          const int id = __ldg(ids + i * kTile);
+#pragma unroll
+          for (int w = 0; w < kVW; ++w)
+            hv[w * P::kHaloRow + lane + i * kTile] = __longlong_as_double(
+                float_w[w] ? 0
+                           : to_fix_mod(a.U[(int64_t)(v0 + w) * a.n_pad + id], sc[w] + 61 - Dot::kBits));
+        }
+#pragma unroll
+        for (int w = 0; w < kVW; ++w) {
+          y0[w] = 0;
+          if (!mine || float_w[w]) continue;
+          const int sT = sc[w] + 61 - Dot::kBits;  // |U - U_0| 2^sT < 2^62
+          sh[w] = max(0, ed[w] + 1 + sT - Dot::kBits);
+          sc[w] = sT - sh[w];
+          // (with half a unit of the cell, so that the shift rounds)
+          y0[w] = to_fix_mod(hv[w * P::kHaloRow + kHaloMax + lane], sT) -
+                  (int64_t)((1ull << sh[w]) >> 1);
+          if (!own_scale<Dot>(es[w], ed[w], kc, sc[w])) float_w[w] = 2;
+        }
+      }
       __syncwarp();
     }
-    float cd[kVW], cu[kVW];  // FP32 scale of a difference, and one unit
-#pragma unroll
-    for (int w = 0; w < kVW; ++w) cd[w] = Dot::c(sc[w]), cu[w] = 80.f * exp2i(-sc[w]);
-    // difference parts of the cell at a byte offset of the halo row, and the
-    // difference in FP32 (error 3u relative plus 2^6 units).  The 64-bit
-    // conversion would take the FP64 pipe.
-    const unsigned char* st = reinterpret_cast<const unsigned char*>(hv);
-    auto dif = [&](int w, int off, typename Dot::D& d) {
-      return Dot::split(*reinterpret_cast<const int64_t*>(st + w * (P::kHaloRow * 8) + off) - y0[w],
-                        cd[w], d);
+    // the difference to the cell at a byte offset of the halo row, in units of
+    // the tile; its FP32 values below err by 3u relative plus 2^7 of these (the
+    // directional ones, which may exceed the large stencil's) or 2^6 of the
+    // cell's.  The 64-bit conversion would take the FP64 pipe.
+    auto dif = [&](int w, int off) {
+      return *reinterpret_cast<const int64_t*>(st + w * (P::kHaloRow * 8) + off) - y0[w];
     };
+    float cd[kVW];  // their FP32 scale
+#pragma unroll
+    for (int w = 0; w < kVW; ++w) cd[w] = exp2i(-sc[w] - sh[w]);
     // ---- directional stencils: FP32 smoothness indicators
-    float ts[kVW][kSmallK], ds[kVW][kSmallK];
-#pragma unroll
-    for (int w = 0; w < kVW; ++w)
-#pragma unroll
-      for (int k = 0; k < kSmallK; ++k) ts[w][k] = ds[w][k] = 0.f;
 #pragma unroll 1
     for (int k = 0; k < kSmallK; ++k, rp.next()) {
       if (!(alive = wait(&full[rp.b], rp.ph))) break;
@@ -2869,8 +2995,9 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
           const int off = nl[(i + j) * kTile];
 #pragma unroll
           for (int w = 0; w < kVW; ++w) {
-            typename Dot::D d;
-            f[w][j] = dif(w, off, d);
+            const int64_t x = dif(w, off);
+            f[w][j] = fmaf((float)(int)((x + 0x80000000LL) >> 32), cd[w] * 4294967296.f,
+                           (float)(int)x * cd[w]);
             dd[w] = fmaf(f[w][j], f[w][j], dd[w]);
           }
         }
@@ -2889,13 +3016,14 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         float q = 0.f;
 #pragma unroll
         for (int l = 0; l < kSmallM; ++l) q = fmaf(s[w][l], s[w][l], q);
-#pragma unroll
-        for (int i = 0; i < kSmallK; ++i)
-          if (i == k) ts[w][i] = q, ds[w][i] = dd[w];
+        tsd[(k * kVW + w) * 2 * kTile] = q;
+        tsd[(k * kVW + w) * 2 * kTile + kTile] = dd[w];
       }
     }
     if (!alive) break;
     // ---- large stencil: W d in fixed point, complement rows in FP32
+#pragma unroll
+    for (int w = 0; w < kVW; ++w) cd[w] = Dot::c(sc[w]);
     typename Dot::A acc[kVW][NQ3];
     float a32[kVW][MC > 0 ? MC : 1], dL[kVW], norm[kSmallK + 1];
     int stat = 0;
@@ -2917,7 +3045,7 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         const int off = nl[s * kTile];
 #pragma unroll
         for (int w = 0; w < kVW; ++w) {
-          f[w][s] = dif(w, off, d[w][s]);
+          f[w][s] = Dot::split(dif(w, off), sh[w], cd[w], d[w][s]);
           dL[w] = fmaf(f[w][s], f[w][s], dL[w]);
         }
       }
@@ -2953,6 +3081,9 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
 #pragma unroll
     for (int w = 0; w < kVW; ++w) {
       const int v = v0 + w;
+      // units of the differences' FP32 errors (the cell's own state is off by half a unit
+      // of the cell)
+      const float cu = 80.f * exp2i(-sc[w]), cs = 160.f * exp2i(-sc[w] - sh[w]) + exp2i(-sc[w]);
       eT[w] = Dot::exp(kc, sc[w]);
       const float s0 = exp2i(eT[w]);
       // Gauss-point values, and W d in FP32 (y)
@@ -3012,20 +3143,21 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
             wa.t.cs_all * fmaf(Dot::kErr, s0, Dot::kErrD * l2 * exp2i(-kc));
 #pragma unroll
         for (int l = 0; l < MC; ++l) bsum = fmaf(a32[w][l], a32[w][l], bsum);
-        if constexpr (MC > 0) E += dot_bound(norm[kSmallK], dL[w], cu[w], NS);
+        if constexpr (MC > 0) E += dot_bound(norm[kSmallK], dL[w], cu, NS);
         t[kSmallK] = bsum + eps;
         rho = beta_rel_bound(bsum, E * 1.0001f, M, eps);
 #pragma unroll
         for (int k = 0; k < kSmallK; ++k) {
-          t[k] = ts[w][k] + eps;
+          const float tk = tsd[(k * kVW + w) * 2 * kTile];
+          t[k] = tk + eps;
           if ((present >> k) & 1)
-            rho = fmaxf(rho, beta_rel_bound(ts[w][k],
-                                            dot_bound(norm[k], ds[w][k], cu[w], kSmallN),
+            rho = fmaxf(rho, beta_rel_bound(tk,
+                                            dot_bound(norm[k], tsd[(k * kVW + w) * 2 * kTile + kTile], cs, kSmallN),
                                             kSmallM, eps));
         }
         // chi lies within the factor f of its FP32 value under the beta bounds
         // (an eps below the squares of flushed differences decides nothing here)
-        near[w] = a.force_near || direct[w] || !(rho < 0.25f) || (sc[w] > 120 && eps < 1e-30f);
+        near[w] = a.force_near || float_w[w] == 1 || !(rho < 0.25f) || (sc[w] > 120 && eps < 1e-30f);
         const float q = (1.f + rho) * rcp_approx(1.f - fminf(rho, 0.5f));
         const float q2 = q * q;
         const float f = q2 * q2 * q2 * 1.0002f;
@@ -3051,7 +3183,7 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
     for (int w = 0; w < kVW; ++w) {
       if (c < a.n_cell && a.sel_out && !near[w])
         a.sel_out[(int64_t)(v0 + w) * a.n_pad + c] = (uint8_t)sel[w];
-      put[w] = c < a.n_cell && !direct[w] && (near[w] || (sel[w] & 8));
+      put[w] = c < a.n_cell && !float_w[w] && (near[w] || (sel[w] & 8));
       both &= put[w];
     }
     {
@@ -3070,11 +3202,11 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
     // ---- defer what the fixed-point values do not settle
 #pragma unroll
     for (int w = 0; w < kVW; ++w) {
-      const bool def = mine && (near[w] || direct[w] || !(sel[w] & 8));
+      const bool def = mine && (near[w] || float_w[w] || !(sel[w] & 8));
       const unsigned bal = __ballot_sync(0xffffffffu, def);
       if (def)
         mylist[n_def + __popc(bal & ((1u << lane) - 1u))] =
-            make_int2((int)c, (near[w] ? kDefNear : 0) | (direct[w] ? kDefDirect : 0) |
+            make_int2((int)c, (near[w] ? kDefNear : 0) | (float_w[w] ? kDefDirect : 0) |
                                   (sel[w] & 15) * kDefSel | (v0 + w) * kDefVar);
       n_def += __popc(bal);
     }
@@ -4861,7 +4993,7 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
 #pragma unroll
       for (int p = 0; p < NQ3; ++p) {
         const int64_t x = bad ? 0 : to_fix(q[p], sb);
-        Dot::split(x, 0.f, bd[p]);
+        Dot::split(x, 0, 0.f, bd[p]);
         u0b += x;
       }
       if (mx == 0u) sb = -kVjpNone;  // nothing to add: no claim on the unit
