@@ -2336,16 +2336,6 @@ template <typename Dot>
 __device__ __forceinline__ bool own_scale(int es, int ed, int kc, int sc) {
   return max(es + Dot::own_weight(kc), ed) >= Dot::kBits - 2 - sc;
 }
-// x 2^e as a pair (|x| < 2^62; e within the FP32 range less 42)
-__device__ __forceinline__ DF fix_to_df(int64_t x, float s2, float s1, float s0) {
-  const float h = (float)(int)(x >> 42) * s2;
-  const float m = (float)(int)((x >> 21) & 0x1fffff) * s1;
-  const float l = (float)(int)(x & 0x1fffff) * s0;
-  DF r = fast_two_sum(h, m);
-  r.l += l;
-  return fast_two_sum(r.h, r.l);
-}
-
 // pair difference U_s - U_0 of a neighbour (FP32 hi/lo splits of the states)
 __device__ __forceinline__ DF pair_dif(float2 q, float2 u0s) {
   DF t = two_sum(q.x, -u0s.x);
@@ -4704,22 +4694,22 @@ __global__ void __launch_bounds__(128) recon_vjp_df_kernel(const float2* __restr
 // (cells whose large stencil is cut) take d_bar_s = (G_k^T Psi_k^T Uq_bar)_s /
 // n_kept from their (hi, lo) matrices; their stages are streamed only for tiles
 // where some (cell, variable) keeps a directional stencil, a predicate the
-// producer and the consumers evaluate from the same selection bytes.  The sums
-// run in fixed point: Uq_bar in units of its largest per cell (53 bits), the
-// contributions in one unit per tile and variable as 64-bit integers, so their
-// order does not matter.  Each lane adds its d_bar_s to the tile's halo
-// accumulator in shared memory at the slot's halo position (lanes with equal
-// positions in turn, by ranks the host stores next to the positions).  The host
-// assigns the large-stencil members to slots so that the lanes of a tile do not
-// share a cell within a slot, and these slots take one round.  At the end of the
-// tile the accumulator is written as one pair per (halo entry, variable), so the
-// reverse gather reads the few halo entries that hold a cell instead of every
-// stencil slot that holds it.  The tile's Uq_bar block is prefetched with
-// cp.async one tile ahead.  Bound: instruction issue (131,072 cells TENO5 153 us,
-// 8,320 cells TENO6 44; without the block barriers at a tile's ends
-// 151, not worth a second copy of the flags).
+// producer and the consumers evaluate from the same selection bytes.  The products
+// W^T Uq_bar run in fixed point, Uq_bar in 53 bits of the cell's largest; the
+// contributions are pairs, so that each keeps its own precision however much the
+// cotangents of a tile's cells differ.  Each lane adds its d_bar_s to the tile's
+// halo accumulator in shared memory at the slot's halo position (lanes with equal
+// positions in lane order, by ranks the host stores next to the positions; slots
+// in stencil order: deterministic sums).  The host assigns the large-stencil
+// members to slots so that the lanes of a tile do not share a cell within a slot,
+// and these slots take one round.  At the end of the tile the accumulator is
+// written as one pair per (halo entry, variable), so the reverse gather reads the
+// few halo entries that hold a cell instead of every stencil slot that holds it.
+// The tile's Uq_bar block is prefetched with cp.async one tile ahead.  Bound:
+// instruction issue (131,072 cells TENO5 154 us, 152 with integer accumulators of
+// one unit a tile; 8,320 cells TENO6 41, 44 with these; 1,048,352 cells TENO6 1,440
+// and 1,425; pair products took 158, 43 and 1,575).
 constexpr int kRingV = 4;
-constexpr int kVjpNone = -(1 << 16);  // an exponent below every value's
 constexpr int kUbStride = 38;  // doubles per cell in the Uq_bar stage (16-byte rows)
 constexpr int kHaccStride = kHaloMax + 4;  // pairs per variable row (conflict-free transpose)
 
@@ -4744,7 +4734,7 @@ struct VjpPlan {
   static constexpr size_t kHaccOff = kUbOff + kUbBytes;
   static constexpr size_t kHaccBytes = (size_t)4 * kHaccStride * 8;
   static constexpr size_t kBarOff = kHaccOff + kHaccBytes;
-  static constexpr size_t kSmem = kBarOff + 2 * kRingV * 8 + 16 + 32 + 4 * 8 * 4;
+  static constexpr size_t kSmem = kBarOff + 2 * kRingV * 8 + 16 + 16;
   static_assert(NQ3 * 4 <= kUbStride, "Uq_bar row");
   static_assert(kSmallN % kSPS == 0, "directional stencil split");
   static_assert(kMat % 16 == 0 && kUbOff % 16 == 0 && kHaccOff % 16 == 0 && kBarOff % 8 == 0,
@@ -4791,13 +4781,11 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
   using Dot = WPairDot<26>;
   extern __shared__ __align__(128) unsigned char smem[];
   double* ubs = reinterpret_cast<double*>(smem + VP::kUbOff);     // [2][32][kUbStride]
-  int64_t* hacc = reinterpret_cast<int64_t*>(smem + VP::kHaccOff);  // [NV][kHaccStride]
+  float2* hacc = reinterpret_cast<float2*>(smem + VP::kHaccOff);  // [NV][kHaccStride]
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + VP::kBarOff);
   uint64_t* empty = full + kRingV;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + kRingV);
   int* need = const_cast<int*>(abort_flag) + 4;  // [NV] per-variable small-stencil flags
-  int* unit = need + NV;                         // [NV] exponents of the accumulators' units
-  unsigned* nanm = reinterpret_cast<unsigned*>(unit + NV);  // [NV][8] halo cells that take a NaN
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_tiles = (n_cell + kTile - 1) / kTile;
   if (threadIdx.x == 0) {
@@ -4886,20 +4874,18 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
     }
     cp_async_commit();
   };
-  int64_t* hrow = hacc + v * kHaccStride;
-  // add t at the halo position of code (bits 0-7); lanes with equal
-  // positions in turn, by their precomputed ranks (bits 8-12); a lane whose
-  // cotangents hold an infinity or a NaN marks the halo cell instead
-  auto accumulate = [&](bool act, bool bad, int code, int64_t t) {
+  float2* hrow = hacc + v * kHaccStride;
+  // add t at the halo position of code (bits 0-7); lanes with equal positions
+  // in the order of their precomputed ranks (bits 8-12)
+  auto accumulate = [&](bool act, int code, DF t) {
     const int hp = code & kHaloPosMask;
     const unsigned rank = (unsigned)code >> 8;
     const unsigned rmax = __reduce_max_sync(0xffffffffu, act ? rank : 0u);
     for (unsigned r = 0; r <= rmax; ++r) {
       if (act && rank == r) {
-        if (bad)
-          atomicOr(&nanm[v * 8 + (hp >> 5)], 1u << (hp & 31));
-        else
-          hrow[hp] += t;
+        const float2 q = hrow[hp];
+        const DF x = DF{q.x, q.y} + t;
+        hrow[hp] = make_float2(x.h, x.l);
       }
       __syncwarp();
     }
@@ -4933,8 +4919,7 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
     const int h0 = h0n, H = Hn, kc = kcn;
     const uint8_t sel = seln;
     pre(nxt, h0n, Hn, seln, kcn);
-    for (int i = lane; i < H; i += kTile) hrow[i] = 0;
-    if (lane < 8) nanm[v * 8 + lane] = 0u;
+    for (int i = lane; i < H; i += kTile) hrow[i] = make_float2(0.f, 0.f);
     const int64_t c = tile * kTile + lane;
     const bool valid = c < n_cell;
     const bool vs = __any_sync(0xffffffffu, valid && vjp_needs_small(sel));
@@ -4950,11 +4935,9 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
     // polynomials (first kSmallM basis functions) in pairs, where the block
     // needs them
     typename Dot::D bd[NQ3];
-    int sb = 0;
-    int64_t u0b = 0;
-    bool bad = false;
+    float sh, sl;  // scales of a contribution's parts
+    DF u0b = {0.f, 0.f};
     DF cbs[kSmallM];
-    int ec = kVjpNone;  // |directional contribution| < 2^ec
 #pragma unroll
     for (int l = 0; l < kSmallM; ++l) cbs[l] = {0.f, 0.f};
     {
@@ -4966,49 +4949,34 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
       for (int p = 0; p < NQ3; ++p) {
         q[p] = valid ? us[p * NV] : make_float2(0.f, 0.f);
         mx = max(mx, mag_bits(q[p]));
+        u0b = u0b + DF{q[p].x, q[p].y};
       }
-      if (small && valid && !large && nd) {
+      if (small && valid && !large) {
 #pragma unroll
         for (int p = 0; p < NQ3; ++p)
 #pragma unroll
           for (int l = 0; l < kSmallM; ++l)
             df_mac(cbs[l], ev.psi[p * kMaxM + l], DF{q[p].x, q[p].y});
-        float cm = 0.f, nm = 0.f;
 #pragma unroll
-        for (int l = 0; l < kSmallM; ++l) {
-          cbs[l] = df_norm(cbs[l]);
-          cm = fmaxf(cm, fabsf(cbs[l].h));
-        }
-#pragma unroll
-        for (int k = 0; k < kSmallK; ++k)
-          nm = fmaxf(nm, __int_as_float(wstat[(tile * kWStat + k) * kTile + lane]));
-        // |sum_l G_ls cb_l| <= max|cb| times the largest column sum
-        ec = mag_exp<float2>((unsigned)__float_as_int(cm)) +
-             mag_exp<float2>((unsigned)__float_as_int(nm)) + 3;
+        for (int l = 0; l < kSmallM; ++l) cbs[l] = df_norm(cbs[l]);
       }
       const int e = mag_exp<float2>(mx);
-      bad = e == kFixExpBad || ec >= kFixExpBad / 2;
-      sb = bad ? 0 : 52 - e;
-      if (bad) ec = kVjpNone;
+      const bool bad = e == kFixExpBad;
+      const int sb = bad ? 0 : 52 - e;
 #pragma unroll
-      for (int p = 0; p < NQ3; ++p) {
-        const int64_t x = bad ? 0 : to_fix(q[p], sb);
-        Dot::split(x, 0, 0.f, bd[p]);
-        u0b += x;
-      }
-      if (mx == 0u) sb = -kVjpNone;  // nothing to add: no claim on the unit
+      for (int p = 0; p < NQ3; ++p) Dot::split(bad ? 0 : to_fix(q[p], sb), 0, 0.f, bd[p]);
+      // (zero where the large stencil gives nothing; an infinity or a NaN goes to
+      // every cell of the stencil; denormal for cotangents below 2^-104)
+      const int uT = Dot::exp(kc, sb);
+      auto scale = [&](int x) {
+        if (!large) return 0.f;
+        if (bad) return __int_as_float(0x7fffffff);
+        return x >= -126 ? exp2i(x) : (x < -149 ? 0.f : __int_as_float(1 << (x + 149)));
+      };
+      sh = scale(uT + 32);
+      sl = scale(uT + 40);
     }
-    // the tile's accumulator unit 2^Ec of this variable: every contribution
-    // (W^T Uq_bar: |T| < 9 2^31 2^27 < 2^61.2 in units of 2^(26 - kc - sb)) stays below
-    // 2^56.2 units, so the at most 96 that meet in one halo cell, and a cell's
-    // own sum over its slots, stay below 2^63
-    const int uT = Dot::exp(kc, sb);
-    int Ec = bad ? kVjpNone : max(4 - sb, ec - 56);
-    if (large && !bad) Ec = max(Ec, uT + 5);
-    Ec = __reduce_max_sync(0xffffffffu, Ec);
-    if (lane == 0) unit[v] = Ec;
-    const int shT = Ec - uT;  // >= 5 on large lanes
-    int64_t tot = 0;
+    DF tot = {0.f, 0.f};
     for (int j = 0; j < n_stages; ++j, ++g) {
       const int b = (int)(g % kRingV);
       int slot0, nslot, k, bytes;
@@ -5024,13 +4992,19 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
       }
       const unsigned char* buf = smem + (size_t)b * VP::kMat;
       const uint16_t* nl = reinterpret_cast<const uint16_t*>(buf + VP::kNOff) + lane;
+      auto add = [&](bool on, int s, DF t) {
+        accumulate(on, nl[s * kTile], t);
+        const DF q = two_sum(tot.h, t.h);  // running sum, renormalised at the end
+        tot.h = q.h;
+        tot.l += q.l + t.l;
+      };
       if (dead) {
         // skip the stage
       } else if (k < 0) {
         if (__any_sync(0xffffffffu, large)) {
           // the stage's slot values first (independent chains), then their
           // accumulation slot by slot
-          int64_t ts[VP::kLPS];
+          DF ts[VP::kLPS];
 #pragma unroll
           for (int s = 0; s < VP::kLPS; ++s) {
             typename Dot::A acc;
@@ -5041,17 +5015,17 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
                   Dot::entry(w_entry<VP::kLay * NQ3>(
                       buf + s / VP::kLay * VP::kLay * VP::kSlotW, lane, s % VP::kLay * NQ3 + p)),
                   bd[p]);
-            // (|x| < 2^35: rounded to 16 units)
+            // |T| < 9 2^31 2^27 < 2^61.2 units of 2^(26 - kc - sb) (its FP32 part below
+            // 2^35, rounded to 16 units) as the pair h 2^32 + l: h its upper word
             const int64_t T = acc.hh + (int64_t)__float2int_rn(acc.x * 0.0625f) * 16;
-            ts[s] = large && s < nslot && !bad && shT < 63 ? (T + ((int64_t)1 << (shT - 1))) >> shT : 0;
+            const int hi = (int)(T >> 32);
+            const float h = (float)hi;
+            const float l = fmaf((float)(hi - (int)h), 0x1p-8f, (float)(unsigned)T * 0x1p-40f);
+            ts[s] = DF{h * sh, l * sl};
           }
 #pragma unroll
-          for (int s = 0; s < VP::kLPS; ++s) {
-            if (s < nslot) {
-              accumulate(large, bad, nl[s * kTile], ts[s]);
-              tot += ts[s];
-            }
-          }
+          for (int s = 0; s < VP::kLPS; ++s)
+            if (s < nslot) add(large, s, ts[s]);
         }
       } else {
         const bool on = valid && !large && ((sel >> k) & 1);
@@ -5059,38 +5033,25 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
           const float2* mat = reinterpret_cast<const float2*>(buf) + lane;
 #pragma unroll
           for (int s = 0; s < VP::kSPS; ++s) {
-            int64_t t = 0;
-            if (on && !bad) {
-              DF q = {0.f, 0.f};
+            DF t = {0.f, 0.f};
+            if (on) {
 #pragma unroll
-              for (int l = 0; l < kSmallM; ++l) df_mac(q, mat[(s * kSmallM + l) * kTile], cbs[l]);
-              q = df_div_small(df_norm(q), nd);
-              t = to_fix(make_float2(q.h, q.l), -Ec);
+              for (int l = 0; l < kSmallM; ++l) df_mac(t, mat[(s * kSmallM + l) * kTile], cbs[l]);
+              t = df_div_small(df_norm(t), nd);
             }
-            accumulate(on, bad, nl[s * kTile], t);
-            tot += t;
+            add(on, s, t);
           }
         }
       }
       __syncwarp();
       if (lane == 0 && !dead) mbar_arrive(&empty[b]);
     }
-    if (valid && !dead) {
-      // sum_p Uq_bar_p - sum_s d_bar_s (the first in units of 2^-sb)
-      const int sh = Ec + sb;
-      const int64_t own = !bad && sh < 63 ? (u0b + ((int64_t)1 << (sh - 1))) >> sh : 0;
-      u_self[(int64_t)v * n_pad + c] =
-          bad ? __longlong_as_double(0x7ff8000000000000LL) : ldexp((double)(own - tot), Ec);
-    }
+    if (valid && !dead) u_self[(int64_t)v * n_pad + c] = to_d(u0b - df_norm(tot));
     consumer_sync();  // every variable's accumulator is complete
     if (!dead) {
       float2* dst = part + (int64_t)h0 * NV;
-      for (int e = tid; e < H * NV; e += kConsumers * kTile) {
-        const int w = e & 3, i = e >> 2, Ew = unit[w];
-        DF r = fix_to_df(hacc[w * kHaccStride + i], exp2i(Ew + 42), exp2i(Ew + 21), exp2i(Ew));
-        if ((nanm[w * 8 + (i >> 5)] >> (i & 31)) & 1) r = DF{__int_as_float(0x7fffffff), 0.f};
-        dst[e] = make_float2(r.h, r.l);
-      }
+      for (int e = tid; e < H * NV; e += kConsumers * kTile)
+        dst[e] = hacc[(e & 3) * kHaccStride + (e >> 2)];
     }
   }
   cp_async_wait<0>();
