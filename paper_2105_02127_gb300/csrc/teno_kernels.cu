@@ -4417,43 +4417,63 @@ __device__ __forceinline__ void store_bar(double* base, int i, S x) {
 // (8,320 cells TENO6, HLLC: 136 us a residual's adjoint, 122 now).  The states
 // load while the cotangents are formed (1,048,352 cells TENO6: 706 us, 746 with
 // the loads after the barrier; 32 faces a block 722).
-template <int NV, int NQ, int FLUX, typename TQ, typename S, int ND>
-__global__ void __launch_bounds__(kFluxFaces * NQ, 384 / (kFluxFaces * NQ))
+// kTurn: one thread per face, its points in turn, 128 faces a block (HLL in pairs).
+// At meshes that fill the machine many times over the latency no longer counts
+// and three times the faces in flight cover the scattered reads better: from
+// 524,288 faces on (points side by side / in turn: 393k faces 184 / 185 us, 786k
+// 358 / 344, 1.57M 704 / 667, 12.6M 5,542 / 5,288).  HLLC and FP64 hold a face's
+// cotangents through the sweeps at the price of spills: 786k faces 413 / 435 and
+// 1,618 / 1,660.
+constexpr int64_t kTurnFaces = (int64_t)1 << 19;
+constexpr int kTurnBlock = 128;
+template <int NV, int NQ, int FLUX, typename TQ, typename S, int ND, bool kTurn>
+__global__ void __launch_bounds__(kTurn ? kTurnBlock : kFluxFaces * NQ,
+                                  kTurn ? 3 : 384 / (kFluxFaces * NQ))
     face_flux_vjp_kernel(const VjpArgs a, const TQ* Uq, const double* w,
                          double* __restrict__ Uq_bar) {
   pdl_wait();
   static_assert((2 * NV) % ND == 0, "directions per pass must divide 2 NV");
   using D = Dual<ND, S>;
-  __shared__ S sK[kFluxFaces * NV];
-  const int64_t f0 = (int64_t)blockIdx.x * kFluxFaces;
+  __shared__ S sK[kTurn ? 1 : kFluxFaces * NV];
+  const int64_t f0 = (int64_t)blockIdx.x * (kTurn ? kTurnBlock : kFluxFaces);
   // Kbar in FP64 from the FP64 weights, once per face in the flux scalar type
-  for (int e = threadIdx.x; e < kFluxFaces * NV; e += kFluxFaces * NQ) {
-    const int64_t f = f0 + e % kFluxFaces;
-    const int v = e / kFluxFaces;
-    if (f >= a.n_face) continue;
+  auto kbar = [&](int64_t f, int v) {
     const int o = a.f_cells[2 * f], n = a.f_cells[2 * f + 1];
     double kb = -w[v * a.n_pad + o] * a.inv_area[o];
     if (n >= 0) kb = fma(w[v * a.n_pad + n], a.inv_area[n], kb);
-    sK[e % kFluxFaces * NV + v] = cst<S>(kb);
-  }
-  const int k = threadIdx.x % NQ;
-  const bool in = f0 + threadIdx.x / NQ < a.n_face;  // (past the end: the last face's loads)
-  const int64_t f = in ? f0 + threadIdx.x / NQ : a.n_face - 1;
+    return cst<S>(kb);
+  };
+  if constexpr (!kTurn)
+    for (int e = threadIdx.x; e < kFluxFaces * NV; e += kFluxFaces * NQ) {
+      const int64_t f = f0 + e % kFluxFaces;
+      if (f < a.n_face) sK[e % kFluxFaces * NV + e / kFluxFaces] = kbar(f, e / kFluxFaces);
+    }
+  const int lf = kTurn ? threadIdx.x : threadIdx.x / NQ;
+  const bool in = f0 + lf < a.n_face;  // (past the end: the last face's loads)
+  if (kTurn && !in) return;
+  const int64_t f = in ? f0 + lf : a.n_face - 1;
   const int o = a.f_cells[2 * f], n = a.f_cells[2 * f + 1];
   const int eo = a.f_edges[2 * f], en = a.f_edges[2 * f + 1];
   const double nx = a.f_geom[5 * f], ny = a.f_geom[5 * f + 1], len = a.f_geom[5 * f + 2];
-  const S* Kb = sK + threadIdx.x / NQ * NV;
+  S kf[NV];
+  if constexpr (kTurn) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) kf[v] = kbar(f, v);
+  }
+  const S* Kb = kTurn ? kf : sK + lf * NV;
   const int n_pass = ((n >= 0 ? 2 * NV : NV) + ND - 1) / ND;
   RiemannK<S> rks;
   S tl;  // |A| in the flux scalar type
   face_k<S>(a.f_geom, a.f_geom2, f, a.gamma, a.g2, a.gm12, rks, tl);
   const RiemannK<D> rk = riemann_k_dual<ND, S>(rks);
-  {
+  for (int k = kTurn ? 0 : threadIdx.x % NQ; k < NQ; k += kTurn ? 1 : NQ) {
     TQ ul[NV], ur[NV];
     ld_group<NV>(Uq + ((int64_t)(o * 3 + eo) * NQ + k) * NV, ul);
     if (n >= 0) ld_group<NV>(Uq + ((int64_t)(n * 3 + en) * NQ + (NQ - 1 - k)) * NV, ur);
-    __syncthreads();  // the cotangents, while the states load
-    if (!in) return;
+    if constexpr (!kTurn) {
+      __syncthreads();  // the cotangents, while the states load
+      if (!in) return;
+    }
     // x of the Gauss point (ghost states and the scalar field only)
     auto xq = [&]() { return a.f_geom[5 * f + 3] - ny * len * a.gt[k]; };
     const S wl = gauss_w<S>(a.gw[k], a.gw2[k]) * tl;
@@ -5641,11 +5661,18 @@ cudaError_t launch_face_flux_vjp(const DeviceMesh& dm, const void* Uq, const dou
     // all 2 NV directions of an interior face in one pass
     if constexpr (std::is_same<TQ, DF>::value) {
       constexpr int ND = NV < kVjpDirs ? NV : kVjpDirs;
-      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, DF, ND>, grid, kFluxFaces * NQ, 0, st, a,
+      if constexpr (NV == 4 && FL == TENO_FLUX_HLL)
+        if (dm.n_face >= kTurnFaces) {
+          launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, DF, ND, true>,
+                 (unsigned)((dm.n_face + kTurnBlock - 1) / kTurnBlock), kTurnBlock, 0, st, a,
+                 (const TQ*)Uq, w, Uq_bar);
+          return;
+        }
+      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, DF, ND, false>, grid, kFluxFaces * NQ, 0, st, a,
              (const TQ*)Uq, w, Uq_bar);
     } else {
-      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, double, 2 * NV>, grid, kFluxFaces * NQ, 0, st, a,
-             (const TQ*)Uq, w, Uq_bar);
+      launch(face_flux_vjp_kernel<NV, NQ, FL, TQ, double, 2 * NV, false>, grid, kFluxFaces * NQ, 0,
+             st, a, (const TQ*)Uq, w, Uq_bar);
     }
   };
   using I1 = std::integral_constant<int, 1>;
