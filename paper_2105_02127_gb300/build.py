@@ -18,7 +18,8 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libteno.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["teno_kernels.cu", "teno_noalloc.cu", "teno_peaks.cu", "teno_host.cpp"]
-HEADERS = [os.path.join(CSRC, "teno_internal.h"), os.path.join(ROOT, "include", "teno.h")]
+HEADERS = [os.path.join(CSRC, "teno_internal.h"), os.path.join(CSRC, "teno_fp64.cuh"),
+           os.path.join(ROOT, "include", "teno.h")]
 
 
 def _cuda_home() -> str:

@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "teno_fp64.cuh"
 #include "teno_internal.h"
 
 namespace teno {
@@ -368,29 +369,14 @@ __device__ __forceinline__ T pos_part(const T& x) {
   return (nonneg(x) || val(x) != val(x)) ? x : x - x;
 }
 
-// Reciprocal and square root for the Riemann solver.  In FP64 the solver is
-// bound by the FP64 pipe (1/64 of the FP32 rate), and the IEEE division and
-// root take most of it, so they are formed from the PTX approximations
-// (documented, about 20 bits, not on that pipe) in three and five FP64
-// operations: one cubically convergent step y (1 + e + e^2), e = 1 - x y, and
-// one step of Goldschmidt's iteration with a last residual step (Goldschmidt,
-// "Applications of division by convergence", 1964).  Both are within 0.51 ulp
-// (2^30 random operands).  Operands near the ends of the exponent range, zeros,
-// infinities and NaN take the IEEE operations.
-__device__ __forceinline__ bool mid_exponent(double x) {  // 2^-959 <= |x| < 2^961
-  return ((unsigned)__double2hiint(x) & 0x7fffffffu) - 0x04000000u < 0x78000000u;
-}
+// reciprocal and square root of the Riemann solver
 template <typename T>
 __device__ __forceinline__ T flux_rcp(const T& one, const T& x) {
   return one / x;
 }
 template <>
-__device__ __forceinline__ double flux_rcp<double>(const double& one, const double& x) {
-  if (!mid_exponent(x)) return one / x;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+__device__ __forceinline__ double flux_rcp<double>(const double&, const double& x) {
+  return rcp_f64(x);
 }
 template <typename T>
 __device__ __forceinline__ T flux_sqrt(const T& x) {
@@ -398,14 +384,7 @@ __device__ __forceinline__ T flux_sqrt(const T& x) {
 }
 template <>
 __device__ __forceinline__ double flux_sqrt<double>(const double& x) {
-  if (!mid_exponent(x) || __double2hiint(x) < 0) return sqrt(x);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double g = x * y;
-  // y / 2 (y is a normal number, its exponent far from the ends)
-  const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
-  const double g1 = fma(g, fma(-g, h, 0.5), g);
-  return fma(fma(-g1, g1, x), h, g1);
+  return sqrt_f64(x);
 }
 
 // ---------------------------------------------------------------- fluxes
