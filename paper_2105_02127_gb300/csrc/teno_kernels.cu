@@ -4705,8 +4705,8 @@ __global__ void __launch_bounds__(128) recon_vjp_df_kernel(const float2* __restr
 // written as one pair per (halo entry, variable), so the reverse gather reads the
 // few halo entries that hold a cell instead of every stencil slot that holds it.
 // The tile's Uq_bar block is prefetched with cp.async one tile ahead.  Bound:
-// instruction issue (131,072 cells TENO5 154 us, 152 with integer accumulators of
-// one unit a tile; 8,320 cells TENO6 41, 44 with these; 1,048,352 cells TENO6 1,440
+// instruction issue (131,072 cells TENO5 158 us, 152 with integer accumulators of
+// one unit a tile; 8,320 cells TENO6 42, 44 with these; 1,048,352 cells TENO6 1,485
 // and 1,425; pair products took 158, 43 and 1,575).
 constexpr int kRingV = 4;
 constexpr int kUbStride = 38;  // doubles per cell in the Uq_bar stage (16-byte rows)
@@ -4934,7 +4934,7 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
     // polynomials (first kSmallM basis functions) in pairs, where the block
     // needs them
     typename Dot::D bd[NQ3];
-    float sh, sl;  // scales of a contribution's parts
+    float sT;  // scale of a contribution
     DF u0b = {0.f, 0.f};
     DF cbs[kSmallM];
 #pragma unroll
@@ -4965,15 +4965,11 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
 #pragma unroll
       for (int p = 0; p < NQ3; ++p) Dot::split(bad ? 0 : to_fix(q[p], sb), 0, 0.f, bd[p]);
       // (zero where the large stencil gives nothing; an infinity or a NaN goes to
-      // every cell of the stencil; denormal for cotangents below 2^-104)
+      // every cell of the stencil; denormal for cotangents below 2^-114)
       const int uT = Dot::exp(kc, sb);
-      auto scale = [&](int x) {
-        if (!large) return 0.f;
-        if (bad) return __int_as_float(0x7fffffff);
-        return x >= -126 ? exp2i(x) : (x < -149 ? 0.f : __int_as_float(1 << (x + 149)));
-      };
-      sh = scale(uT + 32);
-      sl = scale(uT + 40);
+      sT = uT + 42 >= -126 ? exp2i(uT + 42) : __int_as_float(1 << max(uT + 42 + 149, 0));
+      if (!large) sT = 0.f;
+      if (large && bad) sT = __int_as_float(0x7fffffff);
     }
     DF tot = {0.f, 0.f};
     for (int j = 0; j < n_stages; ++j, ++g) {
@@ -5015,12 +5011,13 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), 3)
                       buf + s / VP::kLay * VP::kLay * VP::kSlotW, lane, s % VP::kLay * NQ3 + p)),
                   bd[p]);
             // |T| < 9 2^31 2^27 < 2^61.2 units of 2^(26 - kc - sb) (its FP32 part below
-            // 2^35, rounded to 16 units) as the pair h 2^32 + l: h its upper word
+            // 2^35, rounded to 16 units) as a pair, of limbs of 21 bits that FP32 holds
             const int64_t T = acc.hh + (int64_t)__float2int_rn(acc.x * 0.0625f) * 16;
-            const int hi = (int)(T >> 32);
-            const float h = (float)hi;
-            const float l = fmaf((float)(hi - (int)h), 0x1p-8f, (float)(unsigned)T * 0x1p-40f);
-            ts[s] = DF{h * sh, l * sl};
+            const float h2 = (float)(int)(T >> 42);
+            const float h1 = (float)((int)(T >> 21) & 0x1fffff) * 0x1p-21f;
+            const float h0 = (float)((int)T & 0x1fffff) * 0x1p-42f;
+            const DF x = fast_two_sum(h2, h1);
+            ts[s] = DF{x.h * sT, (x.l + h0) * sT};
           }
 #pragma unroll
           for (int s = 0; s < VP::kLPS; ++s)
