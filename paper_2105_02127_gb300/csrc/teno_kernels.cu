@@ -2017,9 +2017,9 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), kDF ? 2 : 0)
 //    multiply-adds (pairs).  The states' rounding to the tile's unit is one of
 //    the largest difference in the tile, up to 2^-51 of it (pairs) or 2^-57; where
 //    that is more than some cell's own rounding (the small side of a jump that
-//    the tile holds, own_scale) the tile's integers take the 64 bits there are and
-//    each lane the bits of them that its cell needs, and cells for which these do
-//    not do either are summed in floating point (w_direct);
+//    the tile holds, own_scale) the tile's integers take 62 bits and each lane the
+//    bits of them that its cell needs, and cells for which these do not do either
+//    are summed in floating point (w_direct);
 //  - the smoothness indicators feed only the cutoff decision.  beta = |a|^2
 //    for the coefficients a = G d; the part of a in the row space of Psi' is
 //    a linear image T y of the values y = W d that are known anyway, so only
@@ -2034,10 +2034,11 @@ __global__ void __launch_bounds__(kTile * (kConsumers + 1), kDF ? 2 : 0)
 // cell at a time by all lanes, 32 directional cells one per lane, so that their
 // chains of loads stall the warp once and not per cell and slot.
 // Bound: HBM and issue at large meshes (1.56 GB a launch at 262,088 cells TENO6:
-// 318 us; with pair products, all rows and per-tile block barriers 470 us), the
-// FP64 path by issue at four consumer warps a block and four blocks (131,072
-// cells: 234 us; FP64 multiply-adds 608 us), small meshes by the time of one tile
-// (2,046 cells TENO5: 39 us, 52 before).
+// 341 us, 318 without the look at the cells' own scales; with pair products, all
+// rows and per-tile block barriers 470 us), the FP64 path by issue at four
+// consumer warps a block and four blocks (131,072 cells: 235 us; FP64
+// multiply-adds 608 us), small meshes by the time of one tile (2,046 cells TENO5:
+// 39 us, 52 before).
 
 // Variables a consumer warp takes: two on the pair path, where the sums of
 // both share every shared-memory read of W and of the rows (262,088 cells,
@@ -2544,14 +2545,6 @@ __device__ __noinline__ int w_screen(float t0, float t1, float t2, float tK, int
 constexpr int kDefNear = 1, kDefDirect = 2, kDefSel = 8;  // selection from bit 3
 constexpr int kDefVar = 256;                              // variable from bit 8
 
-// the values of two variables of a point, 16 bytes
-__device__ __forceinline__ void st_two(float2* p, float2 x, float2 y) {
-  *reinterpret_cast<float4*>(p) = make_float4(x.x, x.y, y.x, y.y);
-}
-__device__ __forceinline__ void st_two(double* p, double x, double y) {
-  *reinterpret_cast<double2*>(p) = make_double2(x, y);
-}
-
 struct WArgs {
   const void* psi;    // Psi' as pairs or FP64
   const float* g32;   // FP32 rows of the complement and the directional stencils
@@ -2838,8 +2831,9 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         }
       // a cell's scale (own_scale), first without its differences
       const unsigned char* o2 = own2 + (it & 1) * P::kOwn2;
-      const int kc =
-          kN ? (int)(int16_t)(reinterpret_cast<const int32_t*>(o2 + 2 * kTile * 8)[lane] & 0xffff) : 0;
+      int kc = 0;
+      if constexpr (kN)
+        kc = (int)(int16_t)(reinterpret_cast<const int32_t*>(o2 + 2 * kTile * 8)[lane] & 0xffff);
       int es[kVW];
       bool coarse = false;
 #pragma unroll
@@ -2854,7 +2848,8 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         if (v0 + w == 1 || v0 + w == 2) {  // rho and E, in either order
           const double* x = reinterpret_cast<const double*>(o2) + lane;
           const double y = kN ? x[kTile] : hv[(kVW - 1 - w) * P::kHaloRow + kHaloMax + lane];
-          es[w] = max(es[w], ((mag_exp<double>(mag_bits(*x)) + mag_exp<double>(mag_bits(y))) >> 1) - 6);
+          const int e2 = mag_exp<double>(mag_bits(*x)) + mag_exp<double>(mag_bits(y));
+          es[w] = max(es[w], (e2 >> 1) - 6);
         }
         coarse |= mine && mx[w] && !float_w[w] && !own_scale<Dot>(es[w], -5000, kc, sc[w]);
       }
@@ -2912,10 +2907,11 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         for (int i = 0; i < n_mine; ++i) {
           const int id = __ldg(ids + i * kTile);
 #pragma unroll
-          for (int w = 0; w < kVW; ++w)
-            hv[w * P::kHaloRow + lane + i * kTile] = __longlong_as_double(
-                float_w[w] ? 0
-                           : to_fix_mod(a.U[(int64_t)(v0 + w) * a.n_pad + id], sc[w] + 61 - Dot::kBits));
+          for (int w = 0; w < kVW; ++w) {
+            const double u = a.U[(int64_t)(v0 + w) * a.n_pad + id];
+            hv[w * P::kHaloRow + lane + i * kTile] =
+                __longlong_as_double(float_w[w] ? 0 : to_fix_mod(u, sc[w] + 61 - Dot::kBits));
+          }
         }
 #pragma unroll
         for (int w = 0; w < kVW; ++w) {
@@ -3117,16 +3113,16 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         rho = beta_rel_bound(bsum, E * 1.0001f, M, eps);
 #pragma unroll
         for (int k = 0; k < kSmallK; ++k) {
-          const float tk = tsd[(k * kVW + w) * 2 * kTile];
-          t[k] = tk + eps;
+          const float* td = tsd + (k * kVW + w) * 2 * kTile;
+          t[k] = td[0] + eps;
           if ((present >> k) & 1)
-            rho = fmaxf(rho, beta_rel_bound(tk,
-                                            dot_bound(norm[k], tsd[(k * kVW + w) * 2 * kTile + kTile], cs, kSmallN),
+            rho = fmaxf(rho, beta_rel_bound(td[0], dot_bound(norm[k], td[kTile], cs, kSmallN),
                                             kSmallM, eps));
         }
         // chi lies within the factor f of its FP32 value under the beta bounds
         // (an eps below the squares of flushed differences decides nothing here)
-        near[w] = a.force_near || float_w[w] == 1 || !(rho < 0.25f) || (sc[w] > 120 && eps < 1e-30f);
+        near[w] = a.force_near || float_w[w] == 1 || !(rho < 0.25f) ||
+                  (sc[w] > 120 && eps < 1e-30f);
         const float q = (1.f + rho) * rcp_approx(1.f - fminf(rho, 0.5f));
         const float q2 = q * q;
         const float f = q2 * q2 * q2 * 1.0002f;
@@ -3157,10 +3153,16 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
     }
     {
       HT* __restrict__ out = reinterpret_cast<HT*>(a.Uq) + c * kPer + v0;
-      if (kVW == 2 && both) {
+      bool each = true;
+      if constexpr (kVW == 2)  // both variables of a point in 16 bytes
+        if (both) {
+          each = false;
 #pragma unroll
-        for (int p = 0; p < NQ3; ++p) st_two(out + p * NV, val[0][p], val[kVW - 1][p]);
-      } else {
+          for (int p = 0; p < NQ3; ++p)
+            *reinterpret_cast<float4*>(out + p * NV) =
+                make_float4(val[0][p].x, val[0][p].y, val[1][p].x, val[1][p].y);
+        }
+      if (each) {
 #pragma unroll
         for (int w = 0; w < kVW; ++w)
           if (put[w])
@@ -3206,7 +3208,7 @@ template <int M, int NS, int NQ, int NV>
 struct TPlan {
   static constexpr int kVW = NV == 4 ? 2 : 1, kWarps = NV / kVW;  // variables a warp
   static constexpr int kBlocks = NV == 1 ? 6 : 4;
-  static constexpr int kEsz = 4, kVec = 4;
+  static constexpr int kEsz = 4;
   static constexpr int kLPS = tile_lps(NS), kSPS = kSmallN;
   static constexpr int kNL = NS / kLPS;
   static constexpr int kStages = kSmallK + kNL;  // the directional stencils first
@@ -4032,7 +4034,7 @@ __device__ __forceinline__ T gauss_w(double w, float2 w2) {
 // large meshes, the latency of one solve at small ones, where a thread that
 // took a face's points in turn ran three of them in a row (32,768 cells TENO5
 // pairs: 18.6 us for three points a thread, 12.8 now; 262,088 cells TENO6:
-// 63 to 53.6; FP64, 131,072 cells: 199 to 174, 167 with flux_rcp / flux_sqrt).
+// 63 to 53.6; FP64, 131,072 cells: 199 to 174, 139 with the FP64 solver's own form).
 constexpr int kFluxFaces = 64;
 
 template <int NV, int NQ, int FLUX, typename T>
@@ -5263,11 +5265,11 @@ cudaError_t launch_char_finish(const DeviceMesh& dm, const double* U, void* Uq, 
       if constexpr (std::is_same<TQ, double>::value)
         launch(char_finish_kernel<M, NQ, TQ>, grid, 128, 0, st, dm.coef_out, U, dm.smask,
                dm.c_faces, dm.f_geom, dm.eval, (TQ*)Uq, dm.n_recon,
-            dm.n_pad, dm.gamma, dm.ct, dm.eps, dm.linear);
+               dm.n_pad, dm.gamma, dm.ct, dm.eps, dm.linear);
       else
         launch(char_finish_df_kernel<M, NQ, TQ>, grid, 128, 0, st,
                reinterpret_cast<const float2*>(dm.coef_out), U, dm.smask, dm.c_faces, dm.f_geom,
-            dm.eval_df, (TQ*)Uq, dm.n_recon, dm.n_pad, dm.gamma, dm.ct, dm.eps, dm.linear);
+               dm.eval_df, (TQ*)Uq, dm.n_recon, dm.n_pad, dm.gamma, dm.ct, dm.eps, dm.linear);
       return cudaGetLastError();
     };
     if (dm.precision == TENO_FP64) return go(TypeTag<DF>{});
@@ -5459,13 +5461,13 @@ cudaError_t launch_layer_fill(const DeviceMesh& dm, const double* U, void* Uq, c
     constexpr int NV = decltype(nvc)::value, NQ3 = 3 * decltype(nqc)::value;
     if (dm.precision == TENO_FP64)
       launch(layer_fill_kernel<NV, NQ3, DF>, grid, 256, 0, st, U, (DF*)Uq, dm.fo_list, dm.fo_n,
-                                                            dm.n_pad);
+             dm.n_pad);
     else if (dm.precision == TENO_FP32_MIXED)
       launch(layer_fill_kernel<NV, NQ3, float>, grid, 256, 0, st, U, (float*)Uq, dm.fo_list,
-                                                              dm.fo_n, dm.n_pad);
+             dm.fo_n, dm.n_pad);
     else
       launch(layer_fill_kernel<NV, NQ3, double>, grid, 256, 0, st, U, (double*)Uq, dm.fo_list,
-                                                               dm.fo_n, dm.n_pad);
+             dm.fo_n, dm.n_pad);
   };
   using I1 = std::integral_constant<int, 1>;
   using I4 = std::integral_constant<int, 4>;
@@ -5539,7 +5541,7 @@ cudaError_t launch_halo_unpack(double* U, int64_t ld, const int32_t* idx, int64_
 
 cudaError_t launch_split(const DeviceMesh& dm, const double* U, float2* Us, cudaStream_t st) {
   launch(split_kernel, (unsigned)((dm.n_cell + 255) / 256), 256, 0, st, U, Us, dm.n_cell, dm.n_pad,
-                                                                    dm.n_var);
+         dm.n_var);
   return cudaGetLastError();
 }
 
@@ -5553,11 +5555,11 @@ cudaError_t launch_max_lambda(const DeviceMesh& dm, const double* U, double* max
   if (dm.n_var == 1)
     launch(max_lambda_kernel<1>, (unsigned)blocks, 256, 0, st, U, dm.cfl_len, dm.n_update, dm.n_pad,
            dm.gamma, adv, dm.cell_speed,
-        (unsigned long long*)max_lam);
+           (unsigned long long*)max_lam);
   else
     launch(max_lambda_kernel<4>, (unsigned)blocks, 256, 0, st, U, dm.cfl_len, dm.n_update, dm.n_pad,
            dm.gamma, adv, nullptr,
-        (unsigned long long*)max_lam);
+           (unsigned long long*)max_lam);
   return cudaGetLastError();
 }
 
@@ -5570,7 +5572,7 @@ cudaError_t launch_max_lambda_split(const DeviceMesh& dm, const float2* Us, doub
   if (blocks > 152 * 8) blocks = 152 * 8;
   launch(max_lambda_split_kernel, (unsigned)blocks, 256, 0, st, Us, dm.cfl_ilen2, dm.n_update,
          dm.n_pad, split2(dm.gamma), split2(dm.gamma - 1.0),
-      (unsigned long long*)max_lam);
+         (unsigned long long*)max_lam);
   return cudaGetLastError();
 }
 
@@ -5690,7 +5692,7 @@ cudaError_t launch_recon_vjp(const DeviceMesh& dm, const uint8_t* sel, const dou
       if constexpr (std::is_same<TS, float2>::value)
         launch(recon_vjp_df_kernel<M, NS, NQ, NV>, grid, block, 0, st, (const float2*)dm.ahat, sel,
                Uq_bar, (DF*)d_bar, u_self, dm.n_recon, dm.n_pad,
-            dm.eval_df);
+               dm.eval_df);
       else
         launch(recon_vjp_kernel<M, NS, NQ, NV, TS>, grid, block, 0, st, (const TS*)dm.ahat, sel,
                Uq_bar, d_bar, u_self, dm.n_recon, dm.n_pad, dm.eval);
@@ -5714,22 +5716,12 @@ cudaError_t launch_recon_vjp_tma_t(const DeviceMesh& dm, const uint8_t* sel, con
   using VP = VjpPlan<M, NS, 3 * NQ>;
   auto kern = recon_vjp_tma_kernel<M, NS, NQ>;
   const int threads = kTile * (kConsumers + 1);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)VP::kSmem);
+  unsigned grid = 0;
+  const cudaError_t e =
+      resident_grid(kern, threads, VP::kSmem, (dm.n_recon + kTile - 1) / kTile, &grid);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-    return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, VP::kSmem)) !=
-      cudaSuccess)
-    return e;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int64_t tiles = (dm.n_recon + kTile - 1) / kTile;
-  const int64_t grid = std::min<int64_t>(tiles, (int64_t)per_sm * sms);
-  launch(kern, (unsigned)grid, threads, VP::kSmem, st, (const float2*)dm.ahat, dm.wq, dm.wstat,
-                                                   dm.halo, sel, Uq_bar, part, u_self, dm.n_recon, dm.n_pad,
-                                                   dm.eval_df, dm.err_flag);
+  launch(kern, grid, threads, VP::kSmem, st, (const float2*)dm.ahat, dm.wq, dm.wstat, dm.halo, sel,
+         Uq_bar, part, u_self, dm.n_recon, dm.n_pad, dm.eval_df, dm.err_flag);
   return cudaGetLastError();
 }
 
@@ -5755,17 +5747,17 @@ cudaError_t launch_scatter_gather(const DeviceMesh& dm, const int64_t* rev_off,
   if (dm.n_var == 1) {
     if (pairs)
       launch(scatter_gather_kernel<1, DF>, grid, 256, 0, st, rev_off, rev_idx, (const DF*)d_bar,
-                                                         u_self, v, dm.n_cell, dm.n_pad, ubd);
+             u_self, v, dm.n_cell, dm.n_pad, ubd);
     else
       launch(scatter_gather_kernel<1, double>, grid, 256, 0, st, rev_off, rev_idx, d_bar, u_self, v,
-                                                             dm.n_cell, dm.n_pad, ubd);
+             dm.n_cell, dm.n_pad, ubd);
   } else {
     if (pairs)
       launch(scatter_gather_kernel<4, DF>, grid, 256, 0, st, rev_off, rev_idx, (const DF*)d_bar,
-                                                         u_self, v, dm.n_cell, dm.n_pad, ubd);
+             u_self, v, dm.n_cell, dm.n_pad, ubd);
     else
       launch(scatter_gather_kernel<4, double>, grid, 256, 0, st, rev_off, rev_idx, d_bar, u_self, v,
-                                                             dm.n_cell, dm.n_pad, ubd);
+             dm.n_cell, dm.n_pad, ubd);
   }
   return cudaGetLastError();
 }
