@@ -3064,10 +3064,13 @@ __global__ void __launch_bounds__(kTile * (4 / w_vars<HT>() + 1), 4)
         }
       } else {
         const float s2 = exp2i(eT[w] + 42), s1 = exp2i(eT[w] + 21);
-        const DF u0 = d_to_df(u0d);  // the split the state kernels write
+        // the split the state kernels write, and the bits of the state below it
+        const DF u0 = d_to_df(u0d);
+        const float u0r = (float)((u0d - (double)u0.h) - (double)u0.l);
 #pragma unroll
         for (int p = 0; p < NQ3; ++p) {
-          const DF x = Dot::value(acc[w][p], s2, s1, s0);
+          DF x = Dot::value(acc[w][p], s2, s1, s0);
+          x.l += u0r;
           y[p] = x.h;
           const DF r = u0 + x;
           val[w][p] = make_float2(r.h, r.l);
