@@ -59,7 +59,12 @@ KERNELS_SRC = os.path.join(ROOT, "paper_2105_02127_gb300", "csrc", "teno_kernels
 # source hash differs from the current file's is stale and reported as null.
 # Captured on the 131,072-cell shear layer (TENO6; matrices ~2 GB, above L2)
 # and scaled by the cells of a launch: the streamed bytes are per cell.
-NCU_TRAFFIC_PER_CELL = {}
+NCU_TRAFFIC_PER_CELL = {
+    ("fp64_native", 6): (6393.5, "7b818474ca81d5dc"),
+    ("fp64_pairs", 6): (6209.5, "7b818474ca81d5dc"),
+    ("fp32_mixed", 6): (4440.3, "7b818474ca81d5dc"),
+    ("adjoint_vjp", 6): (3641.5, "7b818474ca81d5dc"),
+}
 
 
 def kernels_hash():
